@@ -122,11 +122,10 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * tiles of the products, tiles of the operand preparation) from a device queue, each box's next
  * step queued as soon as its current one completes (an even number of right-hand sides and
  * 16-byte aligned vectors; otherwise, and with 0, two launches per plane step).  Both give
- * bit-identical results.  HELM_TUNE_STENCIL_MARCH: 1 (default) applies complex64 stencils whose column
- * count is a multiple of 16, with constant weights, by walking z-planes (the in-plane terms of a plane are
- * formed once and reused by the three output planes it touches; blocks wholly inside the interior take the
- * class-sum form, the others the product form); 2 the same with the blocks of one absorbing layer (one
- * stretched axis) in product forms specialised to that axis; 0 uses the per-node kernel.  All agree to
+ * bit-identical results.  HELM_TUNE_STENCIL_MARCH: 1 (default) applies stencils with constant weights by
+ * walking z-planes (the in-plane terms of a plane are formed once and reused by the three output planes it
+ * touches; warps wholly inside the interior take class-sum forms, the others the product form), except
+ * complex64 calls of fewer than 2^20 values; 2 the same at every size; 0 uses the per-node kernel.  All agree to
  * FP32 rounding.  Returns HELM_EINVAL for an unknown key or value out of range. */
 #define HELM_TUNE_TC_STAGES 1
 #define HELM_TUNE_COARSE_COOP 2
@@ -151,11 +150,10 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * complex64, 32 for complex128; the rank-NB updates spread over every SM), falling back to full partial pivoting after a tiny block
  * pivot; 0 always uses the fully pivoted elimination.  Read by oras_factor. */
 #define HELM_TUNE_BLOCK_GJ 8
-/* HELM_TUNE_STENCIL_PLANES: output planes per block of the z-marching stencil (HELM_TUNE_STENCIL_MARCH);
- * 0 (default) picks, per grid, the longest walks (at most 64 planes, at least 8) that still give every
- * resident block slot two blocks or more; else 4..128.  The split decides which blocks
- * lie wholly inside the interior (and take the cheaper class-sum form), so results differ with it by FP32
- * rounding only.  Captured graphs are re-captured after a change. */
+/* HELM_TUNE_STENCIL_PLANES: output planes per block of the z-marching stencil (HELM_TUNE_STENCIL_MARCH), at
+ * any size of the call; 0 (default) picks the block shape and the planes per grid from an estimate of the
+ * blocks' time; else 4..128.  The split decides which warps lie wholly inside the interior (and take the
+ * class-sum forms), so results differ with it by rounding only.  Captured graphs are re-captured after a change. */
 #define HELM_TUNE_STENCIL_PLANES 9
 helm_status helm_set_tuning(helm_ctx ctx, int key, int value);
 

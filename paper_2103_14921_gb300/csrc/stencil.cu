@@ -24,6 +24,7 @@
 // reused for the RCH columns.  The grid is (x-line chunks, y, z), so no
 // thread divides 64-bit indices.
 #include <atomic>
+#include <cmath>
 
 #include "internal.h"
 
@@ -183,365 +184,404 @@ __global__ void __launch_bounds__(128) stencil_kernel(const cplx<T>* __restrict_
     *reinterpret_cast<CPack<T, RCH>*>(y + p * nrhs + (long long)ch * RCH) = out;
 }
 
-// ---------------------------------------------------------------- z-march (complex64, columns in chunks of 16)
+// ---------------------------------------------------------------- z-march
 //
-// The same operator grouped by z-planes: with D_a the stretched and P_a the plain second differences,
-//   A u = h^-2 [S0 + D_z S1] + [T0 + P_z T1],
-//   S0 = (D_x + D_y) u + a2 D_x D_y u,   S1 = u + a2 (D_x + D_y) u + a3 D_x D_y u,
-//   T0 = m0 v + m1 (P_x + P_y) v + m2 P_x P_y v,   T1 = m1 v + m2 (P_x + P_y) v + m3 P_x P_y v,   v = k^2 u,
-// where S0, S1, T0, T1 are in-plane.  A thread owns MN consecutive x-nodes of one row j and one column pair
-// and walks a chunk of output planes (a launch parameter): for every plane q it loads the (MN + 2) x 3 in-plane neighbourhood
-// once, forms the in-plane terms of its nodes, and adds their contributions to the outputs q - 1 (last
-// term, then stored), q and q + 1 (first term).  Each output therefore costs (MN + 2) * 3 / MN vector loads
-// instead of 27.  Blocks whose rows all have plain (1, -2, 1) 1-D coefficients take the real-coefficient
-// path; the others use the complex table coefficients.  Ghost nodes contribute zero.
-constexpr int MN = 4;      // x-nodes per thread
-constexpr int MNP = 8;     // column pairs (16 columns)
-
+// The same operator grouped by z-planes.  A thread owns MN consecutive x-nodes of one row and one vector V of
+// columns (two complex64, one complex64 or one complex128) and walks a run of output planes; for every plane q
+// it forms the in-plane terms of its nodes once and adds plane q's contribution to the outputs q - 1 (its last
+// term, then stored), q and q + 1 (its first term), so each output costs (MN + 2) * 3 / MN vector loads instead of
+// 27 and the sums over the rows and the x-neighbours are shared.  Per plane a warp takes one of three forms:
+//
+// * class sums with the mass term folded in (all coefficients plain (1, -2, 1), k^2 real): a neighbour's
+//   coefficient is a_c = Lc_c / h^2 + Mc_c k^2, c = centre, face, edge, corner, four reals per node formed once
+//   per block and plane (shared memory) and used by all columns.  With s_y the sum over the rows j -+ 1:
+//     Q1 = s_y (a_3 u) + a_2 u,  Q0 = s_y (a_2 u) + a_1 u,  R0 = s_y (a_1 u) + a_0 u    (per x-column)
+//     outputs q -+ 1 += Q1(i - 1) + Q1(i + 1) + Q0(i),   output q += Q0(i - 1) + Q0(i + 1) + R0(i).
+//   19 real multiply-adds per complex value at MN = 4 and 17 at MN = 8 (the per-node kernel: 54 and the
+//   coefficients).
+// * class sums of u and of v = k^2 u apart (plain coefficients, complex k^2).
+// * the product form (absorbing layers): with D_a the stretched second differences and a2, a3 the stencil's
+//   product weights, S0 = D_x p + D_y u, S1 = D_x r + p, p = u + a2 D_y u, r = a2 u + a3 D_y u, and plane q adds
+//   h^-2 (S0 + z_c S1) to output q and h^-2 z_-+ S1 to its neighbours; the mass term in class sums of v.
+//
+// The choice is made per warp in x and y and per plane in z, so a run may pass from the interior into the bottom
+// layer.  A plane's neighbourhood ((GX MN + 2) x (MTY + 2) nodes, PC vectors each, and k^2) is copied into one
+// of three shared-memory buffers with cp.async two planes ahead; the source offsets are formed once per thread,
+// not per plane.  Ghost nodes are zero-filled by the copy.
+//
+// complex128 is bound by the FP64 pipe (two lanes per SM and clock): the form with the fewest FP64 operations is
+// taken wherever it holds, and plain axes are tested at run time in the product form too.  112^3 x 16: 2.9 ms
+// (per-node kernel 5.1 ms), 87 % of the pipe while a block runs; 101 x 93 x 77 x 10: 1.30 (2.54) ms; 48^3 x 1: 0.11
+// (0.18) ms.  complex64 is bound by instruction latency at 12 warps per SM (issue 36 % active, DRAM a third of its
+// rate): 112^3 x 16 170 us (per-node 361), 160 x 160 x 80 x 128 with complex k^2 1.39 (5.07) ms, 101 x 93 x 77 x 10
+// 80 (169) us.  MN = 2 (more warps) measured 247, MN = 8 171 us at 112^3 x 16, so 4.
 struct PlainRange {
     int lo[3], hi[3];   // per axis: indices whose stretched coefficients are exactly (1, -2, 1)
 };
 
-// Two complex64 values (re0, im0, re1, im1) in a float4, processed as two (re, im) pairs by the packed FP32
-// instructions (two lanes per instruction, each lane rounded like the scalar operation).
+// Vectors of complex values: float4 (two complex64) and float2 (one), processed as (re, im) pairs by the packed
+// FP32 instructions (two lanes per instruction, each rounded like the scalar operation), and double2.
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 __device__ __forceinline__ float4 cat4(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
 __device__ __forceinline__ float2 sw2(float2 a) { return make_float2(a.y, a.x); }
-__device__ __forceinline__ float4 f4(float a) { return make_float4(a, a, a, a); }
-__device__ __forceinline__ float4 add4(float4 a, float4 b) {
-    return cat4(__fadd2_rn(lo2(a), lo2(b)), __fadd2_rn(hi2(a), hi2(b)));
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
+__device__ __forceinline__ float2 vscal(float s, float2 b) { return __fmul2_rn(make_float2(s, s), b); }
+__device__ __forceinline__ float2 vscal(float2 s, float2 b) { return __fmul2_rn(s, b); }
+__device__ __forceinline__ float2 vaxpy(float2 s, float2 b, float2 a) { return __ffma2_rn(s, b, a); }
+__device__ __forceinline__ float2 vaxpy(float s, float2 b, float2 a) { return __ffma2_rn(make_float2(s, s), b, a); }
+__device__ __forceinline__ float4 vadd(float4 a, float4 b) { return cat4(vadd(lo2(a), lo2(b)), vadd(hi2(a), hi2(b))); }
+__device__ __forceinline__ float4 vsub(float4 a, float4 b) { return cat4(vsub(lo2(a), lo2(b)), vsub(hi2(a), hi2(b))); }
+__device__ __forceinline__ float4 vscal(float s, float4 b) { return cat4(vscal(s, lo2(b)), vscal(s, hi2(b))); }
+__device__ __forceinline__ float4 vaxpy(float s, float4 b, float4 a) {
+    return cat4(vaxpy(s, lo2(b), lo2(a)), vaxpy(s, hi2(b), hi2(a)));
 }
-__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
-    const float2 m = make_float2(-1.f, -1.f);
-    return cat4(__ffma2_rn(m, lo2(b), lo2(a)), __ffma2_rn(m, hi2(b), hi2(a)));
+__device__ __forceinline__ float4 vscal(float2 s, float4 b) { return cat4(vscal(s, lo2(b)), vscal(s, hi2(b))); }
+__device__ __forceinline__ float4 vaxpy(float2 s, float4 b, float4 a) {
+    return cat4(vaxpy(s, lo2(b), lo2(a)), vaxpy(s, hi2(b), hi2(a)));
 }
-// s b (s real)
-__device__ __forceinline__ float4 scal4(float s, float4 b) {
-    const float2 ss = make_float2(s, s);
-    return cat4(__fmul2_rn(ss, lo2(b)), __fmul2_rn(ss, hi2(b)));
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 vsub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 vscal(double s, double2 b) { return make_double2(s * b.x, s * b.y); }
+__device__ __forceinline__ double2 vaxpy(double s, double2 b, double2 a) {
+    return make_double2(fma(s, b.x, a.x), fma(s, b.y, a.y));
 }
-// a + s b (s real)
-__device__ __forceinline__ float4 axpy4(float s, float4 b, float4 a) {
-    const float2 ss = make_float2(s, s);
-    return cat4(__ffma2_rn(ss, lo2(b), lo2(a)), __ffma2_rn(ss, hi2(b), hi2(a)));
+// c b and a + c b for a complex coefficient c
+__device__ __forceinline__ float2 vcmul(c64 c, float2 b) {
+    return __ffma2_rn(make_float2(c.x, c.x), b, __fmul2_rn(make_float2(-c.y, c.y), sw2(b)));
 }
-// a + c b (c complex, b two complex values): per value re = c.x b.re + (-c.y b.im + a.re),
-// im = c.x b.im + (c.y b.re + a.im)
-__device__ __forceinline__ float4 caxpy4(c64 c, float4 b, float4 a) {
-    const float2 cr = make_float2(c.x, c.x), ci = make_float2(-c.y, c.y);
-    return cat4(__ffma2_rn(cr, lo2(b), __ffma2_rn(ci, sw2(lo2(b)), lo2(a))),
-                __ffma2_rn(cr, hi2(b), __ffma2_rn(ci, sw2(hi2(b)), hi2(a))));
+__device__ __forceinline__ float2 vcaxpy(c64 c, float2 b, float2 a) {
+    return __ffma2_rn(make_float2(c.x, c.x), b, __ffma2_rn(make_float2(-c.y, c.y), sw2(b), a));
 }
-// c b (c complex)
-__device__ __forceinline__ float4 cmul4(c64 c, float4 b) {
-    const float2 cr = make_float2(c.x, c.x), ci = make_float2(-c.y, c.y);
-    return cat4(__ffma2_rn(cr, lo2(b), __fmul2_rn(ci, sw2(lo2(b)))),
-                __ffma2_rn(cr, hi2(b), __fmul2_rn(ci, sw2(hi2(b)))));
+__device__ __forceinline__ float4 vcmul(c64 c, float4 b) { return cat4(vcmul(c, lo2(b)), vcmul(c, hi2(b))); }
+__device__ __forceinline__ float4 vcaxpy(c64 c, float4 b, float4 a) {
+    return cat4(vcaxpy(c, lo2(b), lo2(a)), vcaxpy(c, hi2(b), hi2(a)));
 }
-// A complex coefficient c as the pairs (c.re, c.re, c.im, c.im) of one float4.
-__device__ __forceinline__ float4 cpair(c64 c) { return make_float4(c.x, c.x, c.y, c.y); }
-// the 3-point second difference c0 x0 + c1 x1 + c2 x2, plain (1, -2, 1) or with complex coefficients given as
-// pairs: per value the real-coefficient sum R = sum re(c_d) x_d and the imaginary one I = sum im(c_d) x_d are
-// formed first and combined once, R + i I = (R.re - I.im, R.im + I.re)
-template <bool PLAIN>
-__device__ __forceinline__ float4 d3(const float4* c, float4 x0, float4 x1, float4 x2) {
-    if (PLAIN) return axpy4(-2.f, x1, add4(x0, x2));
-    const float2 j = make_float2(-1.f, 1.f);
-    float2 r[2], im[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float2 v0 = h ? hi2(x0) : lo2(x0), v1 = h ? hi2(x1) : lo2(x1), v2 = h ? hi2(x2) : lo2(x2);
-        r[h] = __ffma2_rn(lo2(c[2]), v2, __ffma2_rn(lo2(c[1]), v1, __fmul2_rn(lo2(c[0]), v0)));
-        im[h] = __ffma2_rn(hi2(c[2]), v2, __ffma2_rn(hi2(c[1]), v1, __fmul2_rn(hi2(c[0]), v0)));
-    }
-    return cat4(__ffma2_rn(j, sw2(im[0]), r[0]), __ffma2_rn(j, sw2(im[1]), r[1]));
+__device__ __forceinline__ double2 vcmul(c128 c, double2 b) {
+    return make_double2(fma(c.x, b.x, -c.y * b.y), fma(c.x, b.y, c.y * b.x));
+}
+__device__ __forceinline__ double2 vcaxpy(c128 c, double2 b, double2 a) {
+    return make_double2(fma(c.x, b.x, fma(-c.y, b.y, a.x)), fma(c.x, b.y, fma(c.y, b.x, a.y)));
 }
 
-// The block's planes pass through shared memory: a 128-thread block covers 16 x-nodes x 4 rows x 16
-// columns, and plane q's neighbourhood (18 nodes x 6 rows, all columns, and k^2) is copied in with cp.async
-// two planes ahead of the one computed (three buffers; ghost nodes are zero-filled by the copy).
-constexpr int MTX = (32 / MNP) * MN;       // x-nodes per block (16)
-constexpr int MTY = 4;                     // rows per block (one warp each)
-constexpr int MBX = MTX + 2, MBY = MTY + 2;
-constexpr int MBUF_U = MBX * MBY * MNP;    // float4 entries of one plane buffer
-constexpr int MBUF_K = MBX * MBY;          // float2 entries (k^2) of one plane buffer
-constexpr int MNBUF = 3;                   // plane buffers: q is computed while q + 1 and q + 2 arrive
+template <typename V> struct VTraits;
+template <> struct VTraits<float4> {
+    typedef float T;
+    typedef float4 Coef;   // a complex coefficient as (re, re, im, im)
+    typedef float2 Real;   // a real coefficient as (a, a), the packed instructions' operand
+    static __device__ __forceinline__ float4 zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+};
+template <> struct VTraits<float2> {
+    typedef float T;
+    typedef float4 Coef;
+    typedef float2 Real;
+    static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
+};
+template <> struct VTraits<double2> {
+    typedef double T;
+    typedef c128 Coef;
+    typedef double Real;
+    static __device__ __forceinline__ double2 zero() { return make_double2(0.0, 0.0); }
+};
+__device__ __forceinline__ void make_coef(c64 c, float4& o) { o = make_float4(c.x, c.x, c.y, c.y); }
+__device__ __forceinline__ void make_coef(c128 c, c128& o) { o = c; }
+__device__ __forceinline__ void make_real(float a, float2& o) { o = make_float2(a, a); }
+__device__ __forceinline__ void make_real(double a, double& o) { o = a; }
 
-__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc, bool valid) {
-    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(sdst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gsrc), "r"(valid ? 16 : 0) : "memory");
+// c0 x0 + c1 x1 + c2 x2 with complex coefficients.  Packed FP32: the real-coefficient and the imaginary-coefficient
+// sums are formed first and combined once (one swap instead of three).
+__device__ __forceinline__ float2 d3c(const float4* c, float2 x0, float2 x1, float2 x2) {
+    const float2 r = __ffma2_rn(lo2(c[2]), x2, __ffma2_rn(lo2(c[1]), x1, __fmul2_rn(lo2(c[0]), x0)));
+    const float2 i = __ffma2_rn(hi2(c[2]), x2, __ffma2_rn(hi2(c[1]), x1, __fmul2_rn(hi2(c[0]), x0)));
+    return __ffma2_rn(make_float2(-1.f, 1.f), sw2(i), r);
 }
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc, bool valid) {
+__device__ __forceinline__ float4 d3c(const float4* c, float4 x0, float4 x1, float4 x2) {
+    return cat4(d3c(c, lo2(x0), lo2(x1), lo2(x2)), d3c(c, hi2(x0), hi2(x1), hi2(x2)));
+}
+__device__ __forceinline__ double2 d3c(const c128* c, double2 x0, double2 x1, double2 x2) {
+    return vcaxpy(c[2], x2, vcaxpy(c[1], x1, vcmul(c[0], x0)));
+}
+// x0 - 2 x1 + x2
+template <typename V> __device__ __forceinline__ V d3p(V x0, V x1, V x2) {
+    return vaxpy((typename VTraits<V>::T)-2, x1, vadd(x0, x2));
+}
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* sdst, const void* gsrc, bool valid) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(sdst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(gsrc), "r"(valid ? 8 : 0) : "memory");
+    if (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gsrc), "r"(valid ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(gsrc), "r"(valid ? 8 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// issue the copies of plane q (rows j0-1..j0+MTY, nodes i0-1..i0+MTX); out-of-grid entries become zero
-__device__ __forceinline__ void march_stage(float4* su, float2* sk, const float4* __restrict__ u,
-                                            const c64* __restrict__ k2, int nx, int ny, int nz, int nrs, int i0,
-                                            int j0, int q) {
-    const bool qin = q >= 0 && q < nz;
-    for (int e = threadIdx.x; e < MBUF_U; e += blockDim.x) {
-        const int pc = e % MNP, xn = (e / MNP) % MBX, yr = e / (MNP * MBX);
-        const int ii = i0 + xn - 1, jj = j0 + yr - 1;
-        const bool ok = qin && ii >= 0 && ii < nx && jj >= 0 && jj < ny;
-        const long long node = ok ? ((long long)q * ny + jj) * nx + ii : 0;
-        cp_async16(su + e, u + node * nrs + pc, ok);
-    }
-    for (int e = threadIdx.x; e < MBUF_K; e += blockDim.x) {
-        const int xn = e % MBX, yr = e / MBX;
-        const int ii = i0 + xn - 1, jj = j0 + yr - 1;
-        const bool ok = qin && ii >= 0 && ii < nx && jj >= 0 && jj < ny;
-        const long long node = ok ? ((long long)q * ny + jj) * nx + ii : 0;
-        cp_async8(sk + e, k2 + node, ok);
-    }
+constexpr int MTHREADS = 128;   // threads per block
+constexpr int MNBUF = 3;        // plane buffers: q is computed while q + 1 and q + 2 arrive
+
+// The stencil's constants in the working precision, formed on the host (the class constants Lc / h^2 and Mc).
+template <typename T>
+struct MarchW {
+    T L[4], M[4], a2, a3, ih2;
+};
+
+// A block's tile: PC column vectors x GX groups of MN x-nodes x MTY rows, one thread each.
+struct MarchTile {
+    int pc, gx, mty;   // gx groups of MN nodes
+    int ncc;           // chunks of the columns
+    int threads, mzc;  // threads per block, planes per block
+};
+
+// The vectors of one plane buffer a thread copies at most (the tile is chosen within it).
+template <typename V> struct MarchCfg;
+template <> struct MarchCfg<float4> { static constexpr int MN = 4, NU = 7, BPS = 3, WORK = 220, LAT = 4000; };
+template <> struct MarchCfg<float2> { static constexpr int MN = 4, NU = 8, BPS = 5, WORK = 150, LAT = 4000; };
+template <> struct MarchCfg<double2> { static constexpr int MN = 4, NU = 8, BPS = 2, WORK = 2900, LAT = 3000; };
+
+template <typename V>
+__host__ __device__ constexpr size_t march_smem(int pc, int gx, int mty) {
+    typedef typename VTraits<V>::T T;
+    const size_t ek = (size_t)(mty + 2) * (gx * MarchCfg<V>::MN + 2);
+    return ek * 4 * sizeof(typename VTraits<V>::Real) + MNBUF * ek * pc * sizeof(V) + (size_t)gx * MarchCfg<V>::MN * 3 * sizeof(typename VTraits<V>::Coef) +
+           MNBUF * ek * sizeof(cplx<T>);
 }
 
-// march_run in product form for blocks in the absorbing layers; PX, PY, PZ: the block's rows have plain
-// (1, -2, 1) coefficients along that axis (a block in one layer only is stretched along one axis), so only the
-// stretched axes pay complex products.  The x coefficients of the block's 16 nodes sit in shared memory as
-// pairs (sx, filled before the first barrier of the plane loop), the row's y coefficients in registers.
-template <bool SUB, bool REALK, bool PX, bool PY, bool PZ>
-__device__ __forceinline__ void march_run(const float4* __restrict__ u, const float4* __restrict__ b,
-                                          float4* __restrict__ y, const c64* __restrict__ k2,
-                                          const c64* __restrict__ tab, int nx, int ny, int nz, int nrs,
-                                          const StencilW& w, int i0, int j0, int k0, int k1, float4* su, float2* sk,
-                                          float4* sx) {
-    const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;
-    const int pc = lane % MNP, g = lane / MNP;
-    const int j = j0 + wr, xb = g * MN, ib = i0 + xb;
-    const bool live = j < ny;
-    const float ih2 = (float)w.inv_h2, a2 = (float)w.a2, a3 = (float)w.a3;
-    const float m0 = (float)w.m0, m1 = (float)w.m1, m2 = (float)w.m2, m3 = (float)w.m3;
-    if (!PX && threadIdx.x < MTX * 3) {
-        const int n = threadIdx.x / 3, d = threadIdx.x % 3;
-        sx[threadIdx.x] = i0 + n < nx ? cpair(tab[3 * (i0 + n) + d]) : f4(0.f);
-    }
-    float4 Y[3];
-    if (!PY) {
+// grid: (x tiles, row tiles, plane chunks x column chunks); the column chunk is the fastest part of blockIdx.z
+template <typename V, bool SUB, bool REALK>
+__global__ void __launch_bounds__(MTHREADS, MarchCfg<V>::BPS)
+    stencil_march(const V* __restrict__ u, const V* __restrict__ b, V* __restrict__ y,
+                  const cplx<typename VTraits<V>::T>* __restrict__ k2, const cplx<typename VTraits<V>::T>* __restrict__ tab,
+                  int nx, int ny, int nz, int nrs, MarchTile tl, MarchW<typename VTraits<V>::T> w, PlainRange pl) {
+    typedef typename VTraits<V>::T T;
+    typedef typename VTraits<V>::Coef Coef;
+    typedef typename VTraits<V>::Real Real;
+    typedef cplx<T> C;
+    constexpr int MN = MarchCfg<V>::MN, NU = MarchCfg<V>::NU;
+    struct __align__(16) A4 { Real v[4]; };
+    extern __shared__ __align__(16) unsigned char march_sm[];
+    const int PC = tl.pc, MBX = tl.gx * MN + 2, EK = (tl.mty + 2) * MBX, EU = EK * PC;
+    A4* sa = reinterpret_cast<A4*>(march_sm);
+    Coef* sx = reinterpret_cast<Coef*>(sa + EK);
+    V* su = reinterpret_cast<V*>(sx + tl.gx * MN * 3);
+    C* sk = reinterpret_cast<C*>(su + MNBUF * EU);
+
+    const int tid = threadIdx.x;
+    // the last planes (the bottom layer, the longer work) first
+    const int cc = blockIdx.z % tl.ncc, zc = (gridDim.z - 1 - blockIdx.z) / tl.ncc;
+    const int i0 = blockIdx.x * tl.gx * MN, j0 = blockIdx.y * tl.mty;
+    const int nth = blockDim.x;
+    const int k0 = zc * tl.mzc, k1 = min(k0 + tl.mzc, nz);
+    // columns fastest, then rows, then x-groups, so that a warp spans few rows and groups and its form is seldom mixed
+    const int pc = tid % PC, jr = (tid / PC) % tl.mty, g = tid / (PC * tl.mty);
+    const int j = j0 + jr, ib = i0 + g * MN;
+    const bool live = g < tl.gx && j < ny && ib < nx && cc * PC + pc < nrs;
+    const int xbs = min(g, tl.gx - 1) * MN;   // nodes read by threads past the tile (their values are never stored)
+    const long long pln = (long long)nx * ny * nrs;
+
+    // source offsets of this thread's copies inside a plane
+    int off[NU];
+    uint32_t ok = 0;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) Y[d] = live ? cpair(tab[3 * (nx + j) + d]) : f4(0.f);
-    }
-    const c64* tz = tab + 3 * (nx + ny);
-    float4 P[MN], N[MN];   // outputs q and q + 1, partial
-#pragma unroll
-    for (int c = 0; c < MN; ++c) P[c] = N[c] = f4(0.f);
-    march_stage(su, sk, u, k2, nx, ny, nz, nrs, i0, j0, k0 - 1);
-    cp_async_commit();
-    march_stage(su + MBUF_U, sk + MBUF_K, u, k2, nx, ny, nz, nrs, i0, j0, k0);
-    cp_async_commit();
-    for (int q = k0 - 1, buf = 0; q <= k1; ++q, buf = buf == MNBUF - 1 ? 0 : buf + 1) {
-        // prefetch plane q + 2 into the buffer plane q - 1 used (free since the barrier ending the last step)
-        const int nb = buf >= 1 ? buf - 1 : MNBUF - 1;
-        if (q + 2 <= k1) march_stage(su + nb * MBUF_U, sk + nb * MBUF_K, u, k2, nx, ny, nz, nrs, i0, j0, q + 2);
-        cp_async_commit();
-        cp_async_wait<2>();
-        __syncthreads();
-        // b of the output plane q - 1, loaded now so that its latency overlaps this step's arithmetic
-        float4 bq[MN];
-        if (SUB) {
-#pragma unroll
-            for (int c = 0; c < MN; ++c) {
-                bq[c] = f4(0.f);
-                if (live && q - 1 >= k0 && ib + c < nx)
-                    bq[c] = __ldg(b + (((long long)(q - 1) * ny + j) * nx + ib + c) * nrs + pc);
+    for (int i = 0; i < NU; ++i) {
+        const int e = tid + i * nth;
+        off[i] = 0;
+        if (e < EU) {
+            const int c = e % PC, xn = (e / PC) % MBX, yr = e / (PC * MBX);
+            const int ii = i0 + xn - 1, jj = j0 + yr - 1;
+            if (ii >= 0 && ii < nx && jj >= 0 && jj < ny && cc * PC + c < nrs) {
+                off[i] = (jj * nx + ii) * nrs + cc * PC + c;
+                ok |= 1u << i;
             }
         }
-        const float4* cu = su + buf * MBUF_U;
-        const float2* ck = sk + buf * MBUF_K;
+    }
+    int koff[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int e = tid + i * nth;
+        const int ii = i0 + e % MBX - 1, jj = j0 + e / MBX - 1;
+        const bool in = ii >= 0 && ii < nx && jj >= 0 && jj < ny;
+        koff[i] = in ? jj * nx + ii : 0;
+        if (in) ok |= 1u << (30 + i);
+    }
+    auto stage = [&](int buf, int q) {
+        if (q >= 0 && q < nz) {
+            const V* src = u + q * pln;
+            V* dst = su + buf * EU + tid;
+#pragma unroll
+            for (int i = 0; i < NU; ++i)
+                if (tid + i * nth < EU) cp_async<sizeof(V)>(dst + i * nth, src + off[i], (ok >> i) & 1u);
+            const C* ks = k2 + (long long)q * nx * ny;
+            C* kd = sk + buf * EK;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (tid + i * nth < EK) cp_async<sizeof(C)>(kd + tid + i * nth, ks + koff[i], (ok >> (30 + i)) & 1u);
+            for (int e = tid + 2 * nth; e < EK; e += nth) {   // few columns: more nodes than two per thread
+                const int ii = i0 + e % MBX - 1, jj = j0 + e / MBX - 1;
+                const bool in = ii >= 0 && ii < nx && jj >= 0 && jj < ny;
+                cp_async<sizeof(C)>(kd + e, ks + (in ? jj * nx + ii : 0), in);
+            }
+        }
+        cp_async_commit();
+    };
+
+    // per warp: all its nodes have plain coefficients along x, along y (threads past the grid do not count)
+    const bool px = __all_sync(0xffffffffu, !live || (ib >= pl.lo[0] && min(ib + MN, nx) - 1 <= pl.hi[0]));
+    const bool py = __all_sync(0xffffffffu, !live || (j >= pl.lo[1] && j <= pl.hi[1]));
+    for (int e = tid; e < tl.gx * MN * 3; e += nth) {
+        Coef cf;
+        make_coef(i0 + e / 3 < nx ? tab[3 * i0 + e] : mk<T>(0, 0), cf);
+        sx[e] = cf;
+    }
+    Coef Y[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) make_coef(j < ny ? tab[3 * (nx + j) + d] : mk<T>(0, 0), Y[d]);
+    const C* tz = tab + 3 * (nx + ny);
+    V P[MN], N[MN];   // outputs q and q + 1, partial
+#pragma unroll
+    for (int c = 0; c < MN; ++c) P[c] = N[c] = VTraits<V>::zero();
+    stage(0, k0 - 1);
+    stage(1, k0);
+    for (int q = k0 - 1, buf = 0; q <= k1; ++q, buf = buf == MNBUF - 1 ? 0 : buf + 1) {
+        cp_async_wait<1>();   // plane q has arrived (plane q + 1 may still be in flight)
+        __syncthreads();      // everyone's copies of q; and every thread is done with plane q - 1's buffer
+        {
+            const int nb = buf >= 1 ? buf - 1 : MNBUF - 1;
+            if (q + 2 <= k1) stage(nb, q + 2);
+            else cp_async_commit();
+        }
         const bool qin = q >= 0 && q < nz;
-        c64 zm = mk<float>(0, 0), zc = mk<float>(0, 0), zp = mk<float>(0, 0);
-        if (!PZ) {
-            zm = q - 1 >= 0 && q - 1 < nz ? tz[3 * (q - 1) + 2] : mk<float>(0, 0);
-            zc = qin ? tz[3 * q + 1] : mk<float>(0, 0);
-            zp = q + 1 >= 0 && q + 1 < nz ? tz[3 * (q + 1) + 0] : mk<float>(0, 0);
+        // plain coefficients for every output this plane contributes to
+        const bool zp_ = max(q - 1, k0) >= pl.lo[2] && min(q + 1, k1 - 1) <= pl.hi[2];
+        const bool plain = px && py && zp_;
+        const C* ck = sk + buf * EK;
+        if (REALK && zp_ && qin) {
+            for (int e = tid; e < EK; e += nth) {
+                const T kk = ck[e].x;
+                A4 a;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) make_real(fma(w.M[c], kk, w.L[c]), a.v[c]);
+                sa[e] = a;
+            }
+            __syncthreads();
         }
-        // sliding window over the columns n = c, c + 1, c + 2 of node c (column n = block node xb + n - 1):
-        // D_y u, P_y v, v and u on row j
-        float4 DyU[3], PyV[3], V1[3], U1[3];
-        auto column = [&](int n, int slot) {
-            float4 Ur[3], V[3];
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const int sidx = (wr + r) * MBX + xb + n;
-                Ur[r] = cu[sidx * MNP + pc];
-                const float2 kk = ck[sidx];
-                V[r] = REALK ? scal4(kk.x, Ur[r]) : cmul4(mk<float>(kk.x, kk.y), Ur[r]);
-            }
-            DyU[slot] = d3<PY>(Y, Ur[0], Ur[1], Ur[2]);
-            PyV[slot] = d3<true>(nullptr, V[0], V[1], V[2]);
-            V1[slot] = V[1];
-            U1[slot] = Ur[1];
-        };
-        column(0, 0);
-        column(1, 1);
-#pragma unroll
-        for (int c = 0; c < MN; ++c) {
-            column(c + 2, (c + 2) % 3);
-            const int s0 = c % 3, s1 = (c + 1) % 3, s2 = (c + 2) % 3;
-            float4 X[3];
-            if (!PX) {
-#pragma unroll
-                for (int d = 0; d < 3; ++d) X[d] = sx[(xb + c) * 3 + d];
-            }
-            const float4 u0 = U1[s1];
-            const float4 Eu = add4(d3<PX>(X, U1[s0], U1[s1], U1[s2]), DyU[s1]);
-            const float4 Fu = d3<PX>(X, DyU[s0], DyU[s1], DyU[s2]);
-            const float4 v0 = V1[s1];
-            const float4 Ev = add4(d3<true>(nullptr, V1[s0], V1[s1], V1[s2]), PyV[s1]);
-            const float4 Fv = d3<true>(nullptr, PyV[s0], PyV[s1], PyV[s2]);
-            const float4 S0 = axpy4(a2, Fu, Eu);
-            const float4 S1 = axpy4(a3, Fu, axpy4(a2, Eu, u0));
-            const float4 T0 = axpy4(m2, Fv, axpy4(m1, Ev, scal4(m0, v0)));
-            const float4 T1 = axpy4(m3, Fv, axpy4(m2, Ev, scal4(m1, v0)));
-            const float4 hS1 = scal4(ih2, S1);
-            // output q - 1: its last term
-            const int i = ib + c;
-            if (live && q - 1 >= k0 && i < nx) {
-                float4 o = add4(PZ ? add4(P[c], hS1) : caxpy4(zm, hS1, P[c]), T1);
-                const long long node = ((long long)(q - 1) * ny + j) * nx + i;
-                if (SUB) o = sub4(bq[c], o);
-                __stcs(y + node * nrs + pc, o);
-            }
-            // output q: the centre term; output q + 1: its first term
-            float4 pn = add4(N[c], axpy4(ih2, S0, axpy4(-2.f, T1, T0)));
-            pn = PZ ? axpy4(-2.f, hS1, pn) : caxpy4(zc, hS1, pn);
-            N[c] = add4(PZ ? hS1 : cmul4(zp, hS1), T1);
-            P[c] = pn;
-        }
-        __syncthreads();   // buffer buf is refilled by the next step's prefetch
-    }
-    cp_async_wait<0>();
-}
-
-// march_run for blocks whose rows all have plain (1, -2, 1) coefficients, in class-sum form: with plain
-// differences the coefficient of a neighbour depends only on its class (centre, face, edge, corner), so per
-// plane q and node the in-plane terms of a field w (u for the Laplacian, v = k^2 u for the mass term) are its
-// centre value c, its in-plane face sum F = s_x w + s_y w and its in-plane corner sum E = s_x s_y w (s_a: the sum
-// of the two neighbours along axis a); plane q then adds Lc0 c + Lc1 F + Lc2 E (u) and Mc0 c + Mc1 F + Mc2 E (v)
-// to output q and Lc1 c + Lc2 F + Lc3 E, Mc1 c + Mc2 F + Mc3 E to outputs q - 1 and q + 1, with the class
-// constants Lc = {-6 + 12 a2 - 8 a3, 1 - 4 a2 + 4 a3, a2 - 2 a3, a3} / h^2 and Mc = {m0 - 6 m1 + 12 m2 - 8 m3,
-// m1 - 4 m2 + 4 m3, m2 - 2 m3, m3}.  The same operator as the product form (expanded), in fewer operations.
-template <bool SUB, bool REALK>
-__device__ __forceinline__ void march_run_plain(const float4* __restrict__ u, const float4* __restrict__ b,
-                                                float4* __restrict__ y, const c64* __restrict__ k2, int nx, int ny,
-                                                int nz, int nrs, const StencilW& w, int i0, int j0, int k0, int k1,
-                                                float4* su, float2* sk) {
-    const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;
-    const int pc = lane % MNP, g = lane / MNP;
-    const int j = j0 + wr, xb = g * MN, ib = i0 + xb;
-    const bool live = j < ny;
-    const double ih2 = w.inv_h2;
-    const float L0 = (float)((-6.0 + 12.0 * w.a2 - 8.0 * w.a3) * ih2), L1 = (float)((1.0 - 4.0 * w.a2 + 4.0 * w.a3) * ih2);
-    const float L2 = (float)((w.a2 - 2.0 * w.a3) * ih2), L3 = (float)(w.a3 * ih2);
-    const float M0 = (float)(w.m0 - 6.0 * w.m1 + 12.0 * w.m2 - 8.0 * w.m3), M1 = (float)(w.m1 - 4.0 * w.m2 + 4.0 * w.m3);
-    const float M2 = (float)(w.m2 - 2.0 * w.m3), M3 = (float)w.m3;
-    float4 P[MN], N[MN];
-#pragma unroll
-    for (int c = 0; c < MN; ++c) P[c] = N[c] = f4(0.f);
-    march_stage(su, sk, u, k2, nx, ny, nz, nrs, i0, j0, k0 - 1);
-    cp_async_commit();
-    march_stage(su + MBUF_U, sk + MBUF_K, u, k2, nx, ny, nz, nrs, i0, j0, k0);
-    cp_async_commit();
-    for (int q = k0 - 1, buf = 0; q <= k1; ++q, buf = buf == MNBUF - 1 ? 0 : buf + 1) {
-        const int nb = buf >= 1 ? buf - 1 : MNBUF - 1;
-        if (q + 2 <= k1) march_stage(su + nb * MBUF_U, sk + nb * MBUF_K, u, k2, nx, ny, nz, nrs, i0, j0, q + 2);
-        cp_async_commit();
-        cp_async_wait<2>();
-        __syncthreads();
-        float4 bq[MN];
+        const bool out = live && q - 1 >= k0;
+        V* yq = y + (q - 1) * pln + ((long long)j * nx + ib) * nrs + cc * PC + pc;
+        V bq[MN];
         if (SUB) {
+            const V* bp = b + (yq - y);
+#pragma unroll
+            for (int c = 0; c < MN; ++c) bq[c] = out && ib + c < nx ? __ldcs(bp + c * nrs) : VTraits<V>::zero();
+        }
+        // plane q's contributions to node c: am to output q - 1, a0 to q, ap to q + 1
+        auto emit = [&](int c, V am, V a0, V ap) {
+            if (out && ib + c < nx) {
+                V o = vadd(P[c], am);
+                if (SUB) o = vsub(bq[c], o);
+                __stcs(yq + c * nrs, o);
+            }
+            P[c] = vadd(N[c], a0);
+            N[c] = ap;
+        };
+        const V* cu = su + buf * EU + (jr * MBX + xbs) * PC + pc;
+        if (!qin) {
+#pragma unroll
+            for (int c = 0; c < MN; ++c) emit(c, VTraits<V>::zero(), VTraits<V>::zero(), VTraits<V>::zero());
+        } else if (REALK && plain) {
+            const A4* ca = sa + jr * MBX + xbs;
+            V Q1[3], Q0[3], R0[3];
+            auto column = [&](int n, int s) {
+                const V u0 = cu[n * PC], u1 = cu[(MBX + n) * PC], u2 = cu[(2 * MBX + n) * PC];
+                const A4 a0 = ca[n], a1 = ca[MBX + n], a2 = ca[2 * MBX + n];
+                Q1[s] = vaxpy(a1.v[2], u1, vaxpy(a2.v[3], u2, vscal(a0.v[3], u0)));
+                Q0[s] = vaxpy(a1.v[1], u1, vaxpy(a2.v[2], u2, vscal(a0.v[2], u0)));
+                R0[s] = vaxpy(a1.v[0], u1, vaxpy(a2.v[1], u2, vscal(a0.v[1], u0)));
+            };
+            column(0, 0);
+            column(1, 1);
 #pragma unroll
             for (int c = 0; c < MN; ++c) {
-                bq[c] = f4(0.f);
-                if (live && q - 1 >= k0 && ib + c < nx)
-                    bq[c] = __ldg(b + (((long long)(q - 1) * ny + j) * nx + ib + c) * nrs + pc);
+                column(c + 2, (c + 2) % 3);
+                const int s0 = c % 3, s1 = (c + 1) % 3, s2 = (c + 2) % 3;
+                const V A1 = vadd(vadd(Q1[s0], Q1[s2]), Q0[s1]);
+                emit(c, A1, vadd(vadd(Q0[s0], Q0[s2]), R0[s1]), A1);
+            }
+        } else if (!REALK && plain) {
+            const C* kp = ck + jr * MBX + xbs;
+            V Cu[3], Cv[3], Yu[3], Yv[3];
+            auto column = [&](int n, int s) {
+                const V u0 = cu[n * PC], u1 = cu[(MBX + n) * PC], u2 = cu[(2 * MBX + n) * PC];
+                Cu[s] = u1;
+                Cv[s] = vcmul(kp[MBX + n], u1);
+                Yu[s] = vadd(u0, u2);
+                Yv[s] = vcaxpy(kp[2 * MBX + n], u2, vcmul(kp[n], u0));
+            };
+            column(0, 0);
+            column(1, 1);
+#pragma unroll
+            for (int c = 0; c < MN; ++c) {
+                column(c + 2, (c + 2) % 3);
+                const int s0 = c % 3, s1 = (c + 1) % 3, s2 = (c + 2) % 3;
+                const V cU = Cu[s1], cV = Cv[s1];
+                const V FU = vadd(vadd(Cu[s0], Cu[s2]), Yu[s1]), EU_ = vadd(Yu[s0], Yu[s2]);
+                const V FV = vadd(vadd(Cv[s0], Cv[s2]), Yv[s1]), EV = vadd(Yv[s0], Yv[s2]);
+                const V A0 = vaxpy(w.M[2], EV, vaxpy(w.M[1], FV, vaxpy(w.M[0], cV, vaxpy(w.L[2], EU_, vaxpy(w.L[1], FU, vscal(w.L[0], cU))))));
+                const V A1 = vaxpy(w.M[3], EV, vaxpy(w.M[2], FV, vaxpy(w.M[1], cV, vaxpy(w.L[3], EU_, vaxpy(w.L[2], FU, vscal(w.L[1], cU))))));
+                emit(c, A1, A0, A1);
+            }
+        } else {
+            const C* kp = ck + jr * MBX + xbs;
+            const T ih2 = w.ih2, a2 = w.a2, a3 = w.a3;
+            C zm = mk<T>(0, 0), zz = ih2 * tz[3 * q + 1], zp = mk<T>(0, 0);
+            if (q >= 1) zm = ih2 * tz[3 * (q - 1) + 2];
+            if (q + 1 < nz) zp = ih2 * tz[3 * (q + 1)];
+            V Pw[3], Rw[3], Dy[3], Cv[3], Yv[3];
+            auto column = [&](int n, int s) {
+                const V u0 = cu[n * PC], u1 = cu[(MBX + n) * PC], u2 = cu[(2 * MBX + n) * PC];
+                const V dy = py ? d3p(u0, u1, u2) : d3c(Y, u0, u1, u2);
+                Pw[s] = vaxpy(a2, dy, u1);
+                Rw[s] = vaxpy(a3, dy, vscal(a2, u1));
+                Dy[s] = dy;
+                if (REALK) {
+                    Cv[s] = vscal(kp[MBX + n].x, u1);
+                    Yv[s] = vaxpy(kp[2 * MBX + n].x, u2, vscal(kp[n].x, u0));
+                } else {
+                    Cv[s] = vcmul(kp[MBX + n], u1);
+                    Yv[s] = vcaxpy(kp[2 * MBX + n], u2, vcmul(kp[n], u0));
+                }
+            };
+            column(0, 0);
+            column(1, 1);
+#pragma unroll
+            for (int c = 0; c < MN; ++c) {
+                column(c + 2, (c + 2) % 3);
+                const int s0 = c % 3, s1 = (c + 1) % 3, s2 = (c + 2) % 3;
+                const Coef* X = sx + (xbs + c) * 3;
+                V S0, S1;
+                if (px) {
+                    S0 = d3p(Pw[s0], Pw[s1], Pw[s2]);
+                    S1 = d3p(Rw[s0], Rw[s1], Rw[s2]);
+                } else {
+                    S0 = d3c(X, Pw[s0], Pw[s1], Pw[s2]);
+                    S1 = d3c(X, Rw[s0], Rw[s1], Rw[s2]);
+                }
+                S0 = vadd(S0, Dy[s1]);
+                S1 = vadd(S1, Pw[s1]);
+                const V FV = vadd(vadd(Cv[s0], Cv[s2]), Yv[s1]), EV = vadd(Yv[s0], Yv[s2]);
+                const V B0 = vaxpy(ih2, S0, vaxpy(w.M[2], EV, vaxpy(w.M[1], FV, vscal(w.M[0], Cv[s1]))));
+                const V B1 = vaxpy(w.M[3], EV, vaxpy(w.M[2], FV, vscal(w.M[1], Cv[s1])));
+                if (zp_) {
+                    const V A1 = vaxpy(ih2, S1, B1);
+                    emit(c, A1, vaxpy((T)-2 * ih2, S1, B0), A1);
+                } else {
+                    emit(c, vcaxpy(zm, S1, B1), vcaxpy(zz, S1, B0), vcaxpy(zp, S1, B1));
+                }
             }
         }
-        const float4* cu = su + buf * MBUF_U;
-        const float2* ck = sk + buf * MBUF_K;
-        // sliding window over the columns n of the block row: centre values and the sums over rows j - 1, j + 1
-        float4 Cu[3], Cv[3], Yu[3], Yv[3];
-        auto column = [&](int n, int slot) {
-            float4 U[3], V[3];
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const int sidx = (wr + r) * MBX + xb + n;
-                U[r] = cu[sidx * MNP + pc];
-                const float2 kk = ck[sidx];
-                V[r] = REALK ? scal4(kk.x, U[r]) : cmul4(mk<float>(kk.x, kk.y), U[r]);
-            }
-            Cu[slot] = U[1];
-            Cv[slot] = V[1];
-            Yu[slot] = add4(U[0], U[2]);
-            Yv[slot] = add4(V[0], V[2]);
-        };
-        column(0, 0);
-        column(1, 1);
-#pragma unroll
-        for (int c = 0; c < MN; ++c) {
-            column(c + 2, (c + 2) % 3);
-            const int s0 = c % 3, s1 = (c + 1) % 3, s2 = (c + 2) % 3;
-            const float4 cU = Cu[s1], cV = Cv[s1];
-            const float4 FU = add4(add4(Cu[s0], Cu[s2]), Yu[s1]), EU = add4(Yu[s0], Yu[s2]);
-            const float4 FV = add4(add4(Cv[s0], Cv[s2]), Yv[s1]), EV = add4(Yv[s0], Yv[s2]);
-            // plane q's contribution to output q (A0) and to outputs q -/+ 1 (A1)
-            const float4 A0 = axpy4(M2, EV, axpy4(M1, FV, axpy4(M0, cV, axpy4(L2, EU, axpy4(L1, FU,
-                                  scal4(L0, cU))))));
-            const float4 A1 = axpy4(M3, EV, axpy4(M2, FV, axpy4(M1, cV, axpy4(L3, EU, axpy4(L2, FU,
-                                  scal4(L1, cU))))));
-            const int i = ib + c;
-            if (live && q - 1 >= k0 && i < nx) {
-                float4 o = add4(P[c], A1);
-                const long long node = ((long long)(q - 1) * ny + j) * nx + i;
-                if (SUB) o = sub4(bq[c], o);
-                __stcs(y + node * nrs + pc, o);
-            }
-            P[c] = add4(N[c], A0);
-            N[c] = A1;
-        }
-        __syncthreads();
     }
     cp_async_wait<0>();
-}
-
-// grid: (x-node blocks, row blocks, plane chunks x column chunks); the column chunk (16 columns) is the
-// fastest part of blockIdx.z, so the chunks of one node range run side by side
-template <bool SUB, bool REALK>
-__global__ void __launch_bounds__(128, 3) stencil_march(const c64* __restrict__ u, const c64* __restrict__ b,
-                                                     c64* __restrict__ y, const c64* __restrict__ k2,
-                                                     const c64* __restrict__ tab, int nx, int ny, int nz, int nrhs,
-                                                     int mzc, StencilW w, PlainRange pl, int axis_variants) {
-    __shared__ float4 su[MNBUF * MBUF_U];
-    __shared__ float2 sk[MNBUF * MBUF_K];
-    __shared__ float4 sx[MTX * 3];
-    const int nrs = nrhs >> 1, ncc = nrs / MNP;   // float4 per node, column chunks
-    const int cc = blockIdx.z % ncc, zc = blockIdx.z / ncc;
-    const int i0 = blockIdx.x * MTX, j0 = blockIdx.y * MTY;
-    const int k0 = zc * mzc, k1 = min(k0 + mzc, nz);
-    const float4* u4 = reinterpret_cast<const float4*>(u) + cc * MNP;
-    const float4* b4 = SUB ? reinterpret_cast<const float4*>(b) + cc * MNP : nullptr;
-    float4* y4 = reinterpret_cast<float4*>(y) + cc * MNP;
-    // blocks whose rows all have plain coefficients on every axis take the class-sum form
-    const bool plain = i0 >= pl.lo[0] && min(i0 + MTX, nx) - 1 <= pl.hi[0] && j0 >= pl.lo[1] &&
-                       min(j0 + MTY, ny) - 1 <= pl.hi[1] && k0 >= pl.lo[2] && k1 - 1 <= pl.hi[2];
-    if (plain) {
-        march_run_plain<SUB, REALK>(u4, b4, y4, k2, nx, ny, nz, nrs, w, i0, j0, k0, k1, su, sk);
-        return;
-    }
-    // per axis: the block's rows are plain along it (with axis_variants; else the general product form,
-    // which keeps the kernel's instruction footprint to two loop bodies)
-    const bool px = axis_variants && i0 >= pl.lo[0] && min(i0 + MTX, nx) - 1 <= pl.hi[0];
-    const bool py = axis_variants && j0 >= pl.lo[1] && min(j0 + MTY, ny) - 1 <= pl.hi[1];
-    const bool pz = axis_variants && k0 >= pl.lo[2] && k1 - 1 <= pl.hi[2];
-    if (py && pz) march_run<SUB, REALK, false, true, true>(u4, b4, y4, k2, tab, nx, ny, nz, nrs, w, i0, j0, k0, k1, su, sk, sx);
-    else if (px && pz) march_run<SUB, REALK, true, false, true>(u4, b4, y4, k2, tab, nx, ny, nz, nrs, w, i0, j0, k0, k1, su, sk, sx);
-    else if (px && py) march_run<SUB, REALK, true, true, false>(u4, b4, y4, k2, tab, nx, ny, nz, nrs, w, i0, j0, k0, k1, su, sk, sx);
-    else march_run<SUB, REALK, false, false, false>(u4, b4, y4, k2, tab, nx, ny, nz, nrs, w, i0, j0, k0, k1, su, sk, sx);
 }
 
 struct RowW {
@@ -638,6 +678,91 @@ PlainRange plain_range(helm_grid g) {
     return r;
 }
 
+// The tile of the z-march: PC column vectors (at most 8, the chunks of equal width), and the x-groups, rows and planes
+// per block with the least estimated time on this grid: rounds of resident blocks times the planes they walk
+// (two of them halo) times the larger of a plane's latency and the SM's work on it.
+template <typename V>
+MarchTile march_tile(const helm_grid_desc& d, int nrs, int sms, int planes) {
+    constexpr int MN = MarchCfg<V>::MN;
+    MarchTile t{};
+    t.ncc = (nrs + 7) / 8;
+    t.pc = (nrs + t.ncc - 1) / t.ncc;
+    double best = 1e300;
+    for (int gx = 1; gx <= 32 && (gx == 1 || (gx - 1) * MN < d.nx); gx *= 2)
+        for (int warps = 1; warps <= MTHREADS / 32; warps *= 2) {
+            const int rows = std::min(warps * 32 / (t.pc * gx), d.ny);
+            if (rows < 1) continue;
+            const int threads = (rows * t.pc * gx + 31) / 32 * 32;
+            const long long eu = (long long)(rows + 2) * (gx * MN + 2) * t.pc;
+            if (eu > (long long)MarchCfg<V>::NU * threads) continue;
+            const int per_sm = std::min(MarchCfg<V>::BPS * MTHREADS / threads, (int)(227 * 1024 / (march_smem<V>(t.pc, gx, rows) + 1024)));
+            if (per_sm < 1) continue;
+            const double xy = (double)((d.nx + gx * MN - 1) / (gx * MN)) * ((d.ny + rows - 1) / rows) * t.ncc;
+            for (int nch = 1; nch <= d.nz; ++nch) {
+                const int mzc = planes ? std::min(planes, d.nz) : (d.nz + nch - 1) / nch;
+                if (!planes && mzc > 64) continue;
+                if (!planes && mzc < 4 && nch > 1) break;
+                const double blocks = xy * ((d.nz + mzc - 1) / mzc), slots = (double)per_sm * sms;
+                // clocks of one plane with res blocks on an SM: a warp's latency, or its scheduler's work
+                auto plane = [&](double res) {
+                    return std::max((double)MarchCfg<V>::LAT,
+                                    std::ceil(res * (threads / 32) / 4.0) * MarchCfg<V>::WORK * MN);
+                };
+                const double full = std::floor(blocks / slots), rest = blocks - full * slots;
+                const double time = (full * plane(per_sm) + (rest > 0 ? plane(std::ceil(rest / sms)) : 0.0)) * (mzc + 2);
+                if (time < best) {
+                    best = time;
+                    t.gx = gx;
+                    t.mty = rows;
+                    t.threads = threads;
+                    t.mzc = mzc;
+                }
+                if (planes) break;
+            }
+        }
+    return t;
+}
+
+// Launch of the z-march; false when it does not apply (the per-node kernel then runs).
+template <typename V, bool SUB>
+bool launch_march(helm_grid g, const void* u, const void* b, void* y, int nrs, cudaStream_t s) {
+    typedef typename VTraits<V>::T T;
+    const helm_grid_desc& d = g->d;
+    if ((long long)d.nx * d.ny * nrs >= (1ll << 31)) return false;   // 32-bit offsets inside a plane
+    const MarchTile t = march_tile<V>(d, nrs, std::max(g->ctx->sm_count, 1), g->ctx->stencil_planes);
+    if (!t.gx) return false;
+    const size_t smem = march_smem<V>(t.pc, t.gx, t.mty);
+    const int gx = (d.nx + t.gx * MarchCfg<V>::MN - 1) / (t.gx * MarchCfg<V>::MN), gy = (d.ny + t.mty - 1) / t.mty;
+    const long long gz = (long long)((d.nz + t.mzc - 1) / t.mzc) * t.ncc;
+    if (gy > 65535 || gz > 65535) return false;
+    const PlainRange pl = plain_range(g);
+    const cplx<T>* k2 = sizeof(T) == 8 ? (const cplx<T>*)g->k2 : (const cplx<T>*)g->k2f;
+    const cplx<T>* tab = sizeof(T) == 8 ? (const cplx<T>*)g->tab : (const cplx<T>*)g->tabf;
+    const Interior in = interior_of(g);
+    MarchW<T> w;
+    for (int c = 0; c < 4; ++c) {
+        w.L[c] = (T)(in.Lc[c] * g->w.inv_h2);
+        w.M[c] = (T)in.Mc[c];
+    }
+    w.a2 = (T)g->w.a2;
+    w.a3 = (T)g->w.a3;
+    w.ih2 = (T)g->w.inv_h2;
+    const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
+    static std::atomic<bool> attr{false};
+    if (!attr.load(std::memory_order_acquire)) {
+        cudaFuncSetAttribute(stencil_march<V, SUB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        cudaFuncSetAttribute(stencil_march<V, SUB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        attr.store(true, std::memory_order_release);
+    }
+    if (g->k2_real)
+        stencil_march<V, SUB, true><<<grid, t.threads, smem, s>>>((const V*)u, (const V*)b, (V*)y, k2, tab, d.nx, d.ny,
+                                                                  d.nz, nrs, t, w, pl);
+    else
+        stencil_march<V, SUB, false><<<grid, t.threads, smem, s>>>((const V*)u, (const V*)b, (V*)y, k2, tab, d.nx, d.ny,
+                                                                   d.nz, nrs, t, w, pl);
+    return true;
+}
+
 template <bool SUB>
 helm_status launch_any(helm_grid g, int prec, const void* u, const void* b, void* y, int nrhs, cudaStream_t s) {
     if (nrhs <= 0) return HELM_OK;
@@ -648,45 +773,21 @@ helm_status launch_any(helm_grid g, int prec, const void* u, const void* b, void
     const Interior in = interior_of(g);
     const RowW rw{g->wtab, g->wbin};
     const uintptr_t al = (uintptr_t)u | (uintptr_t)y | (SUB ? (uintptr_t)b : 0);
-    if (prec == HELM_PREC_FP64) {
+    bool done = false;
+    // complex64 calls of fewer than 2^20 values run the per-node kernel: a walk's planes are a serial chain, and too
+    // few blocks hide its latency (48^3 x 1: 27 us per call against 38; 64^3 x 4, 2^20 values: 44 against 40;
+    // 112^3 x 1: 76 against 69).  complex128 is FP64-bound at any size and always walks.
+    const bool walk = g->ctx->stencil_march == 2 || g->ctx->stencil_planes || prec == HELM_PREC_FP64 ||
+                      g->n * nrhs >= (1 << 20);
+    if (g->ctx->stencil_march && !g->wtab && walk) {
+        if (prec == HELM_PREC_FP64) done = (al & 15) == 0 && launch_march<double2, SUB>(g, u, b, y, nrhs, s);
+        else if (nrhs % 2 == 0 && (al & 15) == 0) done = launch_march<float4, SUB>(g, u, b, y, nrhs / 2, s);
+        else done = (al & 7) == 0 && launch_march<float2, SUB>(g, u, b, y, nrhs, s);
+    }
+    if (done) {
+    } else if (prec == HELM_PREC_FP64) {
         dispatch<double, SUB>((const c128*)u, (const c128*)b, (c128*)y, g->k2, g->tab, g->d, nrhs, g->w, in,
                               g->k2_real, rw, s);
-    } else if (g->ctx->stencil_march && nrhs % (2 * MNP) == 0 && !g->wtab && (al & 15) == 0) {
-        const PlainRange pl = plain_range(g);
-        const int gx = (g->d.nx + MTX - 1) / MTX, gy = (g->d.ny + MTY - 1) / MTY, ncc = nrhs / (2 * MNP);
-        int mzc = g->ctx->stencil_planes;
-        if (mzc == 0) {
-            // the fewest plane chunks (longest walks: less halo per output) of at most 64 planes that still give
-            // every resident block slot two blocks or more (measured: fewer blocks than that leave the launch
-            // short of latency hiding), chunks of 8 planes at least
-            static std::atomic<int> occ{0};
-            int per_sm = occ.load(std::memory_order_relaxed);
-            if (per_sm == 0) {
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, stencil_march<SUB, true>, 128, 0) !=
-                    cudaSuccess)
-                    per_sm = 0;
-                occ.store(per_sm, std::memory_order_relaxed);
-            }
-            const long long slots = (long long)std::max(per_sm, 1) * std::max(g->ctx->sm_count, 1);
-            const long long xy = (long long)gx * gy * ncc;
-            const int nz = g->d.nz;
-            mzc = std::min(nz, 8);
-            for (int nch = 1; nch <= nz; ++nch) {
-                const int c = (nz + nch - 1) / nch;
-                if (c > 64) continue;
-                mzc = std::max(c, std::min(nz, 8));
-                if (c <= 8 || xy * ((nz + c - 1) / c) >= 2 * slots) break;
-            }
-        }
-        const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((g->d.nz + mzc - 1) / mzc * ncc));
-        if (g->k2_real)
-            stencil_march<SUB, true><<<grid, 128, 0, s>>>((const c64*)u, (const c64*)b, (c64*)y, g->k2f, g->tabf,
-                                                          g->d.nx, g->d.ny, g->d.nz, nrhs, mzc, g->w, pl,
-                                                          g->ctx->stencil_march == 2 ? 1 : 0);
-        else
-            stencil_march<SUB, false><<<grid, 128, 0, s>>>((const c64*)u, (const c64*)b, (c64*)y, g->k2f, g->tabf,
-                                                           g->d.nx, g->d.ny, g->d.nz, nrhs, mzc, g->w, pl,
-                                                          g->ctx->stencil_march == 2 ? 1 : 0);
     } else {
         dispatch<float, SUB>((const c64*)u, (const c64*)b, (c64*)y, g->k2f, g->tabf, g->d, nrhs, g->w, in,
                              g->k2_real, rw, s);
