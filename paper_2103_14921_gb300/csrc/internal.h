@@ -270,6 +270,9 @@ helm_status planeset_solve(helm_ctx ctx, const PlaneSet& P, void* loc, void* rbu
                            int* err = nullptr);
 helm_status planeset_solve_coop(helm_ctx ctx, const PlaneSet& P, c64* loc, c64* rbuf, int nrhs, cudaStream_t st,
                                 int* err, bool* done);
+// one-level ORAS of a set of small boxes in one launch (boxsolve.cu); *done = false: the boxes do not fit
+helm_status boxes_solve_smem(helm_ctx ctx, const PlaneSet& P, int wp, const void* v, void* out, void* loc, int nx, int ny,
+                             int nrhs, cudaStream_t st, bool* done);
 // tensor-core sweeps (sweep_tc.cu), complex64 local vectors, padded factor layout
 int tc_npad(int nrhs);
 // lb: the restricted right-hand sides b (read by the forward sweep); loc receives y, then x.

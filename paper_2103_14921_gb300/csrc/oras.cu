@@ -847,6 +847,9 @@ helm_status coarse_dd_t(helm_oras o, const PlaneSet& P, const cplx<TV>* v, cplx<
 
 helm_status coarse_dd_apply(helm_oras o, int wp, const void* v, void* out, int nrhs) {
     const PlaneSet& P = o->cdd32.G ? o->cdd32 : o->cdd;
+    bool done = false;
+    HELM_TRY(boxes_solve_smem(o->g->ctx, P, wp, v, out, o->cloc, o->cdims[0], o->cdims[1], nrhs, o->g->ctx->stream, &done));
+    if (done) return HELM_OK;
     const bool l64 = P.prec == HELM_PREC_FP64;
     if (wp == HELM_PREC_FP64)
         return l64 ? coarse_dd_t<double, double>(o, P, (const c128*)v, (c128*)out, nrhs)
