@@ -422,20 +422,6 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_scale_kernel(const cplx
     }
 }
 
-// ||w''|| = sqrt(||w'||^2 - ||h2||^2) per column (V orthonormal; h2 is a rounding-level correction, so there
-// is no cancellation), as the subdiagonal entry H[j+1][j].
-__global__ void second_norm(const double* __restrict__ nw, const c128* __restrict__ h2, int ni, int nrhs,
-                            double* __restrict__ out) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrhs) return;
-    double s = nw[r] * nw[r];
-    for (int i = 0; i < ni; ++i) {
-        const c128 a = h2[(long long)i * nrhs + r];
-        s -= a.x * a.x + a.y * a.y;
-    }
-    out[r] = sqrt(fmax(s, 0.0));
-}
-
 // Re-orthogonalisation test per column: a second projection when ||w'|| < ||w|| / sqrt(2).
 __global__ void reorth_flags(const double* __restrict__ before, const double* __restrict__ after, int* __restrict__ flag,
                              int* __restrict__ any, int nrhs) {
@@ -529,36 +515,23 @@ __global__ void cycle_start(RhsState* __restrict__ S, const double* __restrict__
     g[(long long)r * (m + 1)] = mk<double>(s.active ? beta[r] : 0.0, 0.0);
 }
 
-// Column j of H for every rhs: apply earlier rotations, make a new one, update g and the estimate.
-// H[r][i][j] is (m+1) x m per rhs; hnorm[r] = ||w|| = H[j+1][j]; inv[r] <- 1/hnorm (or 0).
-__global__ void givens_step(RhsState* __restrict__ S, c128* __restrict__ H, double* __restrict__ cs,
-                            c128* __restrict__ sn, c128* __restrict__ g, const double* __restrict__ hnorm,
-                            double* __restrict__ inv, int j, int m, int nrhs, int* __restrict__ running) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrhs) return;
-    RhsState& s = S[r];
-    if (!s.active) {
-        inv[r] = 0.0;
-        return;
-    }
-    c128* h = H + (long long)r * (m + 1) * m;
-    double* c = cs + (long long)r * m;
-    c128* sv = sn + (long long)r * m;
-    c128* gg = g + (long long)r * (m + 1);
-    const double hn = hnorm[r];
-    h[(long long)(j + 1) * m + j] = mk<double>(hn, 0.0);
+// Column j of H of one rhs, h[0..j+1] with h[j+1] = ||w||: apply the earlier rotations (cs, sn), make a new one,
+// update g and the estimate; returns 1/||w|| (0 once the column stops).  h, c and sv may be in shared memory.
+__device__ __forceinline__ double givens_column(RhsState& s, c128* h, int hstride, double* c, c128* sv, c128* gg, double hn,
+                                                int j, int m, int* running) {
+    c128 a = h[0];
     for (int i = 0; i < j; ++i) {
-        const c128 a = h[(long long)i * m + j], b = h[(long long)(i + 1) * m + j];
+        const c128 b = h[(long long)(i + 1) * hstride];
         const c128 si = sv[i];
         const c128 sb = si * b;
         const c128 csa = mk<double>(c[i] * a.x, c[i] * a.y);
-        h[(long long)i * m + j] = csa + sb;
+        h[(long long)i * hstride] = csa + sb;
         // -conj(s) a + c b
         const c128 sca = mk<double>(si.x * a.x + si.y * a.y, si.x * a.y - si.y * a.x);
-        h[(long long)(i + 1) * m + j] = mk<double>(c[i] * b.x - sca.x, c[i] * b.y - sca.y);
+        a = mk<double>(c[i] * b.x - sca.x, c[i] * b.y - sca.y);
     }
-    const c128 a = h[(long long)j * m + j], b = h[(long long)(j + 1) * m + j];
-    const double na = hypot(a.x, a.y), nbv = hypot(b.x, b.y);
+    const c128 b = mk<double>(hn, 0.0);
+    const double na = hypot(a.x, a.y), nbv = hn;
     double cc;
     c128 ss;
     if (nbv == 0.0) {
@@ -576,18 +549,107 @@ __global__ void givens_step(RhsState* __restrict__ S, c128* __restrict__ H, doub
     }
     c[j] = cc;
     sv[j] = ss;
-    h[(long long)j * m + j] = mk<double>(cc * a.x, cc * a.y) + ss * b;
-    h[(long long)(j + 1) * m + j] = mk<double>(0, 0);
+    h[(long long)j * hstride] = mk<double>(cc * a.x, cc * a.y) + ss * b;
+    h[(long long)(j + 1) * hstride] = mk<double>(0, 0);
     const c128 gj = gg[j];
-    gg[j + 1] = mk<double>(-(ss.x * gj.x + ss.y * gj.y), -(ss.x * gj.y - ss.y * gj.x));
+    const c128 gn = mk<double>(-(ss.x * gj.x + ss.y * gj.y), -(ss.x * gj.y - ss.y * gj.x));
+    gg[j + 1] = gn;
     gg[j] = mk<double>(cc * gj.x, cc * gj.y);
     s.steps = j + 1;
     s.iters += 1;
-    s.est = hypot(gg[j + 1].x, gg[j + 1].y) / s.bnorm;
+    s.est = hypot(gn.x, gn.y) / s.bnorm;
     const bool stop = s.est <= s.tol || hn == 0.0 || s.iters >= s.maxit || j + 1 >= m;
-    inv[r] = (hn > 0.0 && !stop) ? 1.0 / hn : 0.0;
     if (stop) s.active = 0;
     else atomicAdd(running, 1);
+    return (hn > 0.0 && !stop) ? 1.0 / hn : 0.0;
+}
+
+// The Givens step of every rhs.  H[r][i][j] is (m+1) x m per rhs; hnorm[r] = ||w||; inv[r] <- 1/hnorm (or 0).
+__global__ void givens_step(RhsState* __restrict__ S, c128* __restrict__ H, double* __restrict__ cs,
+                            c128* __restrict__ sn, c128* __restrict__ g, const double* __restrict__ hnorm,
+                            double* __restrict__ inv, int j, int m, int nrhs, int* __restrict__ running) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= nrhs) return;
+    if (!S[r].active) {
+        inv[r] = 0.0;
+        return;
+    }
+    inv[r] = givens_column(S[r], H + (long long)r * (m + 1) * m + j, m, cs + (long long)r * m, sn + (long long)r * m,
+                           g + (long long)r * (m + 1), hnorm[r], j, m, running);
+}
+
+// End of the first projection of the fused CGS2, one 128-thread block per (i, r): h1_i = sum of the block partials (the
+// order of finish_dots), into hpass and H[r][i][j]; the counter of running columns is cleared for the Givens step.
+__global__ void __launch_bounds__(128) finish_first(const c128* __restrict__ partial, int nblk, int ldp, int nrhs,
+                                                    c128* __restrict__ hpass, c128* __restrict__ H, int m, int j,
+                                                    int* __restrict__ running) {
+    const int i = blockIdx.x / nrhs, r = blockIdx.x % nrhs;
+    c128 sum = mk<double>(0, 0);
+    for (int b = threadIdx.x; b < nblk; b += 128) sum = sum + partial[((long long)b * ldp + i) * nrhs + r];
+    sum = block_sum128(sum);
+    if (threadIdx.x == 0) {
+        hpass[(long long)i * nrhs + r] = sum;
+        H[(long long)r * (m + 1) * m + (long long)i * m + j] = sum;
+        if (blockIdx.x == 0) *running = 0;
+    }
+}
+
+// End of the second projection, one block per rhs: h2 = sums of the block partials (a warp per basis vector, fixed order)
+// into hpass; H[r][.][j] += h2; ||w''|| = sqrt(||w'||^2 - ||h2||^2) (V orthonormal and h2 a rounding-level
+// correction, so there is no cancellation); then the Givens step of column j, whose serial chain reads the column and
+// the rotations from shared memory.  Five launches and a memset of a few microseconds each in one.
+constexpr int FS_THREADS = 512, FS_MAX = 32;   // FS_MAX: basis vectors of the fused CGS2
+__global__ void __launch_bounds__(FS_THREADS) finish_second(const c128* __restrict__ partial,
+                                                            const double* __restrict__ npart, int nblk, int ldp,
+                                                            int nrhs, int ni, c128* __restrict__ hpass,
+                                                            c128* __restrict__ H, RhsState* __restrict__ S,
+                                                            double* __restrict__ cs, c128* __restrict__ sn,
+                                                            c128* __restrict__ g, double* __restrict__ inv, int j, int m,
+                                                            int* __restrict__ running) {
+    __shared__ c128 sh[FS_MAX + 2], ssn[FS_MAX + 1];
+    __shared__ double scs[FS_MAX + 1], snrm, sq[FS_MAX];
+    const int r = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    c128* h = H + (long long)r * (m + 1) * m + j;
+    for (int i = w; i <= ni; i += FS_THREADS / 32) {
+        c128 sum = mk<double>(0, 0);
+        if (i < ni)
+            for (int b = lane; b < nblk; b += 32) sum = sum + partial[((long long)b * ldp + i) * nrhs + r];
+        else
+            for (int b = lane; b < nblk; b += 32) sum.x += npart[(long long)b * nrhs + r];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
+        }
+        if (lane == 0) {
+            if (i < ni) {
+                hpass[(long long)i * nrhs + r] = sum;
+                sh[i] = h[(long long)i * m] + sum;
+                sq[i] = sum.x * sum.x + sum.y * sum.y;
+                if (i < j) {
+                    scs[i] = cs[(long long)r * m + i];
+                    ssn[i] = sn[(long long)r * m + i];
+                }
+            } else {
+                snrm = sum.x;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (!S[r].active) {
+            inv[r] = 0.0;
+        } else {
+            double s2 = snrm;
+            for (int i = 0; i < ni; ++i) s2 -= sq[i];
+            inv[r] = givens_column(S[r], sh, 1, scs, ssn, g + (long long)r * (m + 1), sqrt(fmax(s2, 0.0)), j, m, running);
+            cs[(long long)r * m + j] = scs[j];
+            sn[(long long)r * m + j] = ssn[j];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < ni) h[(long long)threadIdx.x * m] = sh[threadIdx.x];
+    if (threadIdx.x == 0) h[(long long)ni * m] = mk<double>(0, 0);
 }
 
 // y = R^{-1} g for the steps taken this cycle (upper-triangular back substitution).
@@ -677,6 +739,81 @@ __global__ void finite_check_cols(const c128* __restrict__ v, const int* __restr
 }
 
 // ------------------------------------------------------------------ host driver
+
+// What the fused CGS2 of one iteration works on (the outer engine's or the inner coarse solve's workspace).
+template <typename T>
+struct CgsBuffers {
+    cplx<T>*V, *w;
+    long long nel;
+    int S, m, nblk, ldp;
+    c128 *part, *hpass, *H, *sn, *gv;
+    double *cs, *dpart, *inv;
+    RhsState* Sd;
+    int* running;
+};
+
+// Bases the fused CGS2 takes: up to 32 vectors (complex128: 16, the register budget of its kernels), coefficients
+// within 40 KB of shared memory.
+template <typename T>
+inline bool cgs2_fits(int ni, int S) {
+    return ni <= (sizeof(T) == 4 ? 32 : 16) && (size_t)ni * S * sizeof(cplx<T>) <= 40 * 1024;
+}
+
+// CGS2 in three passes over the basis: h1 = V^H w; w' = w - V h1 fused with h2 = V^H w' and ||w'||; H[.][j] = h1 + h2,
+// H[j+1][j] = sqrt(||w'||^2 - ||h2||^2); the Givens step; then v_{j+1} = (w' - V h2) / H[j+1][j] fused with the
+// second update.  Five launches: the three passes and the two small kernels that close the reductions (112^3 x 16:
+// 11 launches before; the inner coarse solve of 32 columns on 33 x 33 x 17 nodes, 17 before).
+template <typename T>
+void fused_cgs2(helm_ctx ctx, cudaStream_t st, const CgsBuffers<T>& B, int j, const char* family) {
+    const int ni = j + 1, S = B.S;
+    const long long nel = B.nel;
+    const cplx<T>* V = B.V;
+    cplx<T>* w = B.w;
+    // resident blocks per SM for the fused kernel (two for bases of up to 4 vectors, whose smaller register
+    // arrays allow it), as the largest multiple of q <= that many blocks
+    int a = RED_THREADS, bq = S;
+    while (bq) { const int t = a % bq; a = bq; bq = t; }
+    const int q = S / a;
+    const int per_sm = ni <= 4 ? 2 : 1;
+    const int nb1 = std::min(B.nblk, std::max(q, (per_sm * std::max(1, ctx->sm_count) / q) * q));
+    int tk = family ? prof_begin(ctx, family) : -1;
+    if (ni <= 2)
+        dots_kernel<T, 8><<<B.nblk, RED_THREADS, 0, st>>>(V, nel, w, nel, S, 0, ni, B.part, B.ldp, nullptr, nullptr);
+    else
+        dots_kernel<T><<<B.nblk, RED_THREADS, 0, st>>>(V, nel, w, nel, S, 0, ni, B.part, B.ldp, nullptr, nullptr);
+    prof_end(ctx, tk, (double)(ni + 1) * nel * sizeof(cplx<T>));
+    finish_first<<<ni * S, 128, 0, st>>>(B.part, B.nblk, B.ldp, S, B.hpass, B.H, B.m, j, B.running);
+    tk = family ? prof_begin(ctx, family) : -1;
+    if (ni <= 2)
+        update_dots_kernel<T, 2><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
+    else if (ni <= 4)
+        update_dots_kernel<T, 4><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
+    else if (ni <= 8)
+        update_dots_kernel<T, 8><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
+    else if (ni <= 16 || sizeof(T) == 8)
+        update_dots_kernel<T, 16><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
+    else if (S <= 16)
+        update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16), true><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass,
+                                                                                            B.part, B.ldp, B.dpart);
+    else
+        update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16)><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass,
+                                                                                       B.part, B.ldp, B.dpart);
+    prof_end(ctx, tk, (double)(ni + 2) * nel * sizeof(cplx<T>));
+    finish_second<<<S, FS_THREADS, 0, st>>>(B.part, B.dpart, nb1, B.ldp, S, ni, B.hpass, B.H, B.Sd, B.cs, B.sn, B.gv, B.inv,
+                                            j, B.m, B.running);
+    tk = family ? prof_begin(ctx, family) : -1;
+    const size_t hsm = (size_t)ni * S * sizeof(cplx<T>);
+    cplx<T>* vn = B.V + (long long)(j + 1) * nel;
+    if (ni <= 2)
+        update_scale_kernel<T, (sizeof(T) == 4 ? 8 : 4), (sizeof(T) == 4 ? 2 : 4)><<<B.nblk, RED_THREADS, hsm, st>>>(
+            V, nel, w, vn, nel, S, ni, B.hpass, B.inv);
+    else if (ni <= 4)
+        update_scale_kernel<T, 4, 4><<<B.nblk, RED_THREADS, hsm, st>>>(V, nel, w, vn, nel, S, ni, B.hpass, B.inv);
+    else
+        update_scale_kernel<T, 2, 8><<<B.nblk, RED_THREADS, hsm, st>>>(V, nel, w, vn, nel, S, ni, B.hpass, B.inv);
+    prof_end(ctx, tk, (double)(ni + 2) * nel * sizeof(cplx<T>));
+    ctx->launches += 5;
+}
 
 // Batched (F)GMRES over S columns: workspaces, per-column state and one restart cycle at a time.
 template <typename T>
@@ -903,60 +1040,10 @@ struct Krylov final : KrylovEngine {
         return HELM_OK;
     }
 
-    // CGS2 in three passes over the basis (up to 32 basis vectors): h1 = V^H w; w' = w - V h1 fused with
-    // h2 = V^H w' and ||w'||; H[.][j] = h1 + h2, H[j+1][j] = sqrt(||w'||^2 - ||h2||^2); the Givens step; then
-    // v_{j+1} = (w' - V h2) / H[j+1][j] fused with the second update.
+    // CGS2 with the Givens step (fused_cgs2 below) on this engine's basis
     helm_status cgs2_fused(int j) {
-        const int ni = j + 1;
-        // resident blocks per SM for the fused kernel (two for bases of up to 4 vectors, whose smaller register
-        // arrays allow it), as the largest multiple of q <= that many blocks
-        int a = RED_THREADS, bq = S;
-        while (bq) { const int t = a % bq; a = bq; bq = t; }
-        const int q = S / a;
-        const int per_sm = ni <= 4 ? 2 : 1;
-        const int nb1 = std::min(nblk, std::max(q, (per_sm * std::max(1, ctx->sm_count) / q) * q));
-        dots_pass(V, w, ni, nullptr, nullptr);
-        finish_into(ni, hpass, S, 1, 0, 0, nullptr, nullptr);
-        finish_into(ni, H, m, (m + 1) * m, j, 0, nullptr, nullptr);
-        {
-            const int tk = prof_begin(ctx, "arnoldi");
-            if (ni <= 2)
-                update_dots_kernel<T, 2><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, hpass, part, ldp, dpart);
-            else if (ni <= 4)
-                update_dots_kernel<T, 4><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, hpass, part, ldp, dpart);
-            else if (ni <= 8)
-                update_dots_kernel<T, 8><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, hpass, part, ldp, dpart);
-            else if (ni <= 16 || sizeof(T) == 8)
-                update_dots_kernel<T, 16><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, hpass, part, ldp, dpart);
-            else if (S <= 16)
-                update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16), true><<<nb1, RED_THREADS, 0, st>>>(
-                    V, nel, w, nel, S, ni, hpass, part, ldp, dpart);
-            else
-                update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16)><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni,
-                                                                                           hpass, part, ldp, dpart);
-            prof_end(ctx, tk, (double)(ni + 2) * nel * sizeof(cplx<T>));
-        }
-        finish_dots<<<ni * S, 128, 0, st>>>(part, nb1, ldp, ni, S, hpass, S, 1, 0, 0, nullptr, nullptr);
-        finish_dots<<<ni * S, 128, 0, st>>>(part, nb1, ldp, ni, S, H, m, (m + 1) * m, j, 1, nullptr, nullptr);
-        finish_norm2<<<S, 128, 0, st>>>(dpart, nb1, S, na);
-        second_norm<<<rg, 128, 0, st>>>(na, hpass, ni, S, hn);
-        ctx->launches += 5;
-        HELM_CUDA(ctx, cudaMemsetAsync(running, 0, sizeof(int), st));
-        givens_step<<<rg, 128, 0, st>>>(Sd, H, cs, sn, gv, hn, inv, j, m, S, running);
-        {
-            const int tk = prof_begin(ctx, "arnoldi");
-            const size_t hsm = (size_t)ni * S * sizeof(cplx<T>);
-            cplx<T>* vn = V + (long long)(j + 1) * nel;
-            if (ni <= 2)
-                update_scale_kernel<T, (sizeof(T) == 4 ? 8 : 4), (sizeof(T) == 4 ? 2 : 4)><<<nblk, RED_THREADS, hsm, st>>>(
-                    V, nel, w, vn, nel, S, ni, hpass, inv);
-            else if (ni <= 4)
-                update_scale_kernel<T, 4, 4><<<nblk, RED_THREADS, hsm, st>>>(V, nel, w, vn, nel, S, ni, hpass, inv);
-            else
-                update_scale_kernel<T, 2, 8><<<nblk, RED_THREADS, hsm, st>>>(V, nel, w, vn, nel, S, ni, hpass, inv);
-            prof_end(ctx, tk, (double)(ni + 2) * nel * sizeof(cplx<T>));
-        }
-        ctx->launches += 2;
+        const CgsBuffers<T> B{V, w, nel, S, m, nblk, ldp, part, hpass, H, sn, gv, cs, dpart, inv, Sd, running};
+        fused_cgs2(ctx, st, B, j, "arnoldi");
         return cuda_check(ctx, cudaGetLastError(), "Krylov iteration");
     }
 
@@ -968,8 +1055,7 @@ struct Krylov final : KrylovEngine {
         HELM_TRY(oras_apply_wp(o, wp, vj, zj, S));
         HELM_TRY(launch_stencil(o->g, wp, zj, w, S, st));
         // (complex128 bases: up to 16 vectors, the register budget of the fused kernel)
-        if (j + 1 <= (sizeof(T) == 4 ? 32 : 16) && (size_t)(j + 1) * S * sizeof(cplx<T>) <= 40 * 1024)
-            return cgs2_fused(j);
+        if (cgs2_fits<T>(j + 1, S)) return cgs2_fused(j);
         // Classical Gram-Schmidt for column j of H (H[r][i][j]) with a second projection for the
         // columns whose norm dropped below 1/sqrt(2) of its value (selective re-orthogonalisation)
         dots_pass(V, w, j + 1, dpart, nullptr);
@@ -1243,6 +1329,12 @@ helm_status inner_solve_t(helm_oras o, InnerKrylov& K, const cplx<T>* c, cplx<T>
     for (int j = 0; j < m; ++j) {
         HELM_TRY(coarse_dd_apply(o, K.wp, V + (long long)j * nel, u, S));
         HELM_TRY(coarse_E_apply(o, K.wp, u, w, S));
+        if (cgs2_fits<T>(j + 1, S)) {
+            const CgsBuffers<T> B{V, w, nel, S, m, nblk, ldp, K.part, K.hpass, K.H, K.sn, K.gv, K.cs, K.dpart, K.inv, K.Sd,
+                                  K.running};
+            fused_cgs2(ctx, st, B, j, nullptr);
+            continue;
+        }
         // classical Gram-Schmidt with selective re-orthogonalisation, as in the outer iteration
         dots(j + 1, K.dpart, nullptr);
         finish_dots<<<(j + 1) * S, 128, 0, st>>>(K.part, nblk, ldp, j + 1, S, K.H, m, (m + 1) * m, j, 0, nullptr,
