@@ -5,16 +5,17 @@
 // Blocked Gauss-Jordan with block pivots.  For the panel J = [j0, j0 + NB) of the m x m matrix A:
 //   P      = A[J,J]^{-1}                      (NB x NB, Gauss-Jordan with partial pivoting inside the block)
 //   A[J,:] = P A[J,:]  (columns outside J),    A[J,J] = P
-//   A[I,:] = A[I,:] - A[I,J] A[J,:]_new  (rows I outside J, columns outside J)
+//   A[I,:] = A[I,:] - (A[I,J] P) A[J,:]  (rows I outside J, columns outside J; A[J,:] before the step)
 //   A[I,J] = -A[I,J] P                      (rows I outside J)
-// After the last panel A holds S^{-1}.  The last two lines are one product: with W = A[:,J] (before the
-// step) and R = the new rows J (R[:,J] = P), A[I,j] = [j not in J] A[I,j] - (W R)[I,j] for I outside J.
+// After the last panel A holds S^{-1}.  With W[I,:] = A[I,J] P outside J, W[J,:] = -P, and R = A[J,:] before the step
+// with the identity in columns J, all four lines are one product: A = [row and column outside J] A - W R.  So only
+// A[I,J] P (one row of tiles) waits for the block inverse, and it runs on the tensor cores too; R is a copy.
 // Pivoting stays inside each diagonal block: for these Helmholtz Schur complements (condition numbers
 // 1e0-1e2 at the workload sizes) block pivots give the same accuracy as full partial pivoting, and a block
 // pivot below 1e-6 of its block's largest entry is reported so that the caller can fall back to the
 // fully pivoted CUDA-core elimination.
 //
-// The product W R (m x NB times NB x m, complex) is one real GEMM with the 2x2 embedding used by the plane
+// The product W R (m x NB times NB x m, complex; W = A[I,J] P is the same with N = 2 NB) is one real GEMM with the 2x2 embedding used by the plane
 // sweeps: A operand = rows of W read as 2 NB reals (K-major), B operand = B^T[2j][2c] = Re R[c][j],
 // B^T[2j][2c+1] = -Im R[c][j], B^T[2j+1][2c] = Im R[c][j], B^T[2j+1][2c+1] = Re R[c][j].  FP32 accuracy
 // from TF32 units: each operand x is split into hi = x with its low 13 mantissa bits cleared (exact in TF32)
@@ -27,7 +28,6 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "blockinv.cuh"
 #include <atomic>
 
 #include "internal.h"
@@ -43,7 +43,6 @@ constexpr int UST = 2;               // operand ring stages
 constexpr int A_TILE = UBM * 128;    // 128 rows x 32 fp32 = 16 KB
 constexpr int B_TILE = UBN * 128;    // 256 rows x 32 fp32 = 32 KB
 constexpr int STAGE = 2 * A_TILE + 2 * B_TILE;
-constexpr int USMEM = UST * STAGE + 1024 + 128;
 constexpr int DIAG_THREADS = 512;
 constexpr int DP = NB + 1;           // row pitch of the diagonal block in shared memory
 
@@ -137,284 +136,222 @@ __global__ void tgj_pad_diag(const BoxInfo* __restrict__ boxes, c64* __restrict_
         S[(size_t)blockIdx.y * L * L + (size_t)i * L + i] = mk<float>(1.f, 0.f);
 }
 
-// ------------------------------------------------------------------ panel: block inverse, rows, W
+// ------------------------------------------------------------------ panel: block inverse, operands
 
-// P = A[J,J]^{-1} by Gauss-Jordan with partial pivoting inside the block, in 16-column sub-panels (one CTA per
-// box, blockinv.cuh).  flag bit 0: a zero pivot; bit 1: a pivot below 1e-6 of the block's largest entry.
-__global__ void __launch_bounds__(DIAG_THREADS) tgj_diag(const BoxInfo* __restrict__ boxes,
-                                                         const c64* __restrict__ S, int L, c64* __restrict__ Pbuf,
-                                                         int* __restrict__ flag, int j0, int k) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    c64* X = reinterpret_cast<c64*>(dsm);   // [NB][DP], then the sub-panel rows [16][NB]
-    __shared__ c64 s_row[NB], s_col[NB];
-    __shared__ int s_perm[NB], s_pos[NB];
-    __shared__ int s_piv;
-    __shared__ float s_wmax[DIAG_THREADS / 32];
-    const BoxInfo B = boxes[blockIdx.x];
-    const int m = B.m;
-    if (k >= B.dims[2] || j0 >= m) return;
-    const c64* A = S + (size_t)blockIdx.x * L * L;
+// P = A[J,J]^{-1} in shared memory by in-place Gauss-Jordan in sub-panels of SB columns, pivots by largest modulus
+// among the block's rows not used yet.  Rows are not swapped: s_p[c] is the row that column c was eliminated with, and
+// the inverse is P[c][s_p[k]] = X[s_p[c]][k].
+//
+// A sub-panel is eliminated by 128 threads, one row each with its SB entries in registers; per column a 32-bit key
+// (|x|^2 in the high bits, the row in the low seven) is reduced with one redux per warp and the scaled pivot row is
+// broadcast through shared memory: two barriers of four warps per column.  Its accumulated transform W then reaches the
+// other columns in one rank-SB step of all 16 warps, 4 x 8 outputs per thread, X <- [rows not used here] X + W X[pivot rows].
+// Bound: the serial column chain (128 x about 400 clocks) and the rank-SB steps (128^3 complex multiply-adds on one
+// SM's FP32 lanes, 32 us).
+constexpr int SB = 16;
+constexpr int DIAG_SMEM = (NB * DP + SB * NB) * (int)sizeof(c64);
+
+__device__ __forceinline__ void diag_inverse(c64* X, c64* Brow, int* s_p, int* s_k, float amax, int* flag) {
+    __shared__ uint32_t s_key[2][4];
+    __shared__ __align__(16) c64 s_row[2][SB];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    float amax = 0.f;
-    for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
-        const int r = e / NB, c = e % NB;
-        const c64 v = A[(size_t)(j0 + r) * L + j0 + c];
-        X[r * DP + c] = v;
-        amax = fmaxf(amax, v.x * v.x + v.y * v.y);
-    }
+    bool used = false;   // this thread's row (threads below NB)
+    for (int c0 = 0; c0 < NB; c0 += SB) {
+        if (tid < NB) {
+            c64 a[SB];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane == 0) s_wmax[wid] = amax;
-    __syncthreads();
-    amax = 0.f;
-    for (int w = 0; w < DIAG_THREADS / 32; ++w) amax = fmaxf(amax, s_wmax[w]);
-    block_inverse<float, NB, DP, 16, DIAG_THREADS>(X, X + NB * DP, s_perm, s_row, s_col, &s_piv, amax, flag);
-    // the row swaps become a column permutation of the inverse (undone in reverse pivot order)
-    if (tid == 0) {
-        for (int j = 0; j < NB; ++j) s_pos[j] = j;
-        for (int c = NB - 1; c >= 0; --c) {
-            const int p = s_perm[c];
-            const int t = s_pos[c];
-            s_pos[c] = s_pos[p];
-            s_pos[p] = t;
-        }
-    }
-    __syncthreads();
-    c64* Pb = Pbuf + (size_t)blockIdx.x * NB * NB;
-    for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
-        const int r = e / NB, j = e % NB;
-        Pb[e] = X[r * DP + s_pos[j]];
-    }
-}
-
-// R = P A[J, :] for the CTA's 64 columns (R[:, J] = P), written into rows J of A (entries below m) and as
-// the hi / lo parts of the B operand B^T (every column below L, so that the operand is finite everywhere).
-// Thread (tx, ty): rows c = tx + 16 i (i < 8), columns col0 + ty + 16 q (q < 4).
-__global__ void __launch_bounds__(256) tgj_rows(const BoxInfo* __restrict__ boxes, c64* __restrict__ S, int L,
-                                                const c64* __restrict__ Pbuf, float* __restrict__ Bh,
-                                                float* __restrict__ Bl, int j0, int k) {
-    __shared__ c64 Ps[NB][17];
-    __shared__ c64 As[16][64];
-    const BoxInfo B = boxes[blockIdx.y];
-    const int m = B.m;
-    if (k >= B.dims[2] || j0 >= m) return;
-    const int col0 = blockIdx.x * 64;
-    c64* A = S + (size_t)blockIdx.y * L * L;
-    const c64* P = Pbuf + (size_t)blockIdx.y * NB * NB;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    c64 acc[8][4];
+            for (int j = 0; j < SB; ++j) a[j] = X[tid * DP + c0 + j];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+            for (int j = 0; j < SB; ++j) {
+                const int c = c0 + j, pb = j & 1;
+                const float q = a[j].x * a[j].x + a[j].y * a[j].y;
+                // rows not used yet: |x|^2 rounded down to 16 mantissa bits, ties to the smallest row; used: 0
+                const uint32_t key = used ? 0u : ((__float_as_uint(q) & 0xFFFFFF80u) | (uint32_t)(NB - 1 - tid)) + 1u;
+                const uint32_t kw = __reduce_max_sync(0xffffffffu, key);
+                if (lane == 0) s_key[pb][wid] = kw;
+                tc::named_bar(1, NB);
+                const uint32_t km = max(max(s_key[pb][0], s_key[pb][1]), max(s_key[pb][2], s_key[pb][3]));
+                const int p = NB - 1 - (int)((km - 1u) & 127u);
+                if (tid == p) {
+                    if (!(q > 0.f)) atomicOr(flag, 1);
+                    else if (q < 1e-12f * amax) atomicOr(flag, 2);
+                    const float d = q > 0.f ? 1.f / q : 1.f;
+                    const c64 inv = q > 0.f ? mk<float>(a[j].x * d, -a[j].y * d) : mk<float>(1.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = mk<float>(0.f, 0.f);
-    for (int k0 = 0; k0 < NB; k0 += 16) {
-        for (int e = tid; e < NB * 16; e += 256) {
-            const int r = e >> 4, kk = e & 15;
-            Ps[r][kk] = P[r * NB + k0 + kk];
-        }
-        for (int e = tid; e < 16 * 64; e += 256) {
-            const int kk = e >> 6, jj = e & 63;
-            As[kk][jj] = A[(size_t)(j0 + k0 + kk) * L + col0 + jj];
+                    for (int i = 0; i < SB; ++i) {
+                        a[i] = i == j ? inv : a[i] * inv;
+                        s_row[pb][i] = a[i];
+                    }
+                    used = true;
+                    s_p[c] = tid;
+                    s_k[tid] = c;
+                }
+                tc::named_bar(1, NB);
+                if (tid != p) {
+                    const c64 f = mk<float>(-a[j].x, -a[j].y);
+                    a[j] = mk<float>(0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < SB; i += 2) {
+                        const float4 r = *reinterpret_cast<const float4*>(&s_row[pb][i]);
+                        cmac(a[i], f, mk<float>(r.x, r.y));
+                        cmac(a[i + 1], f, mk<float>(r.z, r.w));
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < SB; ++j) X[tid * DP + c0 + j] = a[j];
         }
         __syncthreads();
+        for (int e = tid; e < SB * NB; e += DIAG_THREADS) Brow[e] = X[s_p[c0 + e / NB] * DP + e % NB];
+        __syncthreads();
+        // thread (row group of 4, column group of 8): rows 4 rg .. 4 rg + 3, columns cg + 16 i
+        const int rg = tid >> 4, cg = tid & 15;
+        c64 acc[4][8];
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            c64 a[8], b[4];
+        for (int r = 0; r < 4; ++r) {
+            const int k = s_k[4 * rg + r];
+            const bool piv = k >= c0 && k < c0 + SB;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) a[i] = Ps[tx + 16 * i][kk];
+            for (int i = 0; i < 8; ++i) acc[r][i] = piv ? mk<float>(0.f, 0.f) : X[(4 * rg + r) * DP + cg + 16 * i];
+        }
+#pragma unroll 4
+        for (int c = 0; c < SB; ++c) {
+            c64 w[4], b[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) b[q] = As[kk][ty + 16 * q];
+            for (int r = 0; r < 4; ++r) w[r] = X[(4 * rg + r) * DP + c0 + c];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) b[i] = Brow[c * NB + cg + 16 * i];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) cmac(acc[r][i], w[r], b[i]);
+        }
+        // the sub-panel's own columns (i = c0 / 16) are left as they are
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) cmac(acc[i][q], a[i], b[q]);
-        }
+                if (i != c0 / SB) X[(4 * rg + r) * DP + cg + 16 * i] = acc[r][i];
         __syncthreads();
-    }
-    float* bh = Bh + (size_t)blockIdx.y * 2 * L * K2;
-    float* bl = Bl + (size_t)blockIdx.y * 2 * L * K2;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = col0 + ty + 16 * q;
-        const bool inJ = j >= j0 && j < j0 + NB;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = tx + 16 * i;
-            const c64 v = inJ ? P[c * NB + (j - j0)] : acc[i][q];
-            if (j0 + c < m && j < m) A[(size_t)(j0 + c) * L + j] = v;
-            const float re_h = tf32_hi(v.x), im_h = tf32_hi(v.y);
-            const float re_l = v.x - re_h, im_l = v.y - im_h;
-            float* h0 = bh + (size_t)(2 * j) * K2 + 2 * c;
-            float* l0 = bl + (size_t)(2 * j) * K2 + 2 * c;
-            *reinterpret_cast<float2*>(h0) = make_float2(re_h, -im_h);
-            *reinterpret_cast<float2*>(h0 + K2) = make_float2(im_h, re_h);
-            *reinterpret_cast<float2*>(l0) = make_float2(re_l, -im_l);
-            *reinterpret_cast<float2*>(l0 + K2) = make_float2(im_l, re_l);
-        }
     }
 }
 
-// W = A[:, J] (zero on rows J and rows beyond m) as the hi / lo A operand, rows of 2 NB reals.
-__global__ void __launch_bounds__(256) tgj_wcopy(const BoxInfo* __restrict__ boxes, const c64* __restrict__ S,
-                                                 int L, float* __restrict__ Wh, float* __restrict__ Wl, int j0, int k) {
-    const BoxInfo B = boxes[blockIdx.y];
-    const int m = B.m;
-    if (k >= B.dims[2] || j0 >= m) return;
-    const c64* A = S + (size_t)blockIdx.y * L * L;
-    float* wh = Wh + (size_t)blockIdx.y * L * K2;
-    float* wl = Wl + (size_t)blockIdx.y * L * K2;
-    for (int e = threadIdx.x; e < 32 * NB; e += 256) {
-        const int I = blockIdx.x * 32 + e / NB, c = e % NB;
-        c64 v = mk<float>(0.f, 0.f);
-        if (I < m && !(I >= j0 && I < j0 + NB)) v = A[(size_t)I * L + j0 + c];
-        const float re_h = tf32_hi(v.x), im_h = tf32_hi(v.y);
-        *reinterpret_cast<float2*>(wh + (size_t)I * K2 + 2 * c) = make_float2(re_h, im_h);
-        *reinterpret_cast<float2*>(wl + (size_t)I * K2 + 2 * c) = make_float2(v.x - re_h, v.y - im_h);
+// hi and lo parts of the pair (a, b) at an operand position
+__device__ __forceinline__ void split2(float* h, float* l, size_t at, float a, float b) {
+    const float ah = tf32_hi(a), bh = tf32_hi(b);
+    *reinterpret_cast<float2*>(h + at) = make_float2(ah, bh);
+    *reinterpret_cast<float2*>(l + at) = make_float2(a - ah, b - bh);
+}
+
+// The panel's first launch, in which nothing depends on anything else: CTA b < nbox inverts the diagonal block of box b
+// and writes P as the right operand of W P (Ph, Pl) and -P as rows J of the left operand of the update (Wh, Wl);
+// the other CTAs copy W = A[:, J] (rows outside J; zero beyond m) and A[J, :], with the identity in columns J, as the
+// update's right operand (Bh, Bl; every column below L, so that the operand is finite everywhere).
+__global__ void __launch_bounds__(DIAG_THREADS) tgj_panel(const BoxInfo* __restrict__ boxes, const c64* __restrict__ S,
+                                                          int L, int nbox, float* __restrict__ Wh, float* __restrict__ Wl,
+                                                          float* __restrict__ Ph, float* __restrict__ Pl,
+                                                          float* __restrict__ Bh, float* __restrict__ Bl,
+                                                          int* __restrict__ flag, int j0, int k) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ int s_p[NB], s_k[NB];
+    __shared__ float s_wmax[DIAG_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    c64* X = reinterpret_cast<c64*>(dsm);   // [NB][DP], then the pivot rows of a sub-panel [SB][NB]
+    if ((int)blockIdx.x < nbox) {
+        const int box = blockIdx.x;
+        const int m = boxes[box].m;
+        if (k >= boxes[box].dims[2] || j0 >= m) return;
+        const c64* A = S + (size_t)box * L * L;
+        float amax = 0.f;
+        for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
+            const c64 v = A[(size_t)(j0 + e / NB) * L + j0 + e % NB];
+            X[(e / NB) * DP + e % NB] = v;
+            amax = fmaxf(amax, v.x * v.x + v.y * v.y);
+        }
+        if (tid < NB) s_k[tid] = -1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        if (lane == 0) s_wmax[wid] = amax;
+        __syncthreads();
+        amax = 0.f;
+        for (int w = 0; w < DIAG_THREADS / 32; ++w) amax = fmaxf(amax, s_wmax[w]);
+        diag_inverse(X, X + NB * DP, s_p, s_k, amax, flag);
+        float *wh = Wh + ((size_t)box * L + j0) * K2, *wl = Wl + ((size_t)box * L + j0) * K2;
+        float *ph = Ph + (size_t)box * K2 * K2, *pl = Pl + (size_t)box * K2 * K2;
+        for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
+            const int c = e / NB, q = e % NB;
+            const c64 v = X[s_p[c] * DP + s_k[q]];
+            split2(wh, wl, (size_t)c * K2 + 2 * q, -v.x, -v.y);
+            const c64 u = X[s_p[q] * DP + s_k[c]];   // P[q][c]: rows 2c, 2c + 1 of the right operand, K index q
+            split2(ph, pl, (size_t)(2 * c) * K2 + 2 * q, u.x, -u.y);
+            split2(ph, pl, (size_t)(2 * c + 1) * K2 + 2 * q, u.y, u.x);
+        }
+        return;
+    }
+    const int t32 = L / 32;   // 32-row pieces of W and 32-column pieces of A[J, :] per box
+    for (int it = blockIdx.x - nbox; it < nbox * 2 * t32; it += gridDim.x - nbox) {
+        const int box = it / (2 * t32), part = it % (2 * t32);
+        const int m = boxes[box].m;
+        if (k >= boxes[box].dims[2] || j0 >= m) continue;
+        const c64* A = S + (size_t)box * L * L;
+        if (part < t32) {
+            const int I0 = part * 32;
+            if (I0 >= j0 && I0 < j0 + NB) continue;   // rows J: -P, from the block's CTA
+            float *wh = Wh + ((size_t)box * L + I0) * K2, *wl = Wl + ((size_t)box * L + I0) * K2;
+            for (int e = tid; e < 32 * NB; e += DIAG_THREADS) {
+                const int I = e / NB, c = e % NB;
+                const c64 v = I0 + I < m ? A[(size_t)(I0 + I) * L + j0 + c] : mk<float>(0.f, 0.f);
+                split2(wh, wl, (size_t)I * K2 + 2 * c, v.x, v.y);
+            }
+        } else {
+            const int jc = (part - t32) * 32;
+            __syncthreads();
+            for (int e = tid; e < NB * 32; e += DIAG_THREADS) {
+                const int c = e / 32, jj = e % 32, j = jc + jj;
+                X[c * 33 + jj] = j >= j0 && j < j0 + NB ? mk<float>(c == j - j0 ? 1.f : 0.f, 0.f)
+                                                        : A[(size_t)(j0 + c) * L + j];
+            }
+            __syncthreads();
+            float *bh = Bh + ((size_t)box * 2 * L + 2 * jc) * K2, *bl = Bl + ((size_t)box * 2 * L + 2 * jc) * K2;
+            for (int e = tid; e < 32 * NB; e += DIAG_THREADS) {
+                const int jj = e / NB, c = e % NB;
+                const c64 v = X[c * 33 + jj];
+                split2(bh, bl, (size_t)(2 * jj) * K2 + 2 * c, v.x, -v.y);
+                split2(bh, bl, (size_t)(2 * jj + 1) * K2 + 2 * c, v.y, v.x);
+            }
+        }
     }
 }
 
 // ------------------------------------------------------------------ the rank-NB update on the tensor cores
 
-// Tile (tn, tm, box): rows row0 .. row0 + 127, complex columns col0 .. col0 + 127.  Warp 0 lane 0 issues the
-// TMA loads (W hi, W lo, B^T hi, B^T lo per 32-real K chunk), warp 1 lane 0 the MMAs, all four warps the
-// epilogue (thread t of warp w owns row row0 + 32 w + t): A[I][j] = [j not in J] A[I][j] - D[I][j].
-__global__ void __launch_bounds__(128, 1) tgj_update(const __grid_constant__ CUtensorMap mWh,
-                                                     const __grid_constant__ CUtensorMap mWl,
-                                                     const __grid_constant__ CUtensorMap mBh,
-                                                     const __grid_constant__ CUtensorMap mBl,
-                                                     const BoxInfo* __restrict__ boxes, c64* __restrict__ S, int L,
-                                                     int j0, int k, int* __restrict__ err) {
-    extern __shared__ __align__(1024) unsigned char usm_raw[];
-    const int box = blockIdx.z;
-    const BoxInfo B = boxes[box];
-    const int m = B.m;
-    if (k >= B.dims[2] || j0 >= m) return;
-    const int row0 = blockIdx.y * UBM, col0 = blockIdx.x * (UBN / 2);
-    if (row0 >= m || col0 >= m || row0 == j0) return;   // rows J are the panel's own (NB == UBM, j0 % 128 == 0)
-    unsigned char* base =
-        reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(usm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(base + UST * STAGE);
-    uint64_t* empty = full + UST;
-    uint64_t* done = empty + UST;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < UST; ++i) {
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&empty[i], 1);
-        }
-        tc::mbar_init(done, 1);
-        tc::fence_barrier_init();
-        tc::prefetch_tmap(&mWh);
-        tc::prefetch_tmap(&mWl);
-        tc::prefetch_tmap(&mBh);
-        tc::prefetch_tmap(&mBl);
-    }
-    if (warp == 1) {
-        tc::tmem_alloc(tmem_slot, 256);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = *tmem_slot;
-    constexpr int NKC = K2 / 32;
-    int issued = 0;
-    if (warp == 0 && lane == 0) {
-        for (int kc = 0; kc < NKC; ++kc) {
-            const int st = kc % UST;
-            if (kc >= UST && !tc::mbar_wait(&empty[st], ((kc / UST) - 1) & 1, err, 11)) break;
-            unsigned char* s = base + st * STAGE;
-            tc::mbar_arrive_expect_tx(&full[st], STAGE);
-            tc::tma_load_3d(s, &mWh, kc * 32, row0, box, &full[st]);
-            tc::tma_load_3d(s + A_TILE, &mWl, kc * 32, row0, box, &full[st]);
-            tc::tma_load_3d(s + 2 * A_TILE, &mBh, kc * 32, 2 * col0, box, &full[st]);
-            tc::tma_load_3d(s + 2 * A_TILE + B_TILE, &mBl, kc * 32, 2 * col0, box, &full[st]);
-            ++issued;
-        }
-    } else if (warp == 1 && lane == 0) {
-        constexpr uint32_t idesc = tc::idesc_tf32(UBM, UBN);
-        for (int kc = 0; kc < NKC; ++kc) {
-            const int st = kc % UST;
-            if (!tc::mbar_wait(&full[st], (kc / UST) & 1, err, 12)) break;
-            tc::fence_after_sync();
-            const uint32_t sah = tc::smem_u32(base + st * STAGE);
-            const uint32_t sal = sah + A_TILE, sbh = sah + 2 * A_TILE, sbl = sbh + B_TILE;
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ah = tc::desc_k_sw128(sah + kk * 32), al = tc::desc_k_sw128(sal + kk * 32);
-                const uint64_t bh = tc::desc_k_sw128(sbh + kk * 32), bl = tc::desc_k_sw128(sbl + kk * 32);
-                tc::mma_tf32(tmem, ah, bh, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-                tc::mma_tf32(tmem, ah, bl, idesc, 1u);
-                tc::mma_tf32(tmem, al, bh, idesc, 1u);
-            }
-            tc::mma_commit(&empty[st]);
-        }
-        tc::mma_commit(done);
-    }
-    __syncwarp();
-    const bool ok = tc::mbar_wait(done, 0, err, 13);
-    if (!ok) tc::mbar_drain(done, 0);   // products already issued still write TMEM
-    tc::fence_after_sync();
-    if (!ok && threadIdx.x == 0)
-        for (int kc = max(0, issued - UST); kc < issued; ++kc) tc::mbar_drain(&full[kc % UST], (kc / UST) & 1);
-    const int I = row0 + warp * 32 + lane;
-    if (ok) {
-        const bool zero_base = col0 == j0;   // the panel's columns: A[I,J] = -W P
-        c64* arow = S + (size_t)box * L * L + (size_t)I * L + col0;
-#pragma unroll 1
-        for (int cc = 0; cc < UBN / 32; ++cc) {
-            uint32_t v[32];
-            tc::tmem_ld_32x32b_x32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cc * 32), v);
-            tc::tmem_ld_wait();
-            if (I < m) {
-#pragma unroll
-                for (int q = 0; q < 16; q += 2) {
-                    const int j = col0 + cc * 16 + q;   // complex columns j and j + 1
-                    float4* dst = reinterpret_cast<float4*>(arow + cc * 16 + q);
-                    if (j + 1 < m) {
-                        const float4 o = zero_base ? make_float4(0.f, 0.f, 0.f, 0.f) : *dst;
-                        *dst = make_float4(o.x - __uint_as_float(v[2 * q]), o.y - __uint_as_float(v[2 * q + 1]),
-                                           o.z - __uint_as_float(v[2 * q + 2]), o.w - __uint_as_float(v[2 * q + 3]));
-                    } else if (j < m) {
-                        c64* d1 = arow + cc * 16 + q;
-                        const c64 o = zero_base ? mk<float>(0.f, 0.f) : *d1;
-                        *d1 = mk<float>(o.x - __uint_as_float(v[2 * q]), o.y - __uint_as_float(v[2 * q + 1]));
-                    }
-                }
-            }
-        }
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 1) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, 256);
-    }
-}
-
-// Persistent form of the update: one CTA per SM takes the launch's tiles in turn (tile t = box-major, then row
-// tile, then column tile, every gridDim.x-th one), with two TMEM accumulators so that the epilogue of one tile
-// runs while the products of the next are issued.  Warp 0 lane 0 loads the operands (TMA, 2-stage ring),
-// warp 1 lane 0 issues the MMAs, warps 2-5 read the accumulator (warp w owns TMEM lanes 32 (w mod 4)..) and
-// write -D back through shared memory with TMA: a reduce-add into A for the columns outside J (A - D), a
-// store for the panel's own columns (-W P).  The padding diagonal a store overwrites in the panel's column
-// tile is restored before the next plane.  Every wait is bounded; on a give-up each role leaves its loop,
+// The panel's two products, persistent: one CTA per SM takes the launch's tiles in turn (every gridDim.x-th one), with two
+// TMEM accumulators so that the epilogue of one tile runs while the products of the next are issued.  Warp 0 lane 0
+// loads the operands (TMA, 2-stage ring), warp 1 lane 0 issues the MMAs, warps 2-5 read the accumulator (warp w owns
+// TMEM lanes 32 (w mod 4)..) and write it back through shared memory with TMA.
+// WP (tile = box, row tile outside J): W <- W P in place, split into hi and lo again: a tile reads only its own rows of W,
+//   all before its first store.
+// update (tile = box, row tile, column tile): -D with D = W B is added into A (reduce-add) outside rows and columns J,
+//   and stored in them (A[I,J] = -W P, A[J,:] = P A[J,:], the left operand's rows J being -P).
+// The padding diagonal is restored before the next plane.  Every wait is bounded; on a give-up each role leaves its loop,
 // copies and products already issued are waited for, and TMEM is freed.
 constexpr int PW = 6;                     // warps: producer, MMA issuer, four epilogue warps
 constexpr int STG = 2 * UBM * 128;        // staging: two 128-row x 32-float boxes (32 KB)
 constexpr int PSMEM = UST * STAGE + STG + 1024 + 256;
 
+template <bool WP>
 __device__ __forceinline__ bool tile_of(const BoxInfo* __restrict__ boxes, int t, int tl, int j0, int k, int& box,
                                         int& row0, int& col0) {
-    box = t / (tl * tl);
-    const int r = t % (tl * tl);
-    row0 = (r / tl) * UBM;
-    col0 = (r % tl) * (UBN / 2);
+    const int per = WP ? tl : tl * tl;
+    box = t / per;
+    const int r = t % per;
+    row0 = (WP ? r : r / tl) * UBM;
+    col0 = WP ? 0 : (r % tl) * (UBN / 2);
     const BoxInfo& B = boxes[box];
-    return k < B.dims[2] && j0 < B.m && row0 < B.m && col0 < B.m && row0 != j0;
+    return k < B.dims[2] && j0 < B.m && row0 < B.m && col0 < B.m && !(WP && row0 == j0);
 }
 
+template <bool WP>
 __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_constant__ CUtensorMap mWh,
                                                               const __grid_constant__ CUtensorMap mWl,
                                                               const __grid_constant__ CUtensorMap mBh,
@@ -435,7 +372,7 @@ __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_const
     int* s_go = reinterpret_cast<int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tl = L / UBM;
-    const int ntiles = nbox * tl * tl;
+    const int ntiles = nbox * (WP ? tl : tl * tl);
     if (threadIdx.x == 0) {
         for (int i = 0; i < UST; ++i) {
             tc::mbar_init(&full[i], 1);
@@ -468,7 +405,7 @@ __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_const
             uint32_t g = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                if (!tile_of(boxes, t, tl, j0, k, box, row0, col0)) continue;
+                if (!tile_of<WP>(boxes, t, tl, j0, k, box, row0, col0)) continue;
                 for (int kc = 0; kc < NKC; ++kc, ++g) {
                     const int st = g % UST;
                     if (g >= UST && !tc::mbar_wait(&empty[st], ((g / UST) - 1) & 1, err, 21)) {
@@ -493,7 +430,7 @@ __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_const
             uint32_t g = 0, i = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                if (!tile_of(boxes, t, tl, j0, k, box, row0, col0)) continue;
+                if (!tile_of<WP>(boxes, t, tl, j0, k, box, row0, col0)) continue;
                 const uint32_t a = i & 1, u = i >> 1;
                 if (u >= 1 && !tc::mbar_wait(&tempty[a], (u - 1) & 1, err, 22)) break;
                 tc::fence_after_sync();
@@ -532,20 +469,22 @@ __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_const
         const int r = q * 32 + lane;            // tile row of this thread
         uint32_t i = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-            if (!tile_of(boxes, t, tl, j0, k, box, row0, col0)) continue;
+            if (!tile_of<WP>(boxes, t, tl, j0, k, box, row0, col0)) continue;
             const uint32_t a = i & 1, u = i >> 1;
             if (et == 0) *s_go = tc::mbar_wait(&tfull[a], u & 1, err, 24) ? 1 : 0;
             tc::named_bar(1, 128);
             if (!*s_go) break;                  // uniform over the four warps
             tc::fence_after_sync();
-            const bool store = col0 == j0;      // the panel's own columns: A[I,J] = -W P
-            for (int c = 0; c < UBN / 64; ++c) {
+            const bool store = col0 == j0 || row0 == j0;   // the panel's own rows and columns
+            // per trip, update: 64 columns (two boxes of 32); WP: 32 columns, their hi and lo parts
+            constexpr int CW = WP ? 32 : 64;
+            for (int c = 0; c < UBN / CW; ++c) {
                 uint32_t v[2][32];
-                const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + a * 256 + c * 64;
+                const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + a * 256 + c * CW;
                 tc::tmem_ld_32x32b_x32(ta, v[0]);
-                tc::tmem_ld_32x32b_x32(ta + 32, v[1]);
+                if (!WP) tc::tmem_ld_32x32b_x32(ta + 32, v[1]);
                 tc::tmem_ld_wait();
-                if (c == UBN / 64 - 1) {
+                if (c == UBN / CW - 1) {
                     // the accumulator has been read: the MMA issuer may reuse it
                     tc::fence_before_sync();
                     __syncwarp();
@@ -558,20 +497,32 @@ __global__ void __launch_bounds__(PW * 32, 1) tgj_update_pers(const __grid_const
                     unsigned char* rowp = stg + h * (UBM * 128) + r * 128;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const float4 val = make_float4(-__uint_as_float(v[h][4 * j]), -__uint_as_float(v[h][4 * j + 1]),
-                                                       -__uint_as_float(v[h][4 * j + 2]),
-                                                       -__uint_as_float(v[h][4 * j + 3]));
-                        *reinterpret_cast<float4*>(rowp + ((j ^ (r & 7)) << 4)) = val;
+                        float x[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (WP) {
+                                const float f = __uint_as_float(v[0][4 * j + e]), fh = tf32_hi(f);
+                                x[e] = h == 0 ? fh : f - fh;
+                            } else {
+                                x[e] = -__uint_as_float(v[h][4 * j + e]);
+                            }
+                        }
+                        *reinterpret_cast<float4*>(rowp + ((j ^ (r & 7)) << 4)) = make_float4(x[0], x[1], x[2], x[3]);
                     }
                 }
                 tc::fence_proxy_async_smem();
                 tc::named_bar(1, 128);
                 if (et == 0) {
+                    if (WP) {
+                        tc::tma_store_3d(&mWh, stg, c * 32, row0, box);
+                        tc::tma_store_3d(&mWl, stg + UBM * 128, c * 32, row0, box);
+                    } else {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int x = 2 * col0 + c * 64 + h * 32;
-                        if (store) tc::tma_store_3d(&mS, stg + h * (UBM * 128), x, row0, box);
-                        else tc::tma_reduce_add_3d(&mS, stg + h * (UBM * 128), x, row0, box);
+                        for (int h = 0; h < 2; ++h) {
+                            const int x = 2 * col0 + c * 64 + h * 32;
+                            if (store) tc::tma_store_3d(&mS, stg + h * (UBM * 128), x, row0, box);
+                            else tc::tma_reduce_add_3d(&mS, stg + h * (UBM * 128), x, row0, box);
+                        }
                     }
                     tc::bulk_commit();
                 }
@@ -656,8 +607,8 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
     const size_t s_bytes = nb * L * L * sizeof(c64);
     const size_t w_bytes = nb * L * K2 * sizeof(float);
     const size_t b_bytes = nb * 2 * L * K2 * sizeof(float);
-    const size_t p_bytes = nb * NB * NB * sizeof(c64);
-    void *S = nullptr, *T = nullptr, *Wh = nullptr, *Wl = nullptr, *Bh = nullptr, *Bl = nullptr, *Pb = nullptr;
+    const size_t p_bytes = nb * K2 * K2 * sizeof(float);
+    void *S = nullptr, *T = nullptr, *Wh = nullptr, *Wl = nullptr, *Bh = nullptr, *Bl = nullptr, *Ph = nullptr, *Pl = nullptr;
     int* flag = nullptr;   // [0] pivots, [1] bounded waits
     auto cleanup = [&]() {
         dev_free(ctx, S, s_bytes);
@@ -666,7 +617,8 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
         dev_free(ctx, Wl, w_bytes);
         dev_free(ctx, Bh, b_bytes);
         dev_free(ctx, Bl, b_bytes);
-        dev_free(ctx, Pb, p_bytes);
+        dev_free(ctx, Ph, p_bytes);
+        dev_free(ctx, Pl, p_bytes);
         dev_free(ctx, flag, 2 * sizeof(int));
     };
     helm_status rc;
@@ -674,33 +626,34 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
         (rc = dev_alloc(ctx, &T, s_bytes, "tensor-core factor work T")) ||
         (rc = dev_alloc(ctx, &Wh, w_bytes, "factor operand W")) || (rc = dev_alloc(ctx, &Wl, w_bytes, "factor operand W")) ||
         (rc = dev_alloc(ctx, &Bh, b_bytes, "factor operand B")) || (rc = dev_alloc(ctx, &Bl, b_bytes, "factor operand B")) ||
-        (rc = dev_alloc(ctx, &Pb, p_bytes, "block pivots")) ||
+        (rc = dev_alloc(ctx, &Ph, p_bytes, "block pivots")) || (rc = dev_alloc(ctx, &Pl, p_bytes, "block pivots")) ||
         (rc = dev_alloc(ctx, (void**)&flag, 2 * sizeof(int), "factor flags"))) {
         cleanup();
         return rc;
     }
-    CUtensorMap mWh, mWl, mBh, mBl, mS;
+    CUtensorMap mWh, mWl, mBh, mBl, mPh, mPl, mS;
     if (!encode_operand(&mWh, Wh, L, nb, UBM) || !encode_operand(&mWl, Wl, L, nb, UBM) ||
         !encode_operand(&mBh, Bh, 2ull * L, nb, UBN) || !encode_operand(&mBl, Bl, 2ull * L, nb, UBN) ||
-        !encode_matrix(&mS, S, L, nb)) {
+        !encode_operand(&mPh, Ph, K2, nb, UBN) || !encode_operand(&mPl, Pl, K2, nb, UBN) || !encode_matrix(&mS, S, L, nb)) {
         cleanup();
         return set_error(ctx, HELM_ECUDA, "cuTensorMapEncodeTiled failed for the tensor-core factorisation");
     }
     static std::atomic<bool> attr{false};
     if (!attr.load(std::memory_order_acquire)) {
-        cudaFuncSetAttribute(tgj_update, cudaFuncAttributeMaxDynamicSharedMemorySize, USMEM);
-        cudaFuncSetAttribute(tgj_update_pers, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
-        cudaFuncSetAttribute(tgj_diag, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((NB * DP + 16 * NB) * sizeof(c64)));
+        cudaFuncSetAttribute(tgj_update_pers<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
+        cudaFuncSetAttribute(tgj_update_pers<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
+        cudaFuncSetAttribute(tgj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, DIAG_SMEM);
         attr.store(true, std::memory_order_release);
     }
     cudaMemsetAsync(S, 0, s_bytes, st);
     cudaMemsetAsync(flag, 0, 2 * sizeof(int), st);
     const c64* coef = (const c64*)P.coef;
     const int tl = L / NB;
-    // tc_factor 1: persistent update (one CTA per SM, overlapped epilogue); 2: one CTA per tile
-    const bool persistent = ctx->tc_factor == 1;
-    const int pgrid = std::max(1, std::min(ctx->sm_count, P.nbox * tl * tl));
+    const int sms = std::max(1, ctx->sm_count);
+    const int pgrid = std::min(sms, P.nbox * tl * tl), wgrid = std::min(sms, P.nbox * tl);
+    // the block inverses (one CTA each) and the copying CTAs beside them: the SMs the blocks leave free, half of them at
+    // least
+    const int cgrid = P.nbox + std::max(sms - P.nbox, sms / 2);
     const unsigned eb = (unsigned)std::min<long long>(((long long)P.m_max * P.m_max + 255) / 256, 2048);
     const dim3 egrid(eb, P.nbox);
     tgj_pad_diag<<<dim3(1, P.nbox), 128, 0, st>>>(P.dbox, (c64*)S, L);
@@ -709,7 +662,7 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
     // its matrix once; of one panel (block inverse, rows, W): the block, the rows J, the column block J and
     // the operands written
     for (int k = 0; k < P.bz_max; ++k) {
-        if (k > 0 && persistent) {
+        if (k > 0) {
             // the padding diagonal that the panel's column store may have overwritten in the last plane
             tgj_pad_diag<<<dim3(1, P.nbox), 128, 0, st>>>(P.dbox, (c64*)S, L);
             ctx->launches++;
@@ -731,21 +684,19 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
                     pb += (2.0 * NB * b.m + (double)NB * b.m) * sizeof(c64) + (2.0 * 2 * b.m + b.m) * K2 * sizeof(float);
                 }
             int t = prof_begin(ctx, "gj_panel_tc");
-            tgj_diag<<<P.nbox, DIAG_THREADS, (NB * DP + 16 * NB) * sizeof(c64), st>>>(P.dbox, (const c64*)S, L, (c64*)Pb, flag,
-                                                                          j0, k);
-            tgj_rows<<<dim3(L / 64, P.nbox), 256, 0, st>>>(P.dbox, (c64*)S, L, (const c64*)Pb, (float*)Bh, (float*)Bl,
-                                                           j0, k);
-            tgj_wcopy<<<dim3(L / 32, P.nbox), 256, 0, st>>>(P.dbox, (const c64*)S, L, (float*)Wh, (float*)Wl, j0, k);
+            tgj_panel<<<cgrid, DIAG_THREADS, DIAG_SMEM, st>>>(P.dbox, (const c64*)S, L, P.nbox, (float*)Wh, (float*)Wl,
+                                                              (float*)Ph, (float*)Pl, (float*)Bh, (float*)Bl, flag, j0, k);
+            if (tl > 1) {   // W P is empty when the panel is the whole matrix
+                tgj_update_pers<true><<<wgrid, PW * 32, PSMEM, st>>>(mWh, mWl, mPh, mPl, mS, P.dbox, P.nbox, L, j0, k,
+                                                                     flag + 1);
+                ctx->launches++;
+            }
             prof_end(ctx, t, pb);
             t = prof_begin(ctx, "gj_update_tc");
-            if (persistent)
-                tgj_update_pers<<<pgrid, PW * 32, PSMEM, st>>>(mWh, mWl, mBh, mBl, mS, P.dbox, P.nbox, L, j0, k,
-                                                               flag + 1);
-            else
-                tgj_update<<<dim3(tl, tl, P.nbox), 128, USMEM, st>>>(mWh, mWl, mBh, mBl, P.dbox, (c64*)S, L, j0, k,
-                                                                     flag + 1);
+            tgj_update_pers<false><<<pgrid, PW * 32, PSMEM, st>>>(mWh, mWl, mBh, mBl, mS, P.dbox, P.nbox, L, j0, k,
+                                                                  flag + 1);
             prof_end(ctx, t, ub);
-            ctx->launches += 4;
+            ctx->launches += 2;
         }
         tgj_store<<<egrid, 256, 0, st>>>(P.dbox, (const c64*)S, L, (c64*)P.G, k);
         ctx->launches++;
