@@ -145,10 +145,14 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * makes oras_factor factor the set again with full partial pivoting.  0 always uses the fully pivoted
  * Gauss-Jordan on the CUDA cores.  Read by oras_factor. */
 #define HELM_TUNE_TC_FACTOR 7
-/* HELM_TUNE_BLOCK_GJ: 1 (default) factors the other plane sets (FP64 and FP32 local factors, the FP64
- * coarse problem) by the same blocked Gauss-Jordan with block pivots on the CUDA cores (64-column panels for
- * complex64, 32 for complex128; the rank-NB updates spread over every SM), falling back to full partial pivoting after a tiny block
- * pivot; 0 always uses the fully pivoted elimination.  Read by oras_factor. */
+/* HELM_TUNE_BLOCK_GJ: how the other plane sets (FP64 and FP32 local factors, the FP64 coarse problem) are factored.
+ * 2 (default): FP64 planes by the tensor-core elimination in complex64 and two Newton steps whose products are exact
+ * sums of integer digits on the tensor cores (inverses good to FP64; planes of up to 2304 unknowns, a workspace of up to
+ * 4 GB while factoring); a tiny block pivot, a plane that does not come out to FP64 or a workspace that does not fit the
+ * budget goes to 1.  FP32 planes as with 1.  1: the same blocked Gauss-Jordan as the tensor-core elimination with
+ * block pivots on the CUDA cores (64-column panels for complex64, 32 for complex128; the rank-NB updates spread over every
+ * SM), falling back to full partial pivoting after a tiny block pivot.  0: always the fully pivoted elimination.  Read by
+ * oras_factor. */
 #define HELM_TUNE_BLOCK_GJ 8
 /* HELM_TUNE_STENCIL_PLANES: output planes per block of the z-marching stencil (HELM_TUNE_STENCIL_MARCH), at
  * any size of the call; 0 (default) picks the block shape and the planes per grid from an estimate of the

@@ -140,7 +140,7 @@ extern "C" helm_status helm_set_tuning(helm_ctx ctx, int key, int value) {
         return HELM_OK;
     }
     if (key == HELM_TUNE_BLOCK_GJ) {
-        if (value != 0 && value != 1) return set_error(ctx, HELM_EINVAL, "helm_set_tuning: block_gj must be 0 or 1");
+        if (value < 0 || value > 2) return set_error(ctx, HELM_EINVAL, "helm_set_tuning: block_gj must be 0..2");
         ctx->block_gj = value;
         return HELM_OK;
     }

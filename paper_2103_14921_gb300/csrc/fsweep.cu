@@ -98,6 +98,8 @@ extern "C" helm_status helm_frequency_sweep(helm_ctx ctx, const helm_sweep_desc*
         ctx2->tc_flow = ctx->tc_flow;
         ctx2->stencil_march = ctx->stencil_march;
         ctx2->stencil_planes = ctx->stencil_planes;
+        ctx2->tc_factor = ctx->tc_factor;
+        ctx2->block_gj = ctx->block_gj;
     }
     auto ctx_of = [&](int i) { return (d->overlap && (i & 1)) ? ctx2 : ctx; };
 

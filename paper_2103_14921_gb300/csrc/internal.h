@@ -78,7 +78,8 @@ struct helm_ctx_s {
     int stencil_planes = 0;    // tuning: output planes per z-march block (0 = chosen per grid)
     long long flow_wait_us = 2000000;   // tuning: bound of the persistent sweep's queue-slot wait (microseconds)
     int tc_factor = 1;         // tuning: tensor-core blocked Gauss-Jordan for complex64 tensor-core factor sets
-    int block_gj = 1;          // tuning: block-pivot Gauss-Jordan on the CUDA cores for the other factor sets
+    int block_gj = 2;          // tuning: the other factor sets: 1 block-pivot Gauss-Jordan on the CUDA cores, 2 the same
+                               // for complex64, tensor-core inverses with Newton steps for complex128
     uint64_t factor_fallbacks = 0;   // sets refactored with full pivoting after a tiny block pivot
     uint64_t graph_gen = 1;    // bumped when a setting that captured graphs depend on changes
     cudaStream_t cap_stream = nullptr;   // private stream graphs are captured on (the context's may be

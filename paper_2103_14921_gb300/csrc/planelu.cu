@@ -32,6 +32,7 @@
 #include <atomic>
 
 #include "internal.h"
+#include "tgj.h"
 
 namespace {
 
@@ -981,6 +982,78 @@ helm_status factor_block_t(helm_ctx ctx, PlaneSet& P, int* singular, int* weak) 
     return rc;
 }
 
+// complex128 set from complex64 inverses and Newton steps on the tensor cores (planelu_dp.cu), a batch of boxes at a
+// time so that the workspace stays within 4 GB.  *ok = false: no room, a tiny pivot or a plane that did not come out to
+// FP64 (the caller then eliminates in FP64).
+helm_status factor_newton(helm_ctx ctx, PlaneSet& P, bool* ok) {
+    *ok = false;
+    cudaStream_t st = ctx->stream;
+    const int m = P.m_max;
+    const size_t mm = (size_t)m * m;
+    auto bytes = [&](int nb) { return tgj_bytes(nb, m) + dp_bytes(nb, m) + 3 * (size_t)nb * mm * sizeof(c128); };
+    if (m > 2304) return HELM_OK;   // longer sums of digit products are not covered
+    int batch = P.nbox;
+    while (batch > 1 && bytes(batch) > ((size_t)4 << 30)) batch = (batch + 1) / 2;
+    TgjWork T;
+    DpWork D;
+    c128 *S = nullptr, *Tm = nullptr;
+    auto cleanup = [&]() {
+        dev_free(ctx, S, (size_t)batch * mm * sizeof(c128));
+        dev_free(ctx, Tm, (size_t)batch * mm * sizeof(c128));
+        dp_free(ctx, D);
+        tgj_free(ctx, T);
+    };
+    if (tgj_alloc(ctx, batch, m, T) || dp_alloc(ctx, batch, m, D) ||
+        dev_alloc(ctx, (void**)&S, (size_t)batch * mm * sizeof(c128), "factor work S") ||
+        dev_alloc(ctx, (void**)&Tm, (size_t)batch * mm * sizeof(c128), "factor work T")) {
+        cleanup();
+        ctx->last_error.clear();   // not an error of the caller's: the general elimination needs less room
+        return HELM_OK;
+    }
+    const c128* coef = (const c128*)P.coef;
+    c128* G = (c128*)P.G;
+    int hflag[2] = {0, 0};
+    helm_status rc = HELM_OK;
+    for (int b0 = 0; b0 < P.nbox && rc == HELM_OK && !hflag[0] && !hflag[1]; b0 += batch) {
+        const int nb = std::min(batch, P.nbox - b0);
+        const BoxInfo* dbox = P.dbox + b0;
+        const BoxInfo* hbox = P.hbox.data() + b0;
+        if (b0 > 0) {
+            // the padding of the work matrices and slices is zero: boxes of another size follow
+            cudaMemsetAsync(T.S, 0, T.s_bytes, st);
+            cudaMemsetAsync(D.AS, 0, D.as_bytes, st);
+            cudaMemsetAsync(D.AX, 0, D.ax_bytes, st);
+            cudaMemsetAsync(D.B, 0, D.b_bytes, st);
+        }
+        int mb = 0, bz = 0;
+        for (int i = 0; i < nb; ++i) {
+            mb = std::max(mb, hbox[i].m);
+            bz = std::max(bz, hbox[i].dims[2]);
+        }
+        const dim3 egrid((unsigned)std::min<long long>(((long long)mb * mb + 255) / 256, 4096), nb);
+        for (int k = 0; k < bz; ++k) {
+            if (k == 0) {
+                schur_init<double><<<egrid, 256, 0, st>>>(dbox, coef, S, m, k);
+                ctx->launches++;
+            } else {
+                schur_gu<double><<<egrid, 256, 0, st>>>(dbox, coef, G, Tm, m, k);
+                schur_lt<double><<<egrid, 256, 0, st>>>(dbox, coef, Tm, S, m, k);
+                ctx->launches += 2;
+            }
+            dp_invert(ctx, T, D, dbox, hbox, nb, mb, k, S, Tm, G);
+        }
+        rc = cuda_check(ctx, cudaGetLastError(), "plane factorisation launch");
+        if (rc) break;
+        cudaMemcpyAsync(hflag, T.flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+        rc = cuda_check(ctx, cudaStreamSynchronize(st), "plane factorisation");
+    }
+    cleanup();
+    if (rc) return rc;
+    if (hflag[1]) return set_error(ctx, HELM_ETIMEOUT, "plane factorisation: a bounded wait gave up");
+    *ok = hflag[0] == 0;
+    return HELM_OK;
+}
+
 template <typename T, int RN>
 void launch_sweep_rn(const PlaneSet& P, cplx<T>* loc, cplx<T>* rbuf, int nrhs, cudaStream_t st, helm_ctx ctx) {
     const int m = P.m_max;
@@ -1138,6 +1211,14 @@ helm_status planeset_factor(helm_ctx ctx, PlaneSet& P, int* singular) {
         if (!weak && !*singular) return HELM_OK;
         ctx->factor_fallbacks++;   // a tiny (or zero) block pivot: factor the set again with full partial pivoting
     } else if (!P.padded && ctx->block_gj) {
+        if (P.prec == HELM_PREC_FP64 && ctx->block_gj == 2) {
+            bool ok = false;
+            HELM_TRY(factor_newton(ctx, P, &ok));
+            if (ok) {
+                *singular = 0;
+                return HELM_OK;
+            }
+        }
         if (P.prec == HELM_PREC_FP64) HELM_TRY(factor_block_t<double>(ctx, P, singular, &weak));
         else HELM_TRY(factor_block_t<float>(ctx, P, singular, &weak));
         if (!weak && !*singular) return HELM_OK;

@@ -32,6 +32,7 @@
 
 #include "internal.h"
 #include "tc.cuh"
+#include "tgj.h"
 
 namespace {
 
@@ -594,48 +595,49 @@ bool encode_operand(CUtensorMap* map, void* base, uint64_t rows, uint64_t nb, ui
 
 }  // namespace
 
-// Tensor-core factorisation of a padded complex64 plane set (the fine sets of TF32 / BF16 factors).
-// *singular: a zero block pivot; *weak: a block pivot below 1e-6 of its block (the caller then factors the
-// set again with full partial pivoting).  Returns HELM_ETIMEOUT if a bounded wait of the update gave up.
-helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* weak) {
-    *singular = *weak = 0;
-    if (P.prec != HELM_PREC_FP32 || !P.padded)
-        return set_error(ctx, HELM_EINVAL, "planeset_factor_tc: needs a padded complex64 set");
-    cudaStream_t st = ctx->stream;
-    const int L = (P.m_max + NB - 1) / NB * NB;
-    const size_t nb = (size_t)P.nbox;
-    const size_t s_bytes = nb * L * L * sizeof(c64);
-    const size_t w_bytes = nb * L * K2 * sizeof(float);
-    const size_t b_bytes = nb * 2 * L * K2 * sizeof(float);
-    const size_t p_bytes = nb * K2 * K2 * sizeof(float);
-    void *S = nullptr, *T = nullptr, *Wh = nullptr, *Wl = nullptr, *Bh = nullptr, *Bl = nullptr, *Ph = nullptr, *Pl = nullptr;
-    int* flag = nullptr;   // [0] pivots, [1] bounded waits
-    auto cleanup = [&]() {
-        dev_free(ctx, S, s_bytes);
-        dev_free(ctx, T, s_bytes);
-        dev_free(ctx, Wh, w_bytes);
-        dev_free(ctx, Wl, w_bytes);
-        dev_free(ctx, Bh, b_bytes);
-        dev_free(ctx, Bl, b_bytes);
-        dev_free(ctx, Ph, p_bytes);
-        dev_free(ctx, Pl, p_bytes);
-        dev_free(ctx, flag, 2 * sizeof(int));
-    };
+size_t tgj_bytes(int nb, int m_max) {
+    const size_t L = (m_max + NB - 1) / NB * NB;
+    return (size_t)nb * (L * L * sizeof(c64) + 6 * L * K2 * sizeof(float) + 2 * (size_t)K2 * K2 * sizeof(float));
+}
+
+void tgj_free(helm_ctx ctx, TgjWork& W) {
+    dev_free(ctx, W.S, W.s_bytes);
+    dev_free(ctx, W.Wh, W.w_bytes);
+    dev_free(ctx, W.Wl, W.w_bytes);
+    dev_free(ctx, W.Bh, W.b_bytes);
+    dev_free(ctx, W.Bl, W.b_bytes);
+    dev_free(ctx, W.Ph, W.p_bytes);
+    dev_free(ctx, W.Pl, W.p_bytes);
+    dev_free(ctx, W.flag, 2 * sizeof(int));
+    W.S = W.Wh = W.Wl = W.Bh = W.Bl = W.Ph = W.Pl = nullptr;
+    W.flag = nullptr;
+}
+
+helm_status tgj_alloc(helm_ctx ctx, int nbox, int m_max, TgjWork& W) {
+    const int L = (m_max + NB - 1) / NB * NB;
+    const size_t nb = (size_t)nbox;
+    W.nb = nbox;
+    W.L = L;
+    W.s_bytes = nb * L * L * sizeof(c64);
+    W.w_bytes = nb * L * K2 * sizeof(float);
+    W.b_bytes = nb * 2 * L * K2 * sizeof(float);
+    W.p_bytes = nb * K2 * K2 * sizeof(float);
     helm_status rc;
-    if ((rc = dev_alloc(ctx, &S, s_bytes, "tensor-core factor work S")) ||
-        (rc = dev_alloc(ctx, &T, s_bytes, "tensor-core factor work T")) ||
-        (rc = dev_alloc(ctx, &Wh, w_bytes, "factor operand W")) || (rc = dev_alloc(ctx, &Wl, w_bytes, "factor operand W")) ||
-        (rc = dev_alloc(ctx, &Bh, b_bytes, "factor operand B")) || (rc = dev_alloc(ctx, &Bl, b_bytes, "factor operand B")) ||
-        (rc = dev_alloc(ctx, &Ph, p_bytes, "block pivots")) || (rc = dev_alloc(ctx, &Pl, p_bytes, "block pivots")) ||
-        (rc = dev_alloc(ctx, (void**)&flag, 2 * sizeof(int), "factor flags"))) {
-        cleanup();
+    if ((rc = dev_alloc(ctx, &W.S, W.s_bytes, "tensor-core factor work S")) ||
+        (rc = dev_alloc(ctx, &W.Wh, W.w_bytes, "factor operand W")) ||
+        (rc = dev_alloc(ctx, &W.Wl, W.w_bytes, "factor operand W")) ||
+        (rc = dev_alloc(ctx, &W.Bh, W.b_bytes, "factor operand B")) ||
+        (rc = dev_alloc(ctx, &W.Bl, W.b_bytes, "factor operand B")) ||
+        (rc = dev_alloc(ctx, &W.Ph, W.p_bytes, "block pivots")) || (rc = dev_alloc(ctx, &W.Pl, W.p_bytes, "block pivots")) ||
+        (rc = dev_alloc(ctx, (void**)&W.flag, 2 * sizeof(int), "factor flags"))) {
+        tgj_free(ctx, W);
         return rc;
     }
-    CUtensorMap mWh, mWl, mBh, mBl, mPh, mPl, mS;
-    if (!encode_operand(&mWh, Wh, L, nb, UBM) || !encode_operand(&mWl, Wl, L, nb, UBM) ||
-        !encode_operand(&mBh, Bh, 2ull * L, nb, UBN) || !encode_operand(&mBl, Bl, 2ull * L, nb, UBN) ||
-        !encode_operand(&mPh, Ph, K2, nb, UBN) || !encode_operand(&mPl, Pl, K2, nb, UBN) || !encode_matrix(&mS, S, L, nb)) {
-        cleanup();
+    if (!encode_operand(&W.mWh, W.Wh, L, nb, UBM) || !encode_operand(&W.mWl, W.Wl, L, nb, UBM) ||
+        !encode_operand(&W.mBh, W.Bh, 2ull * L, nb, UBN) || !encode_operand(&W.mBl, W.Bl, 2ull * L, nb, UBN) ||
+        !encode_operand(&W.mPh, W.Ph, K2, nb, UBN) || !encode_operand(&W.mPl, W.Pl, K2, nb, UBN) ||
+        !encode_matrix(&W.mS, W.S, L, nb)) {
+        tgj_free(ctx, W);
         return set_error(ctx, HELM_ECUDA, "cuTensorMapEncodeTiled failed for the tensor-core factorisation");
     }
     static std::atomic<bool> attr{false};
@@ -645,60 +647,89 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
         cudaFuncSetAttribute(tgj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, DIAG_SMEM);
         attr.store(true, std::memory_order_release);
     }
-    cudaMemsetAsync(S, 0, s_bytes, st);
-    cudaMemsetAsync(flag, 0, 2 * sizeof(int), st);
-    const c64* coef = (const c64*)P.coef;
-    const int tl = L / NB;
-    const int sms = std::max(1, ctx->sm_count);
-    const int pgrid = std::min(sms, P.nbox * tl * tl), wgrid = std::min(sms, P.nbox * tl);
+    cudaMemsetAsync(W.S, 0, W.s_bytes, ctx->stream);
+    cudaMemsetAsync(W.flag, 0, 2 * sizeof(int), ctx->stream);
+    return HELM_OK;
+}
+
+void tgj_pad(helm_ctx ctx, const TgjWork& W, const BoxInfo* dbox, int nbox) {
+    tgj_pad_diag<<<dim3(1, nbox), 128, 0, ctx->stream>>>(dbox, (c64*)W.S, W.L);
+    ctx->launches++;
+}
+
+void tgj_eliminate(helm_ctx ctx, const TgjWork& W, const BoxInfo* dbox, const BoxInfo* hbox, int nbox, int m_max, int k) {
+    cudaStream_t st = ctx->stream;
+    const int tl = W.L / NB, sms = std::max(1, ctx->sm_count);
+    const int pgrid = std::min(sms, nbox * tl * tl), wgrid = std::min(sms, nbox * tl);
     // the block inverses (one CTA each) and the copying CTAs beside them: the SMs the blocks leave free, half of them at
     // least
-    const int cgrid = P.nbox + std::max(sms - P.nbox, sms / 2);
+    const int cgrid = nbox + std::max(sms - nbox, sms / 2);
+    // algorithmic bytes of one update launch: every active box reads and writes the rows outside J (below m) of its
+    // matrix once; of one panel: the block, the rows J, the column block J and the operands written
+    for (int j0 = 0; j0 < m_max; j0 += NB) {
+        double ub = 0, pb = 0;
+        for (int i = 0; i < nbox; ++i) {
+            const BoxInfo& b = hbox[i];
+            if (k < b.dims[2] && j0 < b.m) {
+                const double rows = b.m - std::min(NB, b.m - j0);
+                ub += 2.0 * rows * b.m * sizeof(c64);
+                pb += (2.0 * NB * b.m + (double)NB * b.m) * sizeof(c64) + (2.0 * 2 * b.m + b.m) * K2 * sizeof(float);
+            }
+        }
+        int t = prof_begin(ctx, "gj_panel_tc");
+        tgj_panel<<<cgrid, DIAG_THREADS, DIAG_SMEM, st>>>(dbox, (const c64*)W.S, W.L, nbox, (float*)W.Wh, (float*)W.Wl,
+                                                          (float*)W.Ph, (float*)W.Pl, (float*)W.Bh, (float*)W.Bl, W.flag, j0,
+                                                          k);
+        if (tl > 1) {   // W P is empty when the panel is the whole matrix
+            tgj_update_pers<true><<<wgrid, PW * 32, PSMEM, st>>>(W.mWh, W.mWl, W.mPh, W.mPl, W.mS, dbox, nbox, W.L, j0, k,
+                                                                 W.flag + 1);
+            ctx->launches++;
+        }
+        prof_end(ctx, t, pb);
+        t = prof_begin(ctx, "gj_update_tc");
+        tgj_update_pers<false><<<pgrid, PW * 32, PSMEM, st>>>(W.mWh, W.mWl, W.mBh, W.mBl, W.mS, dbox, nbox, W.L, j0, k,
+                                                              W.flag + 1);
+        prof_end(ctx, t, ub);
+        ctx->launches += 2;
+    }
+}
+
+// Tensor-core factorisation of a padded complex64 plane set (the fine sets of TF32 / BF16 factors).
+// *singular: a zero block pivot; *weak: a block pivot below 1e-6 of its block (the caller then factors the
+// set again with full partial pivoting).  Returns HELM_ETIMEOUT if a bounded wait of the update gave up.
+helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* weak) {
+    *singular = *weak = 0;
+    if (P.prec != HELM_PREC_FP32 || !P.padded)
+        return set_error(ctx, HELM_EINVAL, "planeset_factor_tc: needs a padded complex64 set");
+    cudaStream_t st = ctx->stream;
+    TgjWork W;
+    HELM_TRY(tgj_alloc(ctx, P.nbox, P.m_max, W));
+    void* T = nullptr;
+    helm_status rc = dev_alloc(ctx, &T, W.s_bytes, "tensor-core factor work T");
+    auto cleanup = [&]() {
+        dev_free(ctx, T, W.s_bytes);
+        tgj_free(ctx, W);
+    };
+    if (rc) {
+        cleanup();
+        return rc;
+    }
+    const c64* coef = (const c64*)P.coef;
+    c64* S = (c64*)W.S;
     const unsigned eb = (unsigned)std::min<long long>(((long long)P.m_max * P.m_max + 255) / 256, 2048);
     const dim3 egrid(eb, P.nbox);
-    tgj_pad_diag<<<dim3(1, P.nbox), 128, 0, st>>>(P.dbox, (c64*)S, L);
-    ctx->launches++;
-    // algorithmic bytes of one update launch: every active box reads and writes the rows outside J (below m) of
-    // its matrix once; of one panel (block inverse, rows, W): the block, the rows J, the column block J and
-    // the operands written
     for (int k = 0; k < P.bz_max; ++k) {
-        if (k > 0) {
-            // the padding diagonal that the panel's column store may have overwritten in the last plane
-            tgj_pad_diag<<<dim3(1, P.nbox), 128, 0, st>>>(P.dbox, (c64*)S, L);
-            ctx->launches++;
-        }
+        tgj_pad(ctx, W, P.dbox, P.nbox);
         if (k == 0) {
-            tgj_schur_init<<<egrid, 256, 0, st>>>(P.dbox, coef, (c64*)S, L);
+            tgj_schur_init<<<egrid, 256, 0, st>>>(P.dbox, coef, S, W.L);
             ctx->launches++;
         } else {
-            tgj_schur_gu<<<egrid, 256, 0, st>>>(P.dbox, coef, (const c64*)S, (c64*)T, L, k);
-            tgj_schur_lt<<<egrid, 256, 0, st>>>(P.dbox, coef, (const c64*)T, (c64*)S, L, k);
+            tgj_schur_gu<<<egrid, 256, 0, st>>>(P.dbox, coef, S, (c64*)T, W.L, k);
+            tgj_schur_lt<<<egrid, 256, 0, st>>>(P.dbox, coef, (const c64*)T, S, W.L, k);
             ctx->launches += 2;
         }
-        for (int j0 = 0; j0 < P.m_max; j0 += NB) {
-            double ub = 0, pb = 0;
-            for (const auto& b : P.hbox)
-                if (k < b.dims[2] && j0 < b.m) {
-                    const double rows = b.m - std::min(NB, b.m - j0);
-                    ub += 2.0 * rows * b.m * sizeof(c64);
-                    pb += (2.0 * NB * b.m + (double)NB * b.m) * sizeof(c64) + (2.0 * 2 * b.m + b.m) * K2 * sizeof(float);
-                }
-            int t = prof_begin(ctx, "gj_panel_tc");
-            tgj_panel<<<cgrid, DIAG_THREADS, DIAG_SMEM, st>>>(P.dbox, (const c64*)S, L, P.nbox, (float*)Wh, (float*)Wl,
-                                                              (float*)Ph, (float*)Pl, (float*)Bh, (float*)Bl, flag, j0, k);
-            if (tl > 1) {   // W P is empty when the panel is the whole matrix
-                tgj_update_pers<true><<<wgrid, PW * 32, PSMEM, st>>>(mWh, mWl, mPh, mPl, mS, P.dbox, P.nbox, L, j0, k,
-                                                                     flag + 1);
-                ctx->launches++;
-            }
-            prof_end(ctx, t, pb);
-            t = prof_begin(ctx, "gj_update_tc");
-            tgj_update_pers<false><<<pgrid, PW * 32, PSMEM, st>>>(mWh, mWl, mBh, mBl, mS, P.dbox, P.nbox, L, j0, k,
-                                                                  flag + 1);
-            prof_end(ctx, t, ub);
-            ctx->launches += 2;
-        }
-        tgj_store<<<egrid, 256, 0, st>>>(P.dbox, (const c64*)S, L, (c64*)P.G, k);
+        tgj_eliminate(ctx, W, P.dbox, P.hbox.data(), P.nbox, P.m_max, k);
+        tgj_store<<<egrid, 256, 0, st>>>(P.dbox, S, W.L, (c64*)P.G, k);
         ctx->launches++;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
@@ -707,7 +738,7 @@ helm_status planeset_factor_tc(helm_ctx ctx, PlaneSet& P, int* singular, int* we
         }
     }
     int hflag[2] = {0, 0};
-    cudaMemcpyAsync(hflag, flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaMemcpyAsync(hflag, W.flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
     rc = cuda_check(ctx, cudaStreamSynchronize(st), "tensor-core plane factorisation");
     cleanup();
     if (rc) return rc;
