@@ -195,17 +195,19 @@ __device__ __forceinline__ void prep_tile(const BoxInfo& B, int box, int t, int 
 // prep_tile for the persistent sweep.  One round of asynchronous copies (all in flight at once) brings into
 // shared memory the tile's neighbour rows (a contiguous stretch of the neighbour plane, read from L2),
 // its 9 coupling coefficients per node and, forward, its right-hand sides; every value is then formed
-// from shared memory with the same operations in the same order as prep_tile, by a thread per
-// (node, column pair) with the node fastest, and written straight into its four B^T rows (coalesced
-// along the node).  Node rows are padded to one float4 more than a chunk against bank conflicts.  When
-// all column pairs do not fit in smem_bytes, they are staged and formed in chunks (the largest halving
-// of the pair count that fits; the coefficients are staged once).  Plane 0 of the forward sweep (no
+// from shared memory with the same operations in the same order as prep_tile: a thread owns one node (its nine
+// coefficients and neighbour offsets stay in registers) and every NT / 128-th column pair, and writes straight into the
+// four B^T rows (coalesced along the node).  Node rows are padded to one float4 more than a chunk against bank
+// conflicts.  When all column pairs do not fit in smem_bytes, they are staged and formed in chunks (the largest
+// halving of the pair count that fits; the coefficients are staged once).  Plane 0 of the forward sweep (no
 // coupling) and tiles whose data exceed smem_bytes even for one pair use prep_tile.
-template <typename E>
+// Issue-bound: with 128 threads per SM and a thread per (node, pair) an item of 128 columns took 57,000 clocks.
+template <typename E, int NT>
 __device__ __forceinline__ void prep_tile_staged(const BoxInfo& B, int box, int t, int tpn,
                                                  const c64* __restrict__ coef, const c64* __restrict__ lb,
                                                  const c64* __restrict__ loc, E* __restrict__ bt, int ld2, int npad,
                                                  int nrhs, int s, int fwd, unsigned char* smem, int smem_bytes) {
+    static_assert(NT % 128 == 0, "a thread per node of a tile of at most 128");
     const int m = B.m, bz = B.dims[2], bx = B.dims[0], by = B.dims[1];
     const int k = fwd ? s : bz - 1 - s;
     if (k < 0 || k >= bz || (!fwd && k == bz - 1)) return;
@@ -237,43 +239,55 @@ __device__ __forceinline__ void prep_tile_staged(const BoxInfo& B, int box, int 
     const float2* csrc = reinterpret_cast<const float2*>(coef + (plane + p0) * 27 + off);
     E* bb = bt + (size_t)box * npad * ld2;
     typedef typename Pair2<E>::type P2;
+    const int tid = threadIdx.x, pl = tid & 127, p = p0 + pl;
+    int nb[9];
+    float2 c[9];
+    {
+        const int px = p % bx, py = p / bx;
+#pragma unroll
+        for (int d = 0; d < 9; ++d) {
+            const int qx = min(max(px + d % 3 - 1, 0), bx - 1), qy = min(max(py + d / 3 - 1, 0), by - 1);
+            nb[d] = ((qy - r_lo) * bx + qx) * sp;
+        }
+    }
     for (int c0 = 0; c0 < npair; c0 += cp) {
         const int cw = min(cp, npair - c0);
-        const int n1 = ns * cw, n2 = nl * cw, n3 = c0 == 0 ? np * 9 : 0;
+        // copies: thread (row, column) of a NT / cw x cw grid
+        const int rows = NT / cw, tr = tid / cw, tc_ = tid % cw;
         if (c0 > 0) __syncthreads();   // the previous chunk's values are read before they are replaced
-        for (int e = threadIdx.x; e < n1; e += blockDim.x)
-            tc::cp_async16(stg + (e / cw) * sp + e % cw, nsrc + (long long)(e / cw) * npair + c0 + e % cw);
-        for (int e = threadIdx.x; e < n2; e += blockDim.x)
-            tc::cp_async16(lbs + (e / cw) * sp + e % cw, lsrc + (long long)(e / cw) * npair + c0 + e % cw);
-        for (int e = threadIdx.x; e < n3; e += blockDim.x) tc::cp_async8(cfs + e, csrc + (e / 9) * 27 + e % 9);
+        if (tr < rows) {
+            for (int r = tr; r < ns; r += rows) tc::cp_async16(stg + r * sp + tc_, nsrc + (long long)r * npair + c0 + tc_);
+            for (int r = tr; r < nl; r += rows) tc::cp_async16(lbs + r * sp + tc_, lsrc + (long long)r * npair + c0 + tc_);
+        }
+        if (c0 == 0)
+            for (int e = tid; e < np * 9; e += NT) tc::cp_async8(cfs + e, csrc + (e / 9) * 27 + e % 9);
         tc::cp_async_wait_all();
         __syncthreads();
-        for (int e = threadIdx.x; e < np * cw; e += blockDim.x) {
-            const int pl = e % np, pc = e / np, pr = c0 + pc, p = p0 + pl;
-            float4 acc = fwd ? lbs[pl * sp + pc] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const int px = p % bx, py = p / bx;
-            float2 c[9];
-            float4 v[9];
+        if (pl < np) {
+            if (c0 == 0) {
 #pragma unroll
-            for (int d = 0; d < 9; ++d) {
-                const int qx = min(max(px + d % 3 - 1, 0), bx - 1), qy = min(max(py + d / 3 - 1, 0), by - 1);
-                c[d] = cfs[pl * 9 + d];
-                v[d] = stg[((qy - r_lo) * bx + qx) * sp + pc];
+                for (int d = 0; d < 9; ++d) {
+                    c[d] = cfs[pl * 9 + d];
+                    if (fwd) c[d] = make_float2(-c[d].x, -c[d].y);   // forward: acc -= c v; backward: acc += c v
+                }
             }
+            for (int pc = tid >> 7; pc < cw; pc += NT / 128) {
+                float4 acc = fwd ? lbs[pl * sp + pc] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int d = 0; d < 9; ++d) {
-                const float sr = fwd ? -c[d].x : c[d].x, si = fwd ? -c[d].y : c[d].y;
-                acc.x = fmaf(sr, v[d].x, fmaf(-si, v[d].y, acc.x));
-                acc.y = fmaf(sr, v[d].y, fmaf(si, v[d].x, acc.y));
-                acc.z = fmaf(sr, v[d].z, fmaf(-si, v[d].w, acc.z));
-                acc.w = fmaf(sr, v[d].w, fmaf(si, v[d].z, acc.w));
+                for (int d = 0; d < 9; ++d) {
+                    const float4 v = stg[nb[d] + pc];
+                    acc.x = fmaf(c[d].x, v.x, fmaf(-c[d].y, v.y, acc.x));
+                    acc.y = fmaf(c[d].x, v.y, fmaf(c[d].y, v.x, acc.y));
+                    acc.z = fmaf(c[d].x, v.z, fmaf(-c[d].y, v.w, acc.z));
+                    acc.w = fmaf(c[d].x, v.w, fmaf(c[d].y, v.z, acc.w));
+                }
+                // columns 2 pr (acc.x, acc.y) and 2 pr + 1 (acc.z, acc.w): B^T rows 4 pr .. 4 pr + 3 at entries 2p, 2p + 1
+                E* row = bb + (size_t)(4 * (c0 + pc)) * ld2 + 2 * p;
+                *reinterpret_cast<P2*>(row) = Pair2<E>::make(acc.x, -acc.y);
+                *reinterpret_cast<P2*>(row + ld2) = Pair2<E>::make(acc.y, acc.x);
+                *reinterpret_cast<P2*>(row + 2 * (size_t)ld2) = Pair2<E>::make(acc.z, -acc.w);
+                *reinterpret_cast<P2*>(row + 3 * (size_t)ld2) = Pair2<E>::make(acc.w, acc.z);
             }
-            // columns 2 pr (acc.x, acc.y) and 2 pr + 1 (acc.z, acc.w): B^T rows 4 pr .. 4 pr + 3 at entries 2p, 2p + 1
-            E* row = bb + (size_t)(4 * pr) * ld2 + 2 * p;
-            *reinterpret_cast<P2*>(row) = Pair2<E>::make(acc.x, -acc.y);
-            *reinterpret_cast<P2*>(row + ld2) = Pair2<E>::make(acc.y, acc.x);
-            *reinterpret_cast<P2*>(row + 2 * (size_t)ld2) = Pair2<E>::make(acc.z, -acc.w);
-            *reinterpret_cast<P2*>(row + 3 * (size_t)ld2) = Pair2<E>::make(acc.w, acc.z);
         }
     }
 }
@@ -295,6 +309,9 @@ struct TcCfg {
     static constexpr int B_BYTES = NPAD * 128;
     static constexpr int STAGE = A_BYTES + B_BYTES;
     static constexpr int STAGES = NST;
+    // threads: warps 0-3 load, multiply and read the accumulator; all of them prepare operands and move results.  One CTA
+    // per SM at N = 256, two or three below it
+    static constexpr int THREADS = NPAD >= 256 ? 512 : 256;
     static constexpr uint32_t TCOLS = NPAD <= 32 ? 32 : (NPAD <= 64 ? 64 : (NPAD <= 128 ? 128 : 256));
     static constexpr int SMEM = STAGES * STAGE + (2 * STAGES + 1) * 8 + 16 + 1024;
 };
@@ -348,8 +365,9 @@ __device__ __forceinline__ void gemm_teardown(uint32_t tmem) {
 }
 
 // Row tile t of box (index box) at plane k: y_k rows (forward) or x_k = y_k - G_k R rows (backward).
-// base: 1024-aligned dynamic shared memory (NST stages, then the barriers).  All 128 threads call it;
-// it ends with a CTA barrier after the accumulator has been read, so the next tile may reuse TMEM and
+// base: 1024-aligned dynamic shared memory (NST stages, then the barriers).  All threads of the CTA call it (warps
+// past the fourth only move results; warp w reads the accumulator's lanes 32 (w mod 4).. of every NT / 128-th piece of
+// 32 columns); it ends with a CTA barrier after the accumulator has been read, so the next tile may reuse TMEM and
 // the stages.  A wait that gives up leaves an error code in *err.
 template <typename E, int NPAD, int NST>
 __device__ __forceinline__ void gemm_core(const CUtensorMap* mapA, const CUtensorMap* mapA32, const CUtensorMap* mapB,
@@ -357,7 +375,7 @@ __device__ __forceinline__ void gemm_core(const CUtensorMap* mapA, const CUtenso
                                           int fwd, int nkc, int* __restrict__ err, unsigned char* base, uint32_t tmem,
                                           Ring& R) {
     using Cfg = TcCfg<E, NPAD, NST>;
-    constexpr int TC_BK = Cfg::BK;
+    constexpr int TC_BK = Cfg::BK, NT = Cfg::THREADS;
     uint64_t* full = reinterpret_cast<uint64_t*>(base + NST * Cfg::STAGE);
     uint64_t* empty = full + NST;
     uint64_t* done = empty + NST;
@@ -431,7 +449,58 @@ __device__ __forceinline__ void gemm_core(const CUtensorMap* mapA, const CUtenso
             const uint32_t gi = R.g + kc;
             tc::mbar_drain(&full[gi % NST], (gi / NST) & 1);
         }
-    if (ok) {
+    if ((nrhs & 1) == 0) {
+        // The tile's output is one contiguous block of loc (rows row0.., all columns).  The accumulator passes through the
+        // stages' shared memory (every load of this tile has been consumed) as column pairs, the pair index XORed with
+        // the row so that the 8 rows of a store phase fall in different banks; the block is then read and written in
+        // 16-byte vectors along memory, four in flight per thread.  (Rows straight from TMEM took an 8-byte access per
+        // column and 32 lines per warp access: at 128 columns more than half of a tile's time.)
+        const int npair = nrhs >> 1, np8 = (npair + 7) & ~7;
+        float4* ep = reinterpret_cast<float4*>(base);
+        if (ok) {
+            const int wq = warp & 3, r = wq * 32 + lane;
+#pragma unroll
+            for (int c0 = 0; c0 < NPAD; c0 += 32) {
+                if (c0 >= 2 * nrhs) break;
+                if ((c0 / 32) % (Cfg::THREADS / 128) != warp / 4) continue;
+                constexpr int W = NPAD < 32 ? NPAD : 32;
+                uint32_t v[32];
+                tc::tmem_ld_32x32b_x32(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)c0, v);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int q = 0; q < W / 4; ++q) {
+                    const int pr = c0 / 4 + q;
+                    if (pr < npair)
+                        ep[r * np8 + ((pr & ~7) | ((pr ^ r) & 7))] =
+                            make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]),
+                                        __uint_as_float(v[4 * q + 3]));
+                }
+            }
+        }
+        __syncthreads();
+        if (ok) {
+            float4* dst = reinterpret_cast<float4*>(loc + (B.loc_off + (long long)k * m + row0) * nrhs);
+            const int total = min(TC_BM, m - row0) * npair;
+            for (int e0 = threadIdx.x; e0 < total; e0 += 4 * NT) {
+                float4 o[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int e = e0 + u * NT;
+                    // y_k may come from another CTA of a persistent launch: read it from L2
+                    o[u] = !fwd && e < total ? __ldcg(dst + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int e = e0 + u * NT;
+                    if (e >= total) break;
+                    const int r = e / npair, pr = e % npair;
+                    const float4 d = ep[r * np8 + ((pr & ~7) | ((pr ^ r) & 7))];
+                    dst[e] = fwd ? d : make_float4(o[u].x - d.x, o[u].y - d.y, o[u].z - d.z, o[u].w - d.w);
+                }
+            }
+        }
+        tc::fence_proxy_async_smem();   // the stages are TMA destinations again
+    } else if (ok && warp < 4) {
         const int row = row0 + warp * 32 + lane;
         c64* dst = loc + (B.loc_off + (long long)k * m + row) * nrhs;
 #pragma unroll
@@ -448,7 +517,6 @@ __device__ __forceinline__ void gemm_core(const CUtensorMap* mapA, const CUtenso
                         if (fwd) {
                             dst[r] = mk<float>(re, im);
                         } else {
-                            // y_k may come from another CTA of a persistent launch: read it from L2
                             const float2 o = __ldcg(reinterpret_cast<const float2*>(dst + r));
                             dst[r] = mk<float>(o.x - re, o.y - im);
                         }
@@ -469,7 +537,7 @@ __device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
 }
 
 template <typename E, int NPAD, int NST>
-__global__ void __launch_bounds__(128, 1) tc_sweep_gemm(const __grid_constant__ CUtensorMap mapA,
+__global__ void __launch_bounds__(TcCfg<E, NPAD, NST>::THREADS, 1) tc_sweep_gemm(const __grid_constant__ CUtensorMap mapA,
                                                         const __grid_constant__ CUtensorMap mapA32,
                                                         const __grid_constant__ CUtensorMap mapB,
                                                         const BoxInfo* __restrict__ boxes, c64* __restrict__ loc,
@@ -570,7 +638,7 @@ __device__ __host__ __forceinline__ int flow_tiles(int m, int j, int tpn) {
 }
 
 template <typename E, int NPAD, int NST>
-__global__ void __launch_bounds__(128, 1) tc_sweep_flow(const __grid_constant__ CUtensorMap mapA,
+__global__ void __launch_bounds__(TcCfg<E, NPAD, NST>::THREADS, TcCfg<E, NPAD, NST>::THREADS == 512 ? 1 : 2) tc_sweep_flow(const __grid_constant__ CUtensorMap mapA,
                                                         const __grid_constant__ CUtensorMap mapA32,
                                                         const __grid_constant__ CUtensorMap mapB,
                                                         const BoxInfo* __restrict__ boxes, const c64* __restrict__ coef,
@@ -612,7 +680,7 @@ __global__ void __launch_bounds__(128, 1) tc_sweep_flow(const __grid_constant__ 
             const int k = fwd ? s : bz - 1 - s;
             gemm_core<E, NPAD, NST>(&mapA, &mapA32, &mapB, B, box, t, k, loc, nrhs, fwd, nkc, err, base, tmem, R);
         } else {
-            prep_tile_staged<E>(B, box, t, tpn, coef, lb, loc, bt, ld2, NPAD, nrhs, s, fwd, base,
+            prep_tile_staged<E, TcCfg<E, NPAD, NST>::THREADS>(B, box, t, tpn, coef, lb, loc, bt, ld2, NPAD, nrhs, s, fwd, base,
                                 NST * TcCfg<E, NPAD, NST>::STAGE);
             tc::fence_proxy_async_smem();   // the stages are TMA destinations again in a later product
             fence_proxy_async_global();     // B operand written here, read by TMA in another CTA
@@ -700,7 +768,7 @@ helm_status run_tc(helm_ctx ctx, const PlaneSet& P, const c64* lb, c64* loc, E* 
             cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) == cudaSuccess &&
             cudaFuncGetAttributes(&fa, tc_sweep_flow<E, NPAD, NST>) == cudaSuccess) {
             const int per_block = Cfg::SMEM + (int)fa.sharedSizeBytes + 1024;   // + the 1 KB reserved per block
-            const int regs = (fa.numRegs + 7) / 8 * 8 * 128;
+            const int regs = (fa.numRegs + 7) / 8 * 8 * Cfg::THREADS;
             flow_occ.store(std::min(std::min(smem_sm / per_block, regs_sm / std::max(1, regs)),
                                     std::min(512 / (int)Cfg::TCOLS, 8)));
         }
@@ -742,7 +810,7 @@ helm_status run_tc(helm_ctx ctx, const PlaneSet& P, const c64* lb, c64* loc, E* 
         const int grid = std::max(1, std::min(flow->total, flow_occ * std::max(1, ctx->sm_count)));
         HELM_CUDA(ctx, cudaMemsetAsync(flow->mem, 0, flow->reset_bytes, st));
         const int t = prof_begin(ctx, "sweep_flow");
-        tc_sweep_flow<E, NPAD, NST><<<grid, 128, Cfg::SMEM, st>>>(mapA, mapA32, mapB, P.dbox, coef, lb, loc, bt, 2 * ld,
+        tc_sweep_flow<E, NPAD, NST><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(mapA, mapA32, mapB, P.dbox, coef, lb, loc, bt, 2 * ld,
                                                                    nrhs, P.pk_chunks, flow->init, flow->ninit,
                                                                    flow->flag, flow->total, flow->ctl, err,
                                                                    (uint64_t)ctx->flow_wait_us * 1000ull, flow->tpn);
@@ -761,7 +829,7 @@ helm_status run_tc(helm_ctx ctx, const PlaneSet& P, const c64* lb, c64* loc, E* 
                 tc_prep<E><<<pgrid, 256, 0, st>>>(P.dbox, coef, lb, loc, bt, 2 * ld, NPAD, nrhs, s, fwd);
             prof_end(ctx, t, pb);
             t = prof_begin(ctx, "sweep_gemm_tc");
-            tc_sweep_gemm<E, NPAD, NST><<<ggrid, 128, Cfg::SMEM, st>>>(mapA, mapA32, mapB, P.dbox, loc, nrhs, s,
+            tc_sweep_gemm<E, NPAD, NST><<<ggrid, Cfg::THREADS, Cfg::SMEM, st>>>(mapA, mapA32, mapB, P.dbox, loc, nrhs, s,
                                                                         fwd, P.pk_chunks, err);
             prof_end(ctx, t, gb);
             ctx->launches += 2;
