@@ -150,6 +150,42 @@ __global__ void e27_apply(const cplx<T>* __restrict__ E27, const cplx<T>* __rest
 
 // ------------------------------------------------------------------ restriction / prolongation
 
+// R_i v for every box and the owner gather for complex64 vectors with an even column count: the same index arithmetic as the
+// two kernels below on 16-byte column pairs.  grid: (x-line chunks, box rows (y, z) strided, box) and (x-line chunks, y, z).
+__global__ void __launch_bounds__(256) restrict_boxes_pairs(const BoxInfo* __restrict__ boxes, const float4* __restrict__ v,
+                                                            float4* __restrict__ loc, int nx, int ny, int npair) {
+    const BoxInfo& B = boxes[blockIdx.z];
+    const int bx = B.dims[0], by = B.dims[1], line = bx * npair;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= line) return;
+    const int rows = by * B.dims[2];
+    const float4* src = v + (long long)B.lo[0] * npair + t;
+    float4* dst = loc + B.loc_off * npair + t;
+    for (int row = blockIdx.y; row < rows; row += gridDim.y) {
+        const int lj = row % by, lk = row / by;
+        dst[(long long)row * line] = src[((long long)(B.lo[2] + lk) * ny + (B.lo[1] + lj)) * nx * npair];
+    }
+}
+template <bool ADDQ>
+__global__ void __launch_bounds__(256) prolong_owner_pairs(const BoxInfo* __restrict__ boxes, const int* __restrict__ owner,
+                                                           const float4* __restrict__ loc, const float4* __restrict__ q,
+                                                           float4* __restrict__ out, int nx, int ny, int nz, int px, int py,
+                                                           int npair) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nx * npair) return;
+    const int i = t / npair, pr = t % npair;
+    const int j = blockIdx.y, k = blockIdx.z;
+    const long long e = ((long long)k * ny + j) * nx * npair + t;
+    const BoxInfo& B = boxes[(owner[nx + ny + k] * py + owner[nx + j]) * px + owner[i]];
+    const long long l = ((long long)(k - B.lo[2]) * B.dims[1] + (j - B.lo[1])) * B.dims[0] + (i - B.lo[0]);
+    float4 y = loc[(B.loc_off + l) * npair + pr];
+    if (ADDQ) {
+        const float4 a = q[e];
+        y = make_float4(y.x + a.x, y.y + a.y, y.z + a.z, y.w + a.w);
+    }
+    out[e] = y;
+}
+
 // loc[(loc_off + l) * nrhs + r] = v[g(l) * nrhs + r]   (R_i v for every box)
 template <typename TV, typename TL>
 __global__ void restrict_boxes(const BoxInfo* __restrict__ boxes, const cplx<TV>* __restrict__ v,
@@ -267,11 +303,43 @@ __global__ void restrict_axis(const cplx<TI>* __restrict__ in, cplx<TO>* __restr
     }
 }
 
+// restrict_axis on 16-byte column pairs (complex64, an even column count); grid: (x-line chunks, y, z) of the output.
+template <int AX>
+__global__ void __launch_bounds__(256) restrict_axis_pairs(const float4* __restrict__ in, float4* __restrict__ out, int n0,
+                                                           int n1, int n2, int nc, int r, int npair, float scale) {
+    const int d0 = AX == 0 ? nc : n0, d1 = gridDim.y;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= d0 * npair) return;
+    const int o0 = t / npair, pr = t % npair, o1 = blockIdx.y, o2 = blockIdx.z;
+    const int n = AX == 0 ? n0 : (AX == 1 ? n1 : n2), J = AX == 0 ? o0 : (AX == 1 ? o1 : o2);
+    const long long sa = (AX == 0 ? 1LL : (AX == 1 ? (long long)n0 : (long long)n0 * n1)) * npair;
+    const float4* base = in + (((long long)(AX == 2 ? 0 : o2) * n1 + (AX == 1 ? 0 : o1)) * n0 + (AX == 0 ? 0 : o0)) * npair + pr;
+    const int i0 = max(0, r * J - r + 1), i1 = min(n - 1, r * J + r - 1);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = i0; i <= i1; ++i) {
+        const float wt = (float)(r - abs(i - r * J));
+        const float4 x = base[(long long)i * sa];
+        acc.x += wt * x.x;
+        acc.y += wt * x.y;
+        acc.z += wt * x.z;
+        acc.w += wt * x.w;
+    }
+    out[(((long long)o2 * d1 + o1) * d0) * npair + t] = make_float4(acc.x * scale, acc.y * scale, acc.z * scale, acc.w * scale);
+}
+
 // cv = Z^T v / r^3 by three axis passes (x into t1, y into t2, z into cv)
 template <typename TV, typename TC>
 void restrict_separable(const cplx<TV>* v, cplx<TV>* t1, cplx<TV>* t2, cplx<TC>* cv, int nx, int ny, int nz, int cx,
                         int cy, int cz, int r, int R, cudaStream_t st) {
     const TV one = (TV)1, s3 = (TV)1 / (TV)(r * r * r);
+    if (sizeof(TV) == 4 && sizeof(TC) == 4 && R % 2 == 0 && (((uintptr_t)v | (uintptr_t)t1 | (uintptr_t)t2 | (uintptr_t)cv) & 15) == 0) {
+        const int np = R / 2;
+        auto grid = [&](int d0, int d1, int d2) { return dim3((unsigned)((d0 * np + 255) / 256), (unsigned)d1, (unsigned)d2); };
+        restrict_axis_pairs<0><<<grid(cx, ny, nz), 256, 0, st>>>((const float4*)v, (float4*)t1, nx, ny, nz, cx, r, np, 1.0f);
+        restrict_axis_pairs<1><<<grid(cx, cy, nz), 256, 0, st>>>((const float4*)t1, (float4*)t2, cx, ny, nz, cy, r, np, 1.0f);
+        restrict_axis_pairs<2><<<grid(cx, cy, cz), 256, 0, st>>>((const float4*)t2, (float4*)cv, cx, cy, nz, cz, r, np, (float)s3);
+        return;
+    }
     restrict_axis<TV, TV><<<grid_for((long long)nz * ny * cx * R), 256, 0, st>>>(v, t1, nx, ny, nz, 0, cx, r, R, one);
     restrict_axis<TV, TV><<<grid_for((long long)nz * cy * cx * R), 256, 0, st>>>(t1, t2, cx, ny, nz, 1, cy, r, R, one);
     restrict_axis<TV, TC><<<grid_for((long long)cz * cy * cx * R), 256, 0, st>>>(t2, cv, cx, cy, nz, 2, cz, r, R, s3);
@@ -305,42 +373,52 @@ __global__ void coarse_prolong(const cplx<TC>* __restrict__ cv, cplx<TV>* __rest
     q[e] = acc;
 }
 
-// The same for complex64 with an even column count: a thread per fine node forms the 8 trilinear weights
-// and corner indices once and sweeps the columns in 16-byte pairs (the per-column kernel repeats that
-// integer work for every column).  grid: (x-line chunks of 128 nodes, y, z).
-__global__ void coarse_prolong_pairs(const c64* __restrict__ cv, c64* __restrict__ q, int nx, int ny, int nz, int cx,
-                                     int cy, int cz, int r, int nrhs) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nx) return;
+// The same for complex64 with an even column count: a thread per (fine node, column pair), the pair fastest, so that a
+// warp's loads and stores are contiguous 16-byte vectors; the x-line is flattened over (node, pair) and the 8 weights are
+// formed per thread (a few integer operations against nine vector accesses).  grid: (x-line chunks, y, z).  Bound by L2:
+// the write and the 8 corner reads, which r^3 fine nodes share.  A thread per node walking its pairs kept one access per
+// lane and line: 331 us at 128 x 128 x 64 x 32 (per-column kernel) and 132 us at 112^3 x 16 (thread per node).
+__global__ void __launch_bounds__(256) coarse_prolong_pairs(const c64* __restrict__ cv, c64* __restrict__ q, int nx, int ny,
+                                                            int nz, int cx, int cy, int cz, int r, int npair) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nx * npair) return;
+    const int i = t / npair, pr = t % npair;
     const int j = blockIdx.y, k = blockIdx.z;
     const float inv_r = 1.0f / (float)r;
     const int I0 = i / r, J0 = j / r, K0 = k / r;
     const float wx1 = (float)(i - r * I0) * inv_r, wy1 = (float)(j - r * J0) * inv_r, wz1 = (float)(k - r * K0) * inv_r;
     const float wx[2] = {1.0f - wx1, wx1}, wy[2] = {1.0f - wy1, wy1}, wz[2] = {1.0f - wz1, wz1};
+    const float4* base = reinterpret_cast<const float4*>(cv) + (((long long)K0 * cy + J0) * cx + I0) * npair + pr;
     float wt[8];
-    long long base[8];
+    float4 x[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const int a = c & 1, b = (c >> 1) & 1, d = c >> 2;
+        // a corner past the coarse grid has weight 0: read the base corner
         const bool in = I0 + a < cx && J0 + b < cy && K0 + d < cz;
         wt[c] = in ? wx[a] * wy[b] * wz[d] : 0.0f;
-        // a corner past the coarse grid has weight 0: point it at the base corner
-        base[c] = in ? (((long long)(K0 + d) * cy + (J0 + b)) * cx + (I0 + a)) * nrhs
-                     : (((long long)K0 * cy + J0) * cx + I0) * nrhs;
+        x[c] = base[in ? (((long long)d * cy + b) * cx + a) * npair : 0];
     }
-    float4* out = reinterpret_cast<float4*>(q + (((long long)k * ny + j) * nx + i) * nrhs);
-    for (int p = 0; p < nrhs / 2; ++p) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float4 x = *reinterpret_cast<const float4*>(cv + base[c] + 2 * p);
-            acc.x += wt[c] * x.x;
-            acc.y += wt[c] * x.y;
-            acc.z += wt[c] * x.z;
-            acc.w += wt[c] * x.w;
-        }
-        out[p] = acc;
+    for (int c = 0; c < 8; ++c) {
+        acc.x += wt[c] * x[c].x;
+        acc.y += wt[c] * x[c].y;
+        acc.z += wt[c] * x[c].z;
+        acc.w += wt[c] * x[c].w;
     }
+    reinterpret_cast<float4*>(q)[((long long)k * ny + j) * nx * npair + t] = acc;
+}
+
+template <typename TC, typename TV>
+void launch_prolong(const cplx<TC>* cv, cplx<TV>* q, int nx, int ny, int nz, int cx, int cy, int cz, int r, int nrhs,
+                    cudaStream_t st) {
+    if (sizeof(TC) == 4 && sizeof(TV) == 4 && nrhs % 2 == 0 && (((uintptr_t)cv | (uintptr_t)q) & 15) == 0)
+        coarse_prolong_pairs<<<dim3((unsigned)((nx * (nrhs / 2) + 255) / 256), (unsigned)ny, (unsigned)nz), 256, 0, st>>>(
+            (const c64*)cv, (c64*)q, nx, ny, nz, cx, cy, cz, r, nrhs / 2);
+    else
+        coarse_prolong<TC, TV><<<dim3((unsigned)((nx * nrhs + 255) / 256), (unsigned)ny, (unsigned)nz), 256, 0, st>>>(
+            cv, q, nx, ny, nz, cx, cy, cz, r, nrhs);
 }
 
 // Probe vectors: zc[i * 27 + c] = (Z e_c)_i, e_c = indicator of the coarse nodes of colour c = (J mod 3).
@@ -748,27 +826,19 @@ helm_status apply_t(helm_oras o, const cplx<TV>* v, cplx<TV>* out, int nrhs) {
             prof_end(ctx, tk, vb);
             HELM_TRY(inner_solve(o, wp, o->cvec, o->cy, nrhs));
             tk = prof_begin(ctx, "coarse_prolong");
-            coarse_prolong<TV, TV><<<dim3((unsigned)((nx * nrhs + 255) / 256), (unsigned)ny, (unsigned)nz), 256, 0,
-                                     st>>>((const cplx<TV>*)o->cy, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs);
+            launch_prolong<TV, TV>((const cplx<TV>*)o->cy, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs, st);
         } else if (o->coarse32.G) {
             restrict_separable<TV, float>(v, t1, t2, (c64*)o->cvec, nx, ny, nz, cx, cy, cz, r, nrhs, st);
             prof_end(ctx, tk, vb);
             HELM_TRY(planeset_solve(ctx, o->coarse32, o->cvec, o->crbuf, nrhs, st, o->dev_err));
             tk = prof_begin(ctx, "coarse_prolong");
-            if (sizeof(TV) == 4 && nrhs % 2 == 0 && (((uintptr_t)o->cvec | (uintptr_t)o->qf) & 15) == 0)
-                coarse_prolong_pairs<<<dim3((unsigned)((nx + 127) / 128), (unsigned)ny, (unsigned)nz), 128, 0, st>>>(
-                    (const c64*)o->cvec, (c64*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs);
-            else
-                coarse_prolong<float, TV><<<dim3((unsigned)((nx * nrhs + 255) / 256), (unsigned)ny, (unsigned)nz), 256,
-                                            0, st>>>((const c64*)o->cvec, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r,
-                                                     nrhs);
+            launch_prolong<float, TV>((const c64*)o->cvec, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs, st);
         } else {
             restrict_separable<TV, double>(v, t1, t2, o->cvec, nx, ny, nz, cx, cy, cz, r, nrhs, st);
             prof_end(ctx, tk, vb);
             HELM_TRY(planeset_solve(ctx, o->coarse, o->cvec, o->crbuf, nrhs, st));
             tk = prof_begin(ctx, "coarse_prolong");
-            coarse_prolong<double, TV><<<dim3((unsigned)((nx * nrhs + 255) / 256), (unsigned)ny, (unsigned)nz), 256, 0,
-                                         st>>>(o->cvec, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs);
+            launch_prolong<double, TV>(o->cvec, (cplx<TV>*)o->qf, nx, ny, nz, cx, cy, cz, r, nrhs, st);
         }
         prof_end(ctx, tk, vb);
         ctx->launches += 4;
@@ -787,8 +857,15 @@ helm_status apply_t(helm_oras o, const cplx<TV>* v, cplx<TV>* out, int nrhs) {
         bxm = std::max(bxm, b.dims[0]);
         rows = std::max(rows, b.dims[1] * b.dims[2]);
     }
-    restrict_boxes<TV, TL><<<dim3((unsigned)((bxm * nrhs + 255) / 256), (unsigned)std::min(rows, 65535), o->fine.nbox),
-                             256, 0, st>>>(o->fine.dbox, src, rdst, nx, ny, nrhs);
+    const bool pairs = sizeof(TV) == 4 && sizeof(TL) == 4 && nrhs % 2 == 0 &&
+                       (((uintptr_t)src | (uintptr_t)rdst | (uintptr_t)o->loc | (uintptr_t)q | (uintptr_t)out) & 15) == 0;
+    const int npair = nrhs / 2;
+    if (pairs)
+        restrict_boxes_pairs<<<dim3((unsigned)((bxm * npair + 255) / 256), (unsigned)std::min(rows, 65535), o->fine.nbox), 256, 0,
+                               st>>>(o->fine.dbox, (const float4*)src, (float4*)rdst, nx, ny, npair);
+    else
+        restrict_boxes<TV, TL><<<dim3((unsigned)((bxm * nrhs + 255) / 256), (unsigned)std::min(rows, 65535), o->fine.nbox),
+                                 256, 0, st>>>(o->fine.dbox, src, rdst, nx, ny, nrhs);
     prof_end(ctx, tr, lb);
     ctx->launches++;
     if (o->fine.padded)
@@ -797,7 +874,14 @@ helm_status apply_t(helm_oras o, const cplx<TV>* v, cplx<TV>* out, int nrhs) {
         HELM_TRY(planeset_solve(ctx, o->fine, o->loc, o->rbuf, nrhs, st));
     tr = prof_begin(ctx, "oras_transfer");
     const dim3 lgrid((unsigned)((nx * nrhs + 255) / 256), (unsigned)ny, (unsigned)nz);   // (x-line chunks, y, z)
-    if (q)
+    const dim3 pgrid((unsigned)((nx * npair + 255) / 256), (unsigned)ny, (unsigned)nz);
+    if (pairs && q)
+        prolong_owner_pairs<true><<<pgrid, 256, 0, st>>>(o->fine.dbox, o->owner, (const float4*)o->loc, (const float4*)q,
+                                                         (float4*)out, nx, ny, nz, o->d.px, o->d.py, npair);
+    else if (pairs)
+        prolong_owner_pairs<false><<<pgrid, 256, 0, st>>>(o->fine.dbox, o->owner, (const float4*)o->loc, nullptr,
+                                                          (float4*)out, nx, ny, nz, o->d.px, o->d.py, npair);
+    else if (q)
         prolong_owner<TL, TV, true><<<lgrid, 256, 0, st>>>(o->fine.dbox, o->owner, (const cplx<TL>*)o->loc, q, out,
                                                            nx, ny, nz, o->d.px, o->d.py, nrhs);
     else
