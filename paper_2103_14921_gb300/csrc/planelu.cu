@@ -478,6 +478,33 @@ __global__ void sweep_prep(const BoxInfo* __restrict__ boxes, const cplx<T>* __r
     }
 }
 
+// Sum over the warp of RN values per lane (RN a power of two), value r in lane r: every step halves either the values a
+// lane holds or, once one is left, the lanes, so RN = 4 costs 9 complex additions where a full exchange per value costs 20
+// (they run on the pipe the products need in complex128).
+template <typename T, int RN>
+__device__ __forceinline__ cplx<T> warp_sum_columns(cplx<T> (&a)[RN], int lane) {
+#pragma unroll
+    for (int h = RN / 2; h > 0; h >>= 1) {
+        const bool up = (lane & h) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const cplx<T> give = up ? a[i] : a[i + h], keep = up ? a[i + h] : a[i];
+            cplx<T> got;
+            got.x = __shfl_xor_sync(0xffffffffu, give.x, h);
+            got.y = __shfl_xor_sync(0xffffffffu, give.y, h);
+            a[i] = keep + got;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o >= RN; o >>= 1) {
+        cplx<T> got;
+        got.x = __shfl_xor_sync(0xffffffffu, a[0].x, o);
+        got.y = __shfl_xor_sync(0xffffffffu, a[0].y, o);
+        a[0] = a[0] + got;
+    }
+    return a[0];
+}
+
 // loc[plane k][row][r0 + r] = (FWD ? 0 : loc[...]) +/- sum_kk G_k[row][kk] rb[kk][r0 + r]
 // One warp per row; the rhs chunk of rb is staged in shared memory as [RN][m].
 template <typename T, int RN, bool FWD>
@@ -510,26 +537,20 @@ __global__ void __launch_bounds__(256) sweep_gemv(const BoxInfo* __restrict__ bo
 #pragma unroll
         for (int r = 0; r < RN; ++r) acc[r] = mk<T>(0, 0);
         const cplx<T>* g = Gk + (size_t)row * B.ld;
+        // two entries of G in flight ahead of their products (G comes from HBM, one pass)
+        cplx<T> gv = lane < m ? g[lane] : mk<T>(0, 0), g1 = lane + 32 < m ? g[lane + 32] : mk<T>(0, 0);
         for (int kk = lane; kk < m; kk += 32) {
-            const cplx<T> gv = g[kk];
+            const cplx<T> g2 = kk + 64 < m ? g[kk + 64] : mk<T>(0, 0);
 #pragma unroll
             for (int r = 0; r < RN; ++r) cmac(acc[r], gv, rs[r * m + kk]);
+            gv = g1;
+            g1 = g2;
         }
-#pragma unroll
-        for (int r = 0; r < RN; ++r) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
-                acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
-            }
-        }
-        cplx<T>* dst = loc + (B.loc_off + (long long)k * m + row) * nrhs + r0;
-#pragma unroll
-        for (int r = 0; r < RN; ++r) {
-            if (lane == r && r < rn) {
-                if (FWD) dst[r] = acc[r];
-                else dst[r] = dst[r] - acc[r];
-            }
+        const cplx<T> sum = warp_sum_columns<T, RN>(acc, lane);
+        const int r = lane & (RN - 1);
+        if (lane < RN && r < rn) {
+            cplx<T>* dst = loc + (B.loc_off + (long long)k * m + row) * nrhs + r0 + r;
+            *dst = FWD ? sum : *dst - sum;
         }
     }
 }
@@ -1061,6 +1082,9 @@ void launch_sweep_rn(const PlaneSet& P, cplx<T>* loc, cplx<T>* rbuf, int nrhs, c
     const int chunks = (nrhs + RN - 1) / RN;
     const long long want = 2LL * std::max(1, ctx->sm_count);
     int rows_per = (int)std::min<long long>(64, std::max<long long>(8, (long long)m * P.nbox * chunks / want / 8 * 8));
+    // complex128 is bound by the FP64 pipe, so an SM's share of rows is what counts: one row per warp (four or more CTAs
+    // per SM, taken as SMs come free) where the staged columns leave room for them
+    if (sizeof(T) == 8 && (size_t)RN * m * sizeof(cplx<T>) <= 48 * 1024) rows_per = 8;
     const dim3 ggrid((m + rows_per - 1) / rows_per, P.nbox, (nrhs + RN - 1) / RN);
     const size_t smem = (size_t)RN * m * sizeof(cplx<T>);
     const unsigned pblocks = (unsigned)std::min<long long>(((long long)m * nrhs + 255) / 256, 1024);
