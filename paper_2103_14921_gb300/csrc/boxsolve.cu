@@ -10,7 +10,9 @@
 // the right-hand side for 2 CT complex multiply-adds); the slices are added in a fixed order, so results do not
 // depend on scheduling.
 //
-// Bound: shared-memory loads and latency of the serial step chain (G comes from L2, where all planes of a set stay).
+// Bound: the product's FP32 multiply-adds (8 x 8-node planes, 16 columns: 4,300 clocks per step and SM with two CTAs, 4,100
+// at full rate); around it the items of a plane belong to fixed threads, so that their indices are formed once and what
+// they read from global memory is loaded a step ahead (with the indices and loads in the loops a step took 14,500).
 #include <atomic>
 
 #include "internal.h"
@@ -18,6 +20,7 @@
 namespace {
 
 constexpr int BS_THREADS = 256;
+constexpr int BS_ITEMS = 4;   // (node, column) items of a plane per thread at most
 
 template <int BYTES>
 __device__ __forceinline__ void bs_copy(void* s, const void* g) {
@@ -33,7 +36,7 @@ struct BoxPlan {
 };
 
 template <typename TV, typename TL, int CT>
-__global__ void __launch_bounds__(BS_THREADS) box_solve(const BoxInfo* __restrict__ boxes,
+__global__ void __launch_bounds__(BS_THREADS, 2) box_solve(const BoxInfo* __restrict__ boxes,
                                                         const cplx<TL>* __restrict__ coef,
                                                         const cplx<TL>* __restrict__ G, const cplx<TV>* __restrict__ v,
                                                         cplx<TV>* __restrict__ out, cplx<TL>* __restrict__ loc, int nx,
@@ -54,7 +57,7 @@ __global__ void __launch_bounds__(BS_THREADS) box_solve(const BoxInfo* __restric
         const int k = plane_of(t), buf = pl.nbuf == 2 ? t & 1 : 0;
         const C* Gk = G + B.fac_off + (long long)k * B.pstride;
         C* gd = gs + (size_t)buf * m_max * gp;
-        if (sizeof(C) == 8 && (m & 1) == 0 && pl.wide) {
+        if (sizeof(C) == 8 && pl.wide) {
             // rows of an even length start on 16 bytes: two entries per copy
             for (int i = tid / 32; i < m; i += BS_THREADS / 32)
                 for (int q = 2 * (tid % 32); q < m; q += 64) bs_copy<16>(gd + i * gp + q, Gk + (long long)i * B.ld + q);
@@ -70,33 +73,69 @@ __global__ void __launch_bounds__(BS_THREADS) box_solve(const BoxInfo* __restric
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     fetch(0);
+    // this thread's items of a plane: column r0 + (tid mod cc), nodes tid / cc + i (256 / cc); per item the in-plane
+    // node (-1: none), its grid offset in plane 0 of the box, and whether the box's core holds it
+    const int cl = tid & (cc - 1), col = r0 + cl, p_first = tid / cc, p_step = BS_THREADS / cc;
+    const bool has = col < nrhs;
+    int px_[BS_ITEMS], py_[BS_ITEMS];
+    uint32_t core = 0;
+#pragma unroll
+    for (int i = 0; i < BS_ITEMS; ++i) {
+        const int p = p_first + i * p_step;
+        px_[i] = p < m ? p % bx : -1;
+        py_[i] = p / bx;
+        const int gi = B.lo[0] + px_[i], gj = B.lo[1] + py_[i];
+        if (p < m && gi >= B.core_lo[0] && gi < B.core_hi[0] && gj >= B.core_lo[1] && gj < B.core_hi[1]) core |= 1u << i;
+    }
+    auto at_grid = [&](int i, int k) {
+        return (((long long)(B.lo[2] + k) * ny + B.lo[1] + py_[i]) * nx + B.lo[0] + px_[i]) * nrhs + col;
+    };
+    auto at_loc = [&](int i, int k) { return (B.loc_off + (long long)k * m + p_first + i * p_step) * nrhs + col; };
+    // b of the next forward plane, loaded a step ahead; backward, y of the current one, loaded before its product
+    C nxt[BS_ITEMS];
+#pragma unroll
+    for (int i = 0; i < BS_ITEMS; ++i) {
+        nxt[i] = mk<TL>(0, 0);
+        if (px_[i] >= 0 && has) {
+            const cplx<TV> a = v[at_grid(i, 0)];
+            nxt[i] = mk<TL>((TL)a.x, (TL)a.y);
+        }
+    }
     const int mh = (m + 1) / 2, ncg = cc / CT, units = mh * ncg, kw = (m + pl.ks - 1) / pl.ks;
     for (int t = 0; t < nsteps; ++t) {
         const bool fwd = t < bz;
         const int k = plane_of(t), buf = pl.nbuf == 2 ? t & 1 : 0;
         asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();   // step t's G and coefficients, the previous step's plane of vec
+        __syncthreads();   // step t's G and coefficients, the previous step's plane of win
         if (pl.nbuf == 2 && t + 1 < nsteps) fetch(t + 1);
         // the prepared right-hand side; couplings that leave the box have zero coefficients, their index is clamped
         const C* ck = cs + (size_t)buf * m_max * 9;
-        for (int e = tid; e < m * cc; e += BS_THREADS) {
-            const int p = e / cc, r = e % cc;
-            const int px = p % bx, py = p / bx;
-            C acc = mk<TL>(0, 0);
-            if (fwd && r0 + r < nrhs) {
-                const cplx<TV> a = v[(((long long)(B.lo[2] + k) * ny + B.lo[1] + py) * nx + B.lo[0] + px) * nrhs + r0 + r];
-                acc = mk<TL>((TL)a.x, (TL)a.y);
-            }
+#pragma unroll
+        for (int i = 0; i < BS_ITEMS; ++i) {
+            if (px_[i] < 0) break;
+            const int p = p_first + i * p_step;
+            C acc = fwd ? nxt[i] : mk<TL>(0, 0);
             if (t > 0) {
+                const int xo[3] = {max(px_[i] - 1, 0), px_[i], min(px_[i] + 1, bx - 1)};
 #pragma unroll
                 for (int d = 0; d < 9; ++d) {
-                    const int qx = min(max(px + d % 3 - 1, 0), bx - 1), qy = min(max(py + d / 3 - 1, 0), by - 1);
+                    const int qy = min(max(py_[i] + d / 3 - 1, 0), by - 1);
                     C c = ck[p * 9 + d];
                     if (fwd) c = mk<TL>(-c.x, -c.y);
-                    cmac(acc, c, win[(qy * bx + qx) * cc + r]);
+                    cmac(acc, c, win[(qy * bx + xo[d % 3]) * cc + cl]);
                 }
             }
-            rb[e] = acc;
+            rb[p * cc + cl] = acc;
+        }
+#pragma unroll
+        for (int i = 0; i < BS_ITEMS; ++i) {
+            if (px_[i] < 0 || !has) break;
+            if (t + 1 < bz) {
+                const cplx<TV> a = v[at_grid(i, t + 1)];
+                nxt[i] = mk<TL>((TL)a.x, (TL)a.y);
+            } else if (!fwd) {
+                nxt[i] = loc[at_loc(i, k)];
+            }
         }
         __syncthreads();
         const C* gk = gs + (size_t)buf * m_max * gp;
@@ -128,20 +167,17 @@ __global__ void __launch_bounds__(BS_THREADS) box_solve(const BoxInfo* __restric
         if (pl.nbuf == 1 && t + 1 < nsteps) fetch(t + 1);
         // y_k (kept for the backward sweep), or x_k: written by the box whose core holds the node (owner partition of
         // unity; the last forward plane is also the first of the backward sweep)
-        const int gk_z = B.lo[2] + k;
-        const bool core_z = t >= bz - 1 && gk_z >= B.core_lo[2] && gk_z < B.core_hi[2];
-        for (int e = tid; e < m * cc; e += BS_THREADS) {
-            C sum = part[e];
-            for (int s = 1; s < pl.ks; ++s) sum = sum + part[(size_t)s * m_max * cc + e];
-            const int p = e / cc, r = r0 + e % cc;
-            C x = sum;
-            if (r < nrhs) {
-                C* y = loc + (B.loc_off + (long long)k * m + p) * nrhs + r;
-                if (t < bz - 1) *y = sum;
-                if (!fwd) x = *y - sum;
-                const int gi = B.lo[0] + p % bx, gj = B.lo[1] + p / bx;
-                if (core_z && gi >= B.core_lo[0] && gi < B.core_hi[0] && gj >= B.core_lo[1] && gj < B.core_hi[1])
-                    out[(((long long)gk_z * ny + gj) * nx + gi) * nrhs + r] = mk<TV>((TV)x.x, (TV)x.y);
+        const bool core_z = t >= bz - 1 && B.lo[2] + k >= B.core_lo[2] && B.lo[2] + k < B.core_hi[2];
+#pragma unroll
+        for (int i = 0; i < BS_ITEMS; ++i) {
+            if (px_[i] < 0) break;
+            const int e = (p_first + i * p_step) * cc + cl;
+            C x = part[e];
+            for (int s = 1; s < pl.ks; ++s) x = x + part[(size_t)s * m_max * cc + e];
+            if (has) {
+                if (t < bz - 1) loc[at_loc(i, k)] = x;
+                if (!fwd) x = nxt[i] - x;
+                if (core_z && ((core >> i) & 1u)) out[at_grid(i, k)] = mk<TV>((TV)x.x, (TV)x.y);
             }
             win[e] = x;
         }
@@ -156,7 +192,7 @@ BoxPlan box_plan(helm_ctx ctx, const PlaneSet& P, int nrhs) {
     const size_t es = sizeof(cplx<TL>);
     const int m = P.m_max, mh = (m + 1) / 2;
     for (int cc = 16; cc >= 1; cc >>= 1) {
-        if (cc > 1 && cc >= 2 * nrhs) continue;
+        if ((cc > 1 && cc >= 2 * nrhs) || m * cc > BS_ITEMS * BS_THREADS) continue;
         BoxPlan p;
         p.cc = cc;
         // pitch: the rows a warp reads fall in different banks (odd, or 2 mod 4 where 16-byte copies need an even one)
