@@ -96,8 +96,10 @@ __global__ void __launch_bounds__(RED_THREADS, 2) dots_kernel(const cplx<T>* __r
     if (any && *any == 0) return;
     const long long t = (long long)blockIdx.x * RED_THREADS + threadIdx.x;
     const long long stride = (long long)gridDim.x * RED_THREADS;
-    for (int ib = 0; ib < ni; ib += IC) {
-        const int nq = min(IC, ni - ib);
+    // passes of equal width (9 vectors: 5 + 4, not 8 + 1)
+    const int wid = (ni + (ni + IC - 1) / IC - 1) / ((ni + IC - 1) / IC);
+    for (int ib = 0; ib < ni; ib += wid) {
+        const int nq = min(wid, ni - ib);
         const bool with_norm = npart && ib == 0;
         CAcc<T> acc[IC];
         cplx<T> part[IC];
@@ -274,9 +276,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_norm_kernel(const cplx<
 // projection's coefficients, plain FP32 sums per thread: they only correct rounding-level remainders) and of
 // |w'|^2 (compensated) are reduced per block.  Runs on the reduction grid (one column per thread), one
 // resident block per SM.
-// HS: the coefficients h are read from shared memory at every use instead of being held in registers
-// (needs ni * nrhs <= 16 IM); the freed registers carry twice as many elements per trip.
-template <typename T, int IM, bool HS = false>
+template <typename T, int IM>
 __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kernel(const cplx<T>* __restrict__ V, long long vstride,
                                                                     cplx<T>* __restrict__ w, long long n_el, int nrhs,
                                                                     int ni, const c128* __restrict__ hsrc,
@@ -292,15 +292,13 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
     if (hsm)
         for (int e = threadIdx.x; e < ni * nrhs; e += RED_THREADS) hs[e] = mk<T>((T)hsrc[e].x, (T)hsrc[e].y);
     __syncthreads();
-    cplx<T> h[HS ? 1 : IM];
-    if (!HS) {
+    cplx<T> h[IM];
 #pragma unroll
-        for (int q = 0; q < IM; ++q)
-            if (q < ni) {
-                if (hsm) h[q] = hs[q * nrhs + r];
-                else h[q] = mk<T>((T)hsrc[(long long)q * nrhs + r].x, (T)hsrc[(long long)q * nrhs + r].y);
-            }
-    }
+    for (int q = 0; q < IM; ++q)
+        if (q < ni) {
+            if (hsm) h[q] = hs[q * nrhs + r];
+            else h[q] = mk<T>((T)hsrc[(long long)q * nrhs + r].x, (T)hsrc[(long long)q * nrhs + r].y);
+        }
     cplx<T> acc[IM];
 #pragma unroll
     for (int q = 0; q < IM; ++q) acc[q] = mk<T>(0, 0);
@@ -308,9 +306,8 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
     // EPT elements per trip (e, e + stride, ...: the same column), so that every trip keeps the same number
     // of basis loads in flight whatever IM is
     // (bases of up to 4 vectors: 8 elements (8 / IM in FP64), two blocks per SM)
-    constexpr int EPT0 = IM <= 4 ? (sizeof(T) == 4 ? 8 : 8 / IM)
+    constexpr int EPT = IM <= 4 ? (sizeof(T) == 4 ? 8 : 8 / IM)
                                  : ((sizeof(T) == 4 ? 32 : 16) / IM > 0 ? (sizeof(T) == 4 ? 32 : 16) / IM : 1);
-    constexpr int EPT = HS ? 2 * EPT0 : EPT0;
     for (long long e0 = t; e0 < n_el; e0 += EPT * stride) {
         cplx<T> v[EPT][IM];
         cplx<T> x[EPT];
@@ -330,7 +327,7 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
 #pragma unroll
             for (int q = 0; q < IM; ++q)
                 if (q < ni) {
-                    const cplx<T> hq = HS ? hs[q * nrhs + r] : h[HS ? 0 : q];
+                    const cplx<T> hq = h[q];
                     x[u].x -= hq.x * v[u][q].x - hq.y * v[u][q].y;
                     x[u].y -= hq.x * v[u][q].y + hq.y * v[u][q].x;
                 }
@@ -366,6 +363,94 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
         for (int u = threadIdx.x; u < RED_THREADS; u += nrhs) sum += sn[u];
         const int rr = (int)(((long long)blockIdx.x * RED_THREADS + threadIdx.x) % nrhs);
         npart[(long long)blockIdx.x * nrhs + rr] = sum;
+    }
+}
+
+// update_dots_kernel for 9 to 2 IMH basis vectors and at most 128 columns, each element shared by two lanes of a warp (l and
+// l + 16): lane half z owns the vectors q = 2 i + z, the halves of w - V h1 are exchanged with one shuffle pair, and
+// each half forms its own projections.  Half the registers per thread, so two blocks are resident per SM with EPT * IMH
+// (16 or more) basis loads in flight per thread, and the template widths follow ni in steps of four vectors.  112^3 x
+// 16: 5.1 - 5.8 TB/s, where the wide kernel (one block per SM, widths 16 and 32) ran at 3.2 - 4.7 (17 vectors: 1084 -> 671
+// us, 24: 1167 -> 809); at 5 to 8 vectors the wide kernel is the faster one (8: 348 us against 407).
+template <typename T, int IMH, int EPT>
+__global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T>* __restrict__ V, long long vstride,
+                                                                   cplx<T>* __restrict__ w, long long n_el, int nrhs, int ni,
+                                                                   const c128* __restrict__ hsrc,
+                                                                   c128* __restrict__ partial, int ldp,
+                                                                   double* __restrict__ npart) {
+    extern __shared__ __align__(16) unsigned char uds_smem[];
+    cplx<T>* hs = reinterpret_cast<cplx<T>*>(uds_smem);   // [ni][nrhs]
+    constexpr int SLOTS = RED_THREADS / 2, QG = 4;
+    __shared__ c128 s[QG][2][SLOTS];
+    __shared__ double sn[SLOTS];
+    const int lane = threadIdx.x & 31, z = lane >> 4, slot = (threadIdx.x >> 5) * 16 + (lane & 15);
+    const long long t = (long long)blockIdx.x * SLOTS + slot, stride = (long long)gridDim.x * SLOTS;
+    const int r = (int)(t % nrhs);
+    for (int e = threadIdx.x; e < ni * nrhs; e += RED_THREADS) hs[e] = mk<T>((T)hsrc[e].x, (T)hsrc[e].y);
+    __syncthreads();
+    const cplx<T>* hz = hs + z * nrhs + r;
+    cplx<T> acc[IMH];
+#pragma unroll
+    for (int i = 0; i < IMH; ++i) acc[i] = mk<T>(0, 0);
+    RAcc<T> nrm;
+    // the loop bound is that of the warp's first element, so that all its lanes take part in the exchanges
+    for (long long e0 = t; e0 - (lane & 15) < n_el; e0 += EPT * stride) {
+        cplx<T> v[EPT][IMH], x[EPT];
+#pragma unroll
+        for (int u = 0; u < EPT; ++u) {
+            const long long e = e0 + u * stride, ec = e < n_el ? e : 0;
+#pragma unroll
+            for (int i = 0; i < IMH; ++i)
+                if (2 * i + z < ni) v[u][i] = V[(long long)(2 * i + z) * vstride + ec];
+            x[u] = z == 0 ? w[ec] : mk<T>(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < EPT; ++u) {
+            const long long e = e0 + u * stride;
+#pragma unroll
+            for (int i = 0; i < IMH; ++i)
+                if (2 * i + z < ni) {
+                    const cplx<T> h = hz[2 * i * nrhs];
+                    x[u].x -= h.x * v[u][i].x - h.y * v[u][i].y;
+                    x[u].y -= h.x * v[u][i].y + h.y * v[u][i].x;
+                }
+            x[u].x += __shfl_xor_sync(0xffffffffu, x[u].x, 16);
+            x[u].y += __shfl_xor_sync(0xffffffffu, x[u].y, 16);
+            if (e < n_el) {
+                if (z == 0) {
+                    w[e] = x[u];
+                    nrm.add(x[u].x * x[u].x + x[u].y * x[u].y);
+                }
+#pragma unroll
+                for (int i = 0; i < IMH; ++i)
+                    if (2 * i + z < ni) cmac_conj(acc[i], v[u][i], x[u]);
+            }
+        }
+    }
+    if (z == 0) sn[slot] = nrm.value();
+    const int nr = min(nrhs, SLOTS);
+#pragma unroll
+    for (int i0 = 0; i0 < IMH; i0 += QG) {
+        if (2 * i0 >= ni) break;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < QG; ++i)
+            if (i0 + i < IMH) s[i][z][slot] = widen(acc[i0 + i]);
+        __syncthreads();
+        const int nq = min(2 * QG, ni - 2 * i0);
+        for (int o = threadIdx.x; o < nq * nr; o += RED_THREADS) {
+            const int q = o / nr, u0 = o % nr;
+            c128 sum = mk<double>(0, 0);
+            for (int u = u0; u < SLOTS; u += nrhs) sum = sum + s[q >> 1][q & 1][u];
+            const int rr = (int)(((long long)blockIdx.x * SLOTS + u0) % nrhs);
+            partial[((long long)blockIdx.x * ldp + 2 * i0 + q) * nrhs + rr] = sum;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < nr) {
+        double sum = 0.0;
+        for (int u = threadIdx.x; u < SLOTS; u += nrhs) sum += sn[u];
+        npart[(long long)blockIdx.x * nrhs + (int)(((long long)blockIdx.x * SLOTS + threadIdx.x) % nrhs)] = sum;
     }
 }
 
@@ -759,6 +844,22 @@ inline bool cgs2_fits(int ni, int S) {
     return ni <= (sizeof(T) == 4 ? 32 : 16) && (size_t)ni * S * sizeof(cplx<T>) <= 40 * 1024;
 }
 
+// Widths in steps of four vectors (eight above 24: width 14 measured as slow as the wide kernel); EPT keeps 16 basis loads
+// or more in flight per thread (half in complex128).
+template <typename T, typename... Args>
+void launch_update_dots_split(int nblk, size_t hsm, cudaStream_t st, const cplx<T>* V, long long vs, cplx<T>* w, long long n_el,
+                              int S, int ni, Args... args) {
+    constexpr bool F = sizeof(T) == 4;
+    auto go = [&](auto kern) { kern<<<nblk, RED_THREADS, hsm, st>>>(V, vs, w, n_el, S, ni, args...); };
+    if (ni <= 12) go(update_dots_split<T, 6, F ? 3 : 1>);
+    else if (ni <= 16) go(update_dots_split<T, 8, F ? 2 : 1>);
+    else if constexpr (F) {
+        if (ni <= 20) go(update_dots_split<T, 10, 2>);
+        else if (ni <= 24) go(update_dots_split<T, 12, 2>);
+        else go(update_dots_split<T, 16, 1>);
+    }
+}
+
 // CGS2 in three passes over the basis: h1 = V^H w; w' = w - V h1 fused with h2 = V^H w' and ||w'||; H[.][j] = h1 + h2,
 // H[j+1][j] = sqrt(||w'||^2 - ||h2||^2); the Givens step; then v_{j+1} = (w' - V h2) / H[j+1][j] fused with the
 // second update.  Five launches: the three passes and the two small kernels that close the reductions (112^3 x 16:
@@ -769,12 +870,13 @@ void fused_cgs2(helm_ctx ctx, cudaStream_t st, const CgsBuffers<T>& B, int j, co
     const long long nel = B.nel;
     const cplx<T>* V = B.V;
     cplx<T>* w = B.w;
-    // resident blocks per SM for the fused kernel (two for bases of up to 4 vectors, whose smaller register
-    // arrays allow it), as the largest multiple of q <= that many blocks
+    // resident blocks per SM for the fused kernel (two for bases of up to 4 vectors and for the split form, whose smaller
+    // register arrays allow it), as the largest multiple of q <= that many blocks
     int a = RED_THREADS, bq = S;
     while (bq) { const int t = a % bq; a = bq; bq = t; }
     const int q = S / a;
-    const int per_sm = ni <= 4 ? 2 : 1;
+    const bool split = ni > 8 && S <= RED_THREADS / 2;
+    const int per_sm = ni <= 4 || split ? 2 : 1;
     const int nb1 = std::min(B.nblk, std::max(q, (per_sm * std::max(1, ctx->sm_count) / q) * q));
     int tk = family ? prof_begin(ctx, family) : -1;
     if (ni <= 2)
@@ -784,7 +886,10 @@ void fused_cgs2(helm_ctx ctx, cudaStream_t st, const CgsBuffers<T>& B, int j, co
     prof_end(ctx, tk, (double)(ni + 1) * nel * sizeof(cplx<T>));
     finish_first<<<ni * S, 128, 0, st>>>(B.part, B.nblk, B.ldp, S, B.hpass, B.H, B.m, j, B.running);
     tk = family ? prof_begin(ctx, family) : -1;
-    if (ni <= 2)
+    const size_t hsm = (size_t)ni * S * sizeof(cplx<T>);
+    if (split)
+        launch_update_dots_split<T>(nb1, hsm, st, V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
+    else if (ni <= 2)
         update_dots_kernel<T, 2><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
     else if (ni <= 4)
         update_dots_kernel<T, 4><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
@@ -792,9 +897,6 @@ void fused_cgs2(helm_ctx ctx, cudaStream_t st, const CgsBuffers<T>& B, int j, co
         update_dots_kernel<T, 8><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
     else if (ni <= 16 || sizeof(T) == 8)
         update_dots_kernel<T, 16><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass, B.part, B.ldp, B.dpart);
-    else if (S <= 16)
-        update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16), true><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass,
-                                                                                            B.part, B.ldp, B.dpart);
     else
         update_dots_kernel<T, (sizeof(T) == 4 ? 32 : 16)><<<nb1, RED_THREADS, 0, st>>>(V, nel, w, nel, S, ni, B.hpass,
                                                                                        B.part, B.ldp, B.dpart);
@@ -802,7 +904,6 @@ void fused_cgs2(helm_ctx ctx, cudaStream_t st, const CgsBuffers<T>& B, int j, co
     finish_second<<<S, FS_THREADS, 0, st>>>(B.part, B.dpart, nb1, B.ldp, S, ni, B.hpass, B.H, B.Sd, B.cs, B.sn, B.gv, B.inv,
                                             j, B.m, B.running);
     tk = family ? prof_begin(ctx, family) : -1;
-    const size_t hsm = (size_t)ni * S * sizeof(cplx<T>);
     cplx<T>* vn = B.V + (long long)(j + 1) * nel;
     if (ni <= 2)
         update_scale_kernel<T, (sizeof(T) == 4 ? 8 : 4), (sizeof(T) == 4 ? 2 : 4)><<<B.nblk, RED_THREADS, hsm, st>>>(
