@@ -337,9 +337,9 @@ struct MarchTile {
 
 // The vectors of one plane buffer a thread copies at most (the tile is chosen within it).
 template <typename V> struct MarchCfg;
-template <> struct MarchCfg<float4> { static constexpr int MN = 4, NU = 7, BPS = 3, WORK = 220, LAT = 4000; };
-template <> struct MarchCfg<float2> { static constexpr int MN = 4, NU = 8, BPS = 5, WORK = 150, LAT = 4000; };
-template <> struct MarchCfg<double2> { static constexpr int MN = 4, NU = 8, BPS = 2, WORK = 2900, LAT = 3000; };
+template <> struct MarchCfg<float4> { static constexpr int MN = 4, NU = 7, BPS = 3, WORK = 110, LAT = 3600; };
+template <> struct MarchCfg<float2> { static constexpr int MN = 4, NU = 8, BPS = 5, WORK = 75, LAT = 3600; };
+template <> struct MarchCfg<double2> { static constexpr int MN = 4, NU = 8, BPS = 2, WORK = 2900, LAT = 2000; };
 
 template <typename V>
 __host__ __device__ constexpr size_t march_smem(int pc, int gx, int mty) {
@@ -679,8 +679,8 @@ PlainRange plain_range(helm_grid g) {
 }
 
 // The tile of the z-march: PC column vectors (at most 8, the chunks of equal width), and the x-groups, rows and planes
-// per block with the least estimated time on this grid: rounds of resident blocks times the planes they walk
-// (two of them halo) times the larger of a plane's latency and the SM's work on it.
+// per block with the least estimated time on this grid: the blocks' walks (two planes of halo each), a plane costing
+// its latency and the schedulers' work on it.
 template <typename V>
 MarchTile march_tile(const helm_grid_desc& d, int nrs, int sms, int planes) {
     constexpr int MN = MarchCfg<V>::MN;
@@ -705,11 +705,13 @@ MarchTile march_tile(const helm_grid_desc& d, int nrs, int sms, int planes) {
                 const double blocks = xy * ((d.nz + mzc - 1) / mzc), slots = (double)per_sm * sms;
                 // clocks of one plane with res blocks on an SM: a warp's latency, or its scheduler's work
                 auto plane = [&](double res) {
-                    return std::max((double)MarchCfg<V>::LAT,
-                                    std::ceil(res * (threads / 32) / 4.0) * MarchCfg<V>::WORK * MN);
+                    const double warps = std::ceil(res * (threads / 32) / 4.0);   // per scheduler
+                    return MarchCfg<V>::LAT + warps * MarchCfg<V>::WORK * MN;
                 };
-                const double full = std::floor(blocks / slots), rest = blocks - full * slots;
-                const double time = (full * plane(per_sm) + (rest > 0 ? plane(std::ceil(rest / sms)) : 0.0)) * (mzc + 2);
+                // blocks are replaced as they finish, so the total work spread over the slots, but no less than one walk,
+                // and a quarter of a walk of tail
+                const double walk = (mzc + 2) * plane(std::min((double)per_sm, std::ceil(blocks / sms)));
+                const double time = std::max(blocks * (mzc + 2) * plane(per_sm) / slots, walk) + 0.25 * walk;
                 if (time < best) {
                     best = time;
                     t.gx = gx;
