@@ -36,8 +36,8 @@ namespace {
 constexpr int SAS = 8;    // digits of S
 constexpr int SAX = 3;    // digits of X as a left operand
 constexpr int SBM = 5;    // digits of a right operand at most
-constexpr int GM = 128, GN = 64, GK = 64;
-constexpr int A_SLOT = GM * 128, B_SLOT = GN * 128;
+constexpr int GM = 128, GK = 64;
+constexpr int A_SLOT = GM * 128;
 
 __device__ __forceinline__ double pow2(int e) {
     e = min(max(e, -1022), 1023);
@@ -125,18 +125,19 @@ __device__ __forceinline__ c128 col_at(const ColSrc& c, const BoxInfo& B, int bo
     return c.g[B.fac_off + (long long)k * B.pstride + (long long)p * B.ld + j];
 }
 
-// exponents of the columns: 32 columns per block, 8 rows at a time
-__global__ void __launch_bounds__(256) dp_col_exponents(const BoxInfo* __restrict__ boxes, ColSrc src, int* __restrict__ eout,
+// exponents of the columns: 32 columns per block, 32 rows at a time
+__global__ void __launch_bounds__(1024) dp_col_exponents(const BoxInfo* __restrict__ boxes, ColSrc src, int* __restrict__ eout,
                                                         int Lc, int k, int* __restrict__ flag,
                                                         const int* __restrict__ gate) {
-    __shared__ uint32_t red[8][32];
+    __shared__ uint32_t red[32][32];
     const int box = blockIdx.y;
     const BoxInfo B = boxes[box];
     if (k >= B.dims[2] || (int)blockIdx.x * 32 >= B.m || gated_out(gate, box)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
     uint32_t hi = 0;
     if (j < B.m)
-        for (int p = w; p < B.m; p += 8) {
+#pragma unroll 4
+        for (int p = w; p < B.m; p += 32) {
             const c128 v = col_at(src, B, box, k, p, j);
             hi = max(hi, max(high_word(v.x), high_word(v.y)));
         }
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(256) dp_col_exponents(const BoxInfo* __restric
     __syncthreads();
     if (w == 0 && j < B.m) {
 #pragma unroll
-        for (int i = 1; i < 8; ++i) hi = max(hi, red[i][lane]);
+        for (int i = 1; i < 32; ++i) hi = max(hi, red[i][lane]);
         eout[box * Lc + j] = exponent_of(hi, flag);
     }
 }
@@ -195,46 +196,203 @@ __global__ void __launch_bounds__(256) dp_slice_cols(const BoxInfo* __restrict__
     }
 }
 
-template <int SA, int SB>
-constexpr int dp_smem() { return SA * A_SLOT + 2 * SB * B_SLOT + 1024 + 256; }
+// x 2^e for finite x; results below the normal range become 0
+__device__ __forceinline__ double scale2(double x, int e) {
+    const int hi = __double2hiint(x), E = ((hi >> 20) & 2047) + e;
+    if (((hi >> 20) & 2047) == 0 || E <= 0) return 0.0;
+    return E >= 2047 ? __hiloint2double((hi & 0x80000000) | 0x7FF00000, 0) : __hiloint2double(hi + e * (1 << 20), __double2loint(x));
+}
+// the double of an integer below 2^51 in size: one addition on the FP64 pipe
+__device__ __forceinline__ double small_double(long long v) {
+    return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0;
+}
 
-// D = (left operand) (right operand) of one 128 x 64 (real) tile per CTA, the orders below O.  ADD = false: R = I - D (pitch
-// m); true: G += D.  Warp 0 lane 0 loads (TMA), warp 1 lane 0 issues the MMAs, warps 2-5 read the accumulators.  Each digit of
-// the left operand has one shared-memory slot, loaded again as soon as its products of a chunk are done: the products
-// run from the last digit (fewest partners) to the first, so that a slot's load has most of a chunk's time; the right
-// operand's slots are double.  Every wait is bounded.
-template <int SA, int SB, int O, bool ADD>
-__global__ void __launch_bounds__(192, 1) dp_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
+// One pass of dp_gemm: the orders LO <= i + j < HI of the products of digits i < SA and j < SB, which need the digits
+// A0 <= i < A1 and B0 <= j < B1.  Each operand has a ring of slots, filled in the order of first use (A digits descend).
+template <int SA, int SB, int LO, int HI, int GN>
+struct DpPass {
+    static constexpr int A0 = LO - SB + 1 > 0 ? LO - SB + 1 : 0, A1 = SA < HI ? SA : HI;
+    static constexpr int B0 = LO - SA + 1 > 0 ? LO - SA + 1 : 0, B1 = SB < HI ? SB : HI;
+    static constexpr int NA = GN == 64 || A1 - A0 > 7 ? 8 : 7, NB = (14 - NA) * (128 / GN);
+    static __device__ constexpr int first(int j) { return HI - 1 - j < A1 - 1 ? HI - 1 - j : A1 - 1; }   // first i that uses B_j
+    static __device__ constexpr int last(int j) { return LO - j > A0 ? LO - j : A0; }
+};
+constexpr int DP_SLOTS = 20;                           // barriers: 8 + 12 slots at 64 columns, 14 at 128
+constexpr int dp_smem() { return 14 * A_SLOT + 1024 + 512; }
+
+struct DpPipe {
+    unsigned char* base;
+    uint64_t *full, *empty, *done, *drained;
+    int* err;
+    uint32_t phase;   // one bit per slot: producer, the phase of its last load (ones before the first); consumer, the next phase
+    bool ok;
+};
+
+template <int GN>
+__device__ __forceinline__ unsigned char* dp_slot(unsigned char* base, int s, int na) {
+    return s < na ? base + s * A_SLOT : base + na * A_SLOT + (s - na) * (GN * 128);
+}
+
+template <class P, int GN>
+__device__ __forceinline__ void dp_load(DpPipe& p, uint32_t& used, int s, const CUtensorMap& map, int x, int y, int z) {
+    if (p.ok) p.ok = tc::mbar_wait(&p.empty[s], (p.phase >> s) & 1, p.err, 32);
+    if (!p.ok) return;
+    tc::mbar_arrive_expect_tx(&p.full[s], s < P::NA ? A_SLOT : GN * 128);
+    tc::tma_load_3d(dp_slot<GN>(p.base, s, P::NA), &map, x, y, z, &p.full[s]);
+    p.phase ^= 1u << s;
+    used |= 1u << s;
+}
+
+template <class P, int GN>
+__device__ __forceinline__ void dp_produce(DpPipe& p, uint32_t& used, const CUtensorMap& mA, const CUtensorMap& mB, int nK, int row0,
+                                           int n0, int nb, int box) {
+    int a = 0, b = 0;
+    for (int kc = 0; kc < nK && p.ok; ++kc) {
+#pragma unroll
+        for (int i = P::A1 - 1; i >= P::A0; --i) {
+            dp_load<P, GN>(p, used, a, mA, kc * GK, row0, i * nb + box);
+            a = a + 1 == P::NA ? 0 : a + 1;
+#pragma unroll
+            for (int j = P::B0; j < P::B1; ++j) {
+                if (P::first(j) != i) continue;
+                dp_load<P, GN>(p, used, P::NA + b, mB, kc * GK, n0, j * nb + box);
+                b = b + 1 == P::NB ? 0 : b + 1;
+            }
+        }
+    }
+}
+
+template <class P, int LO, int HI, int GN>
+__device__ __forceinline__ void dp_consume(DpPipe& p, uint32_t tmem, int nK) {
+    constexpr uint32_t idesc = tc::idesc_bf16(GM, GN);
+    uint32_t seen = 0;   // orders that hold a product already
+    int a = 0, b = 0, bs[P::B1];
+    for (int kc = 0; kc < nK && p.ok; ++kc) {
+#pragma unroll
+        for (int i = P::A1 - 1; i >= P::A0; --i) {
+            if (p.ok) p.ok = tc::mbar_wait(&p.full[a], (p.phase >> a) & 1, p.err, 34);
+            p.phase ^= 1u << a;
+#pragma unroll
+            for (int j = P::B0; j < P::B1; ++j) {
+                if (P::first(j) != i) continue;
+                bs[j] = P::NA + b;
+                b = b + 1 == P::NB ? 0 : b + 1;
+                if (p.ok) p.ok = tc::mbar_wait(&p.full[bs[j]], (p.phase >> bs[j]) & 1, p.err, 33);
+                p.phase ^= 1u << bs[j];
+            }
+            if (!p.ok) continue;
+            tc::fence_after_sync();
+            const uint32_t aa = tc::smem_u32(dp_slot<GN>(p.base, a, P::NA));
+#pragma unroll
+            for (int j = P::B0; j < P::B1; ++j) {
+                if (i + j < LO || i + j >= HI) continue;
+                const int o = i + j - LO;
+                const uint32_t ab = tc::smem_u32(dp_slot<GN>(p.base, bs[j], P::NA));
+#pragma unroll
+                for (int kk = 0; kk < GK / 16; ++kk)
+                    tc::mma_f16(tmem + o * GN, tc::desc_k_sw128(aa + kk * 32), tc::desc_k_sw128(ab + kk * 32), idesc,
+                                ((seen >> o) & 1u) | (kk > 0 ? 1u : 0u));
+                seen |= 1u << o;
+            }
+            tc::mma_commit(&p.empty[a]);
+            a = a + 1 == P::NA ? 0 : a + 1;
+#pragma unroll
+            for (int j = P::B0; j < P::B1; ++j)
+                if (P::last(j) == i) tc::mma_commit(&p.empty[bs[j]]);
+        }
+    }
+    tc::mma_commit(p.done);
+}
+
+// The orders LO .. HI - 1 of the tile as doubles.  ADD: G += them; else R = -them, and with LAST R = I - them + what the pass
+// before left there.
+template <int LO, int HI, int GN, bool ADD, bool LAST, bool FIRST>
+__device__ __forceinline__ void dp_epilogue(uint32_t tmem, int c_begin, int n0, int I, int m, int er, const int* __restrict__ eb,
+                                            c128* __restrict__ row, bool& bad, uint32_t& big) {
+    constexpr int O = HI - LO, OH = O < 4 ? O : 4;   // orders of the first 64-bit integer
+#pragma unroll 1
+    for (int c0 = c_begin; c0 < c_begin + GN / 2; c0 += 8) {
+        const int j0 = (n0 + c0) / 2;
+        uint32_t v[O][8];
+#pragma unroll
+        for (int o = 0; o < O; ++o) tc::tmem_ld_32x32b_x8(tmem + (uint32_t)(o * GN + c0), v[o]);
+        c128 old[4];
+        int ej[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const bool in = I < m && j0 + h < m;
+            ej[h] = in ? eb[j0 + h] : 0;
+            old[h] = (ADD || !FIRST) && in ? row[j0 + h] : mk<double>(0, 0);
+        }
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int j = j0 + h;
+            if (I >= m || j >= m) continue;
+            const int E = er + ej[h];
+            double d[2], l[2];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                long long vh = 0, vl = 0;
+#pragma unroll
+                for (int o = 0; o < O; ++o) {
+                    const float a = __uint_as_float(v[o][2 * h + x]);
+                    bad |= !(fabsf(a) < 8388608.f);
+                    if (o < OH) vh = vh * 256 + __float2int_rn(a);
+                    else vl = vl * 256 + __float2int_rn(a);
+                }
+                d[x] = scale2(small_double(vh), E - 8 * (LO + OH - 1));
+                l[x] = O > 4 ? scale2(small_double(vl), E - 8 * (HI - 1)) : 0.0;
+            }
+            if (ADD) {
+                row[j] = mk<double>(old[h].x + d[0], old[h].y + d[1]);
+            } else if (!LAST) {
+                row[j] = mk<double>(-d[0], -d[1]);
+            } else {
+                double re = (I == j ? 1.0 : 0.0) - d[0], im = -d[1];
+                if (O > 4) re -= l[0], im -= l[1];
+                if (!FIRST) re += old[h].x, im += old[h].y;
+                row[j] = mk<double>(re, im);
+                big = max(big, max(high_word(re), high_word(im)));
+            }
+        }
+    }
+}
+
+// D = (left operand) (right operand) of one 128 x GN (real) tile per CTA, the orders below O.  ADD = false: R = I - D (pitch
+// m); true: G += D.  Warp 0 lane 0 loads (TMA), warp 1 lane 0 issues the MMAs, warps 2-9 read the accumulators.  TMEM holds
+// 4 orders of 128 columns or 8 of 64: at 128 columns more than four orders take two passes over K, the small orders last
+// (the first pass leaves its part in the output).  A digit's slot is free again after its last product of a chunk; the
+// order of the products gives each load at least six products' time.  Every wait is bounded.
+template <int SA, int SB, int O, bool ADD, int GN>
+__global__ void __launch_bounds__(320, 1) dp_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
                                                   const BoxInfo* __restrict__ boxes, const int* __restrict__ ea,
                                                   const int* __restrict__ eb, int nb, int Lr, int Lc, int m_max,
                                                   c128* __restrict__ out, float limit, int k, int* __restrict__ flag,
                                                   int* __restrict__ stat, const int* __restrict__ gate) {
     extern __shared__ __align__(1024) unsigned char dp_raw[];
+    constexpr bool TWO = O * GN > 512;
+    static_assert(!(TWO && ADD), "an addition is one pass");
+    using PL = DpPass<SA, SB, TWO ? 4 : 0, O, GN>;            // the first pass: the large orders, or all
+    using PH = DpPass<SA, SB, 0, TWO ? 4 : O, GN>;
+    constexpr uint32_t TCOLS = (TWO ? 4 : O) * GN <= 256 ? 256 : 512;
     const int box = blockIdx.z;
     const BoxInfo B = boxes[box];
     const int m = B.m, row0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
     if (k >= B.dims[2] || row0 >= m || n0 >= 2 * m || gated_out(gate, box)) return;
-    unsigned char* sa = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dp_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    unsigned char* sb = sa + SA * A_SLOT;
-    uint64_t* fullA = reinterpret_cast<uint64_t*>(sb + 2 * SB * B_SLOT);
-    uint64_t* emptyA = fullA + SA;
-    uint64_t* fullB = emptyA + SA;
-    uint64_t* emptyB = fullB + 2;
-    uint64_t* done = emptyB + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-    constexpr uint32_t TCOLS = O * GN <= 256 ? 256 : 512;
-    int* err = flag + 1;
+    DpPipe p;
+    p.base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dp_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    p.full = reinterpret_cast<uint64_t*>(p.base + 14 * A_SLOT);
+    p.empty = p.full + DP_SLOTS;
+    p.done = p.empty + DP_SLOTS;
+    p.drained = p.done + 1;
+    p.err = flag + 1;
+    p.ok = true;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(p.drained + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < SA; ++i) {
-            tc::mbar_init(&fullA[i], 1);
-            tc::mbar_init(&emptyA[i], 1);
-        }
-        for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&fullB[i], 1);
-            tc::mbar_init(&emptyB[i], 1);
-        }
-        tc::mbar_init(done, 1);
+        for (int i = 0; i < 2 * DP_SLOTS + 1; ++i) tc::mbar_init(&p.full[i], 1);
+        tc::mbar_init(p.drained, 8);
         tc::fence_barrier_init();
         tc::prefetch_tmap(&mA);
         tc::prefetch_tmap(&mB);
@@ -250,117 +408,50 @@ __global__ void __launch_bounds__(192, 1) dp_gemm(const __grid_constant__ CUtens
     const int nK = (2 * m + GK - 1) / GK;
     if (warp == 0) {
         if (lane == 0) {
-            int na[SA], nbuf[2] = {0, 0};   // loads issued per barrier
-#pragma unroll
-            for (int i = 0; i < SA; ++i) na[i] = 0;
-            bool ok = true;
-            for (int kc = 0; kc < nK && ok; ++kc) {
-                const int buf = kc & 1;
-                if (kc >= 2 && !tc::mbar_wait(&emptyB[buf], ((kc >> 1) - 1) & 1, err, 31)) break;
-                tc::mbar_arrive_expect_tx(&fullB[buf], SB * B_SLOT);
-                for (int j = 0; j < SB; ++j)
-                    tc::tma_load_3d(sb + (buf * SB + j) * B_SLOT, &mB, kc * GK, n0, j * nb + box, &fullB[buf]);
-                nbuf[buf]++;
-#pragma unroll
-                for (int i = SA - 1; i >= 0; --i) {
-                    if (ok && kc >= 1) ok = tc::mbar_wait(&emptyA[i], (kc - 1) & 1, err, 32);
-                    if (!ok) continue;
-                    tc::mbar_arrive_expect_tx(&fullA[i], A_SLOT);
-                    tc::tma_load_3d(sa + i * A_SLOT, &mA, kc * GK, row0, i * nb + box, &fullA[i]);
-                    na[i]++;
-                }
-            }
+            uint32_t used = 0;
+            p.phase = 0xFFFFFFFFu;
+            dp_produce<PL, GN>(p, used, mA, mB, nK, row0, n0, nb, box);
+            if (TWO) dp_produce<PH, GN>(p, used, mA, mB, nK, row0, n0, nb, box);
             // a give-up anywhere: let the loads already issued land before the slots are left
-            if (!ok || *reinterpret_cast<volatile int*>(err) != 0) {
-#pragma unroll
-                for (int i = 0; i < SA; ++i)
-                    if (na[i]) tc::mbar_drain(&fullA[i], (na[i] - 1) & 1);
-                for (int i = 0; i < 2; ++i)
-                    if (nbuf[i]) tc::mbar_drain(&fullB[i], (nbuf[i] - 1) & 1);
-            }
+            if (!p.ok || *reinterpret_cast<volatile int*>(p.err) != 0)
+                for (int s = 0; s < DP_SLOTS; ++s)
+                    if ((used >> s) & 1) tc::mbar_drain(&p.full[s], (p.phase >> s) & 1);
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16(GM, GN);
-            uint32_t seen = 0;   // orders that hold a product already
-            bool ok = true;
-            for (int kc = 0; kc < nK && ok; ++kc) {
-                const int buf = kc & 1;
-                if (!tc::mbar_wait(&fullB[buf], (kc >> 1) & 1, err, 33)) break;
-                const uint32_t ab = tc::smem_u32(sb + buf * SB * B_SLOT);
-#pragma unroll
-                for (int i = SA - 1; i >= 0; --i) {
-                    if (ok) ok = tc::mbar_wait(&fullA[i], kc & 1, err, 34);
-                    if (!ok) continue;
-                    tc::fence_after_sync();
-                    const uint32_t aa = tc::smem_u32(sa + i * A_SLOT);
-#pragma unroll
-                    for (int j = 0; j < SB; ++j) {
-                        if (i + j >= O) break;
-                        const int o = i + j;
-#pragma unroll
-                        for (int kk = 0; kk < GK / 16; ++kk)
-                            tc::mma_f16(tmem + o * GN, tc::desc_k_sw128(aa + kk * 32), tc::desc_k_sw128(ab + j * B_SLOT + kk * 32),
-                                        idesc, ((seen >> o) & 1u) | (kk > 0 ? 1u : 0u));
-                        seen |= 1u << o;
-                    }
-                    tc::mma_commit(&emptyA[i]);
-                }
-                if (ok) tc::mma_commit(&emptyB[buf]);
+            p.phase = 0;
+            dp_consume<PL, TWO ? 4 : 0, O, GN>(p, tmem, nK);
+            if (TWO) {
+                if (p.ok) p.ok = tc::mbar_wait(p.drained, 0, p.err, 36);
+                tc::fence_after_sync();
+                dp_consume<PH, 0, 4, GN>(p, tmem, nK);
             }
-            tc::mma_commit(done);
         }
     } else {
-        const bool ok = tc::mbar_wait(done, 0, err, 35);
-        if (!ok) tc::mbar_drain(done, 0);   // products already issued still write TMEM
+        const int q = warp & 3, I = row0 + q * 32 + lane, cb = (warp - 2) / 4 * (GN / 2);
+        const int er = I < m ? ea[box * Lr + I] - 14 : 0;
+        const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16);
+        const int* ebb = eb + box * Lc;
+        c128* row = ADD ? out + B.fac_off + (long long)k * B.pstride + (long long)I * B.ld
+                        : out + (size_t)box * m_max * m_max + (size_t)I * m;
+        bool bad = false, ok = tc::mbar_wait(p.done, 0, p.err, 35);
+        uint32_t big = 0;
+        if (!ok) tc::mbar_drain(p.done, 0);   // products already issued still write TMEM
         tc::fence_after_sync();
-        if (ok) {
-            const int q = warp & 3, I = row0 + q * 32 + lane;
-            const int er = I < m ? ea[box * Lr + I] - 14 : 0;
-            constexpr int OH = O < 4 ? O : 4;   // orders of the first 64-bit integer
-            bool bad = false;
-            float big = 0.f;
-#pragma unroll 1
-            for (int c0 = 0; c0 < GN; c0 += 8) {
-                uint32_t v[O][8];
-#pragma unroll
-                for (int o = 0; o < O; ++o) tc::tmem_ld_32x32b_x8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(o * GN + c0), v[o]);
-                tc::tmem_ld_wait();
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const int j = (n0 + c0) / 2 + h;
-                    if (I >= m || j >= m) continue;
-                    const int E = er + eb[box * Lc + j];
-                    const double sh = pow2(E - 8 * (OH - 1)), sl = pow2(E - 8 * (O - 1));
-                    double d[2];
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        long long vh = 0, vl = 0;
-#pragma unroll
-                        for (int o = 0; o < O; ++o) {
-                            const float a = __uint_as_float(v[o][2 * h + x]);
-                            bad |= !(fabsf(a) < 8388608.f);
-                            if (o < OH) vh = vh * 256 + __float2int_rn(a);
-                            else vl = vl * 256 + __float2int_rn(a);
-                        }
-                        d[x] = (double)vh * sh;
-                        if (O > 4) d[x] = fma((double)vl, sl, d[x]);
-                    }
-                    if (ADD) {
-                        c128* g = out + B.fac_off + (long long)k * B.pstride + (long long)I * B.ld + j;
-                        *g = mk<double>(g->x + d[0], g->y + d[1]);
-                    } else {
-                        const double re = (I == j ? 1.0 : 0.0) - d[0];
-                        out[(size_t)box * m_max * m_max + (size_t)I * m + j] = mk<double>(re, -d[1]);
-                        big = fmaxf(big, fmaxf(fabsf((float)re), fabsf((float)d[1])));
-                    }
-                }
-            }
-            if (bad || (!ADD && !(big <= limit))) atomicOr(flag, 2);
-            if (!ADD && stat) {   // the largest entry (non-negative floats compare like their bits)
-                const int b = __reduce_max_sync(0xffffffffu, __float_as_int(big));
-                if (lane == 0) atomicMax(stat + box, b);
-            }
+        if (ok) dp_epilogue<TWO ? 4 : 0, O, GN, ADD, !TWO, true>(tm, cb, n0, I, m, er, ebb, row, bad, big);
+        if (TWO) {
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(p.drained);
+            if (ok && !(ok = tc::mbar_wait(p.done, 1, p.err, 37))) tc::mbar_drain(p.done, 1);
+            tc::fence_after_sync();
+            if (ok) dp_epilogue<0, 4, GN, ADD, true, false>(tm, cb, n0, I, m, er, ebb, row, bad, big);
+        }
+        const float f = (float)__hiloint2double((int)big, 0);
+        if (ok && (bad || (!ADD && !(f <= limit)))) atomicOr(flag, 2);
+        if (ok && !ADD && stat) {   // the largest entry (non-negative floats compare like their bits)
+            const int b = __reduce_max_sync(0xffffffffu, __float_as_int(f));
+            if (lane == 0) atomicMax(stat + box, b);
         }
     }
     tc::fence_before_sync();
@@ -390,18 +481,28 @@ bool encode_slices(CUtensorMap* map, void* base, uint64_t cols, uint64_t rows, u
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int SA, int SB, int O, bool ADD>
-void launch_gemm(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const int* ea, const BoxInfo* dbox, int nbox, int m_max,
-                 c128* out, float limit, int k, int* flag, int* stat = nullptr, const int* gate = nullptr) {
+template <int SA, int SB, int O, bool ADD, int GN>
+void launch_gemm_n(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const CUtensorMap& mB, const int* ea, const BoxInfo* dbox,
+                   int nbox, int m_max, c128* out, float limit, int k, int* flag, int* stat, const int* gate) {
     static std::atomic<bool> attr{false};
     if (!attr.load(std::memory_order_acquire)) {
-        cudaFuncSetAttribute(dp_gemm<SA, SB, O, ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, dp_smem<SA, SB>());
+        cudaFuncSetAttribute(dp_gemm<SA, SB, O, ADD, GN>, cudaFuncAttributeMaxDynamicSharedMemorySize, dp_smem());
         attr.store(true, std::memory_order_release);
     }
     const dim3 grid((2 * m_max + GN - 1) / GN, (m_max + GM - 1) / GM, nbox);
-    dp_gemm<SA, SB, O, ADD><<<grid, 192, dp_smem<SA, SB>(), ctx->stream>>>(mA, D.mB, dbox, ea, D.eB, D.nb, D.Lr, D.Nr / 2, D.m_max,
-                                                                           out, limit, k, flag, stat, gate);
+    dp_gemm<SA, SB, O, ADD, GN><<<grid, 320, dp_smem(), ctx->stream>>>(mA, mB, dbox, ea, D.eB, D.nb, D.Lr, D.Nr / 2, D.m_max, out,
+                                                                       limit, k, flag, stat, gate);
     ctx->launches++;
+}
+
+template <int SA, int SB, int O, bool ADD>
+void launch_gemm(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const int* ea, const BoxInfo* dbox, int nbox, int m_max,
+                 c128* out, float limit, int k, int* flag, int* stat = nullptr, const int* gate = nullptr) {
+    const long long tiles = (long long)((2 * m_max + 127) / 128) * ((m_max + GM - 1) / GM) * nbox;
+    if (tiles > ctx->sm_count)
+        launch_gemm_n<SA, SB, O, ADD, 128>(ctx, D, mA, D.mB128, ea, dbox, nbox, m_max, out, limit, k, flag, stat, gate);
+    else
+        launch_gemm_n<SA, SB, O, ADD, 64>(ctx, D, mA, D.mB64, ea, dbox, nbox, m_max, out, limit, k, flag, stat, gate);
 }
 
 template <int S>
@@ -416,7 +517,7 @@ template <int S>
 void slice_cols(helm_ctx ctx, const DpWork& D, const TgjWork& T, const BoxInfo* dbox, int nbox, int m_max, const ColSrc& src,
                 c128* gout, int k, const int* gate = nullptr) {
     const int t = (m_max + 31) / 32;
-    dp_col_exponents<<<dim3(t, nbox), 256, 0, ctx->stream>>>(dbox, src, D.eB, D.Nr / 2, k, T.flag, gate);
+    dp_col_exponents<<<dim3(t, nbox), 1024, 0, ctx->stream>>>(dbox, src, D.eB, D.Nr / 2, k, T.flag, gate);
     dp_slice_cols<S><<<dim3(t, t, nbox), 256, 0, ctx->stream>>>(dbox, src, (__nv_bfloat16*)D.B, D.nb, D.Nr, D.Kp, D.eB, gout, k, gate);
     ctx->launches += 2;
 }
@@ -427,7 +528,7 @@ static void dp_sizes(int nb, int m_max, DpWork& W) {
     W.nb = nb;
     W.m_max = m_max;
     W.Lr = (m_max + GM - 1) / GM * GM;
-    W.Nr = 2 * ((m_max + 31) / 32 * 32);
+    W.Nr = std::max(128, 2 * ((m_max + 31) / 32 * 32));
     W.Kp = (2 * m_max + GK - 1) / GK * GK;
     W.as_bytes = (size_t)SAS * nb * W.Lr * W.Kp * 2;
     W.ax_bytes = (size_t)SAX * nb * W.Lr * W.Kp * 2;
@@ -470,7 +571,8 @@ helm_status dp_alloc(helm_ctx ctx, int nb, int m_max, DpWork& W) {
     const uint64_t c = 2ull * m_max;
     if (!encode_slices(&W.mAS, W.AS, c, W.Lr, (uint64_t)SAS * nb, W.Kp, GM) ||
         !encode_slices(&W.mAX, W.AX, c, W.Lr, (uint64_t)SAX * nb, W.Kp, GM) ||
-        !encode_slices(&W.mB, W.B, c, W.Nr, (uint64_t)SBM * nb, W.Kp, GN)) {
+        !encode_slices(&W.mB64, W.B, c, W.Nr, (uint64_t)SBM * nb, W.Kp, 64) ||
+        !encode_slices(&W.mB128, W.B, c, W.Nr, (uint64_t)SBM * nb, W.Kp, 128)) {
         dp_free(ctx, W);
         return set_error(ctx, HELM_ECUDA, "cuTensorMapEncodeTiled failed for the digit slices");
     }

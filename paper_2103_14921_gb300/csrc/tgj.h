@@ -27,7 +27,7 @@ struct DpWork {
     size_t as_bytes = 0, ax_bytes = 0, b_bytes = 0, e_bytes = 0;
     void *AS = nullptr, *AX = nullptr, *B = nullptr;   // digit slices of S and X (left operands) and of a right operand
     int *eS = nullptr, *eX = nullptr, *eB = nullptr;   // their row and column exponents
-    CUtensorMap mAS, mAX, mB;
+    CUtensorMap mAS, mAX, mB64, mB128;   // (right operand: boxes of 64 and of 128 rows)
 };
 size_t dp_bytes(int nb, int m_max);
 helm_status dp_alloc(helm_ctx ctx, int nb, int m_max, DpWork& W);

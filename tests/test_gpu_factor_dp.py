@@ -21,6 +21,8 @@ pytestmark = pytest.mark.gpu
     ((43, 3, 4), (1, 1, 1), 0, None),          # 129
     ((33, 31, 6), (2, 2, 1), 1, 80.0),         # boxes of 16..18 x 16..17 nodes
     ((40, 22, 5), (1, 1, 1), 0, None),         # 880: seven panels, the last partial
+    ((43, 41, 3), (1, 1, 1), 0, None),         # 1763: more 128-column tiles than SMs, two passes of four orders
+    ((70, 62, 3), (2, 2, 1), 1, 80.0),         # the same with boxes of up to 36 x 32 = 1152 = 9 x 128 nodes
 ])
 def test_newton_inverses_match_pivoted_fp64_elimination(dims, parts, ov, Q):
     from paper_2103_14921_gb300 import build, helm
