@@ -44,7 +44,7 @@ constexpr int UST = 2;               // operand ring stages
 constexpr int A_TILE = UBM * 128;    // 128 rows x 32 fp32 = 16 KB
 constexpr int B_TILE = UBN * 128;    // 256 rows x 32 fp32 = 32 KB
 constexpr int STAGE = 2 * A_TILE + 2 * B_TILE;
-constexpr int DIAG_THREADS = 512;
+constexpr int DIAG_THREADS = 640;   // 16 warps of the rank steps, 4 of the column chain
 constexpr int DP = NB + 1;           // row pitch of the diagonal block in shared memory
 
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
@@ -139,109 +139,208 @@ __global__ void tgj_pad_diag(const BoxInfo* __restrict__ boxes, c64* __restrict_
 
 // ------------------------------------------------------------------ panel: block inverse, operands
 
-// P = A[J,J]^{-1} in shared memory by in-place Gauss-Jordan in sub-panels of SB columns, pivots by largest modulus
-// among the block's rows not used yet.  Rows are not swapped: s_p[c] is the row that column c was eliminated with, and
-// the inverse is P[c][s_p[k]] = X[s_p[c]][k].
+// P = A[J,J]^{-1} by in-place Gauss-Jordan in sub-panels of SB columns, pivots by largest modulus among the block's rows not
+// used yet.  Rows are not swapped: s_p[c] is the row that column c was eliminated with (s_k its inverse), and
+// P[s_k[row]][s_p[col]] = X[row][col] in the end.
 //
-// A sub-panel is eliminated by 128 threads, one row each with its SB entries in registers; per column a 32-bit key
-// (|x|^2 in the high bits, the row in the low seven) is reduced with one redux per warp and the scaled pivot row is
-// broadcast through shared memory: two barriers of four warps per column.  Its accumulated transform W then reaches the
-// other columns in one rank-SB step of all 16 warps, 4 x 8 outputs per thread, X <- [rows not used here] X + W X[pivot rows].
-// Bound: the serial column chain (128 x about 400 clocks) and the rank-SB steps (128^3 complex multiply-adds on one
-// SM's FP32 lanes, 32 us).
+// X stays in registers: thread (rg, cg) of 32 x 16 holds rows 4 rg .. 4 rg + 3 and columns cg + 16 i.  A sub-panel (slot 0
+// of every thread; the slots rotate) goes to shared memory and is eliminated by four warps, a row per thread; per column
+// a 32-bit key (|x|^2 in the high bits, the row in the low seven) is reduced with one redux per warp, each warp's best
+// row is published with it (and the pivot's reciprocal), and every thread scales by itself: one barrier of four warps per
+// column.  The transform W
+// then reaches the other columns in a rank-SB step of the other 16 warps, X <- [rows not used here] X + W X[pivot rows]: the
+// next sub-panel's columns first, so that the four warps eliminate it during the rest of the step.
+// Bound: the serial column chain, and the rank-SB steps (128^3 complex multiply-adds on one SM's FP32 lanes, 32 us).
 constexpr int SB = 16;
-constexpr int DIAG_SMEM = (NB * DP + SB * NB) * (int)sizeof(c64);
+constexpr int SWP = SB + 2;           // row pitch of a sub-panel in shared memory
+constexpr int DIAG_SMEM = NB * DP * (int)sizeof(c64);
+static_assert(2 * NB * SWP + SB * NB <= NB * DP, "the sub-panels and the pivot rows share the block's memory");
 
-__device__ __forceinline__ void diag_inverse(c64* X, c64* Brow, int* s_p, int* s_k, float amax, int* flag) {
-    __shared__ uint32_t s_key[2][4];
-    __shared__ __align__(16) c64 s_row[2][SB];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    bool used = false;   // this thread's row (threads below NB)
-    for (int c0 = 0; c0 < NB; c0 += SB) {
-        if (tid < NB) {
-            c64 a[SB];
+struct DiagShared {
+    uint4 key[2];
+    c64 row[2][4][SB + 2];   // a warp's best row and 1 / its pivot
+    int p[NB], k[NB];
+};
+
+// One sub-panel, columns c0 .. c0 + SB - 1 of the block, by 128 threads: Wr is the row'th row.  The columns rotate through
+// the registers, so that the loop stays rolled: sixteen copies of its body ran at the speed of instruction fetch.
+__device__ __forceinline__ void diag_columns(c64* Wr, DiagShared& D, bool& used, int row, int c0, float amax, int* flag) {
+    const int lane = row & 31, wid = row >> 5;
+    c64 a[SB];
 #pragma unroll
-            for (int j = 0; j < SB; ++j) a[j] = X[tid * DP + c0 + j];
+    for (int j = 0; j < SB; j += 2) {
+        const float4 v = *reinterpret_cast<const float4*>(Wr + j);
+        a[j] = mk<float>(v.x, v.y);
+        a[j + 1] = mk<float>(v.z, v.w);
+    }
+    float q;
+    c64 inv;
+    uint32_t key, kw;
+    auto candidate = [&]() {
+        q = a[0].x * a[0].x + a[0].y * a[0].y;
+        const float d = q > 0.f ? 1.f / q : 1.f;
+        inv = q > 0.f ? mk<float>(a[0].x * d, -a[0].y * d) : mk<float>(1.f, 0.f);
+        // rows not used yet: |x|^2 rounded down to 16 mantissa bits, ties to the smallest row; used: 0
+        key = used ? 0u : ((__float_as_uint(q) & 0xFFFFFF80u) | (uint32_t)(NB - 1 - row)) + 1u;
+        kw = __reduce_max_sync(0xffffffffu, key);
+    };
+    candidate();
+#pragma unroll 1
+    for (int j = 0; j < SB; ++j) {
+        const int pb = j & 1;
+        if (lane == 0) reinterpret_cast<uint32_t*>(&D.key[pb])[wid] = kw;
+        if (key == kw && kw) {
+            float4* o = reinterpret_cast<float4*>(D.row[pb][wid]);
 #pragma unroll
-            for (int j = 0; j < SB; ++j) {
-                const int c = c0 + j, pb = j & 1;
-                const float q = a[j].x * a[j].x + a[j].y * a[j].y;
-                // rows not used yet: |x|^2 rounded down to 16 mantissa bits, ties to the smallest row; used: 0
-                const uint32_t key = used ? 0u : ((__float_as_uint(q) & 0xFFFFFF80u) | (uint32_t)(NB - 1 - tid)) + 1u;
-                const uint32_t kw = __reduce_max_sync(0xffffffffu, key);
-                if (lane == 0) s_key[pb][wid] = kw;
-                tc::named_bar(1, NB);
-                const uint32_t km = max(max(s_key[pb][0], s_key[pb][1]), max(s_key[pb][2], s_key[pb][3]));
-                const int p = NB - 1 - (int)((km - 1u) & 127u);
-                if (tid == p) {
-                    if (!(q > 0.f)) atomicOr(flag, 1);
-                    else if (q < 1e-12f * amax) atomicOr(flag, 2);
-                    const float d = q > 0.f ? 1.f / q : 1.f;
-                    const c64 inv = q > 0.f ? mk<float>(a[j].x * d, -a[j].y * d) : mk<float>(1.f, 0.f);
+            for (int i = 0; i < SB / 2; ++i) o[i] = make_float4(a[2 * i].x, a[2 * i].y, a[2 * i + 1].x, a[2 * i + 1].y);
+            D.row[pb][wid][SB] = inv;
+        }
+        __syncwarp();
+        tc::named_bar(1, NB);
+        const uint4 k4 = D.key[pb];
+        const uint32_t km = max(max(k4.x, k4.y), max(k4.z, k4.w));
+        const int p = NB - 1 - (int)((km - 1u) & 127u);
+        const c64* r = D.row[pb][p >> 5];
+        // the pivot row becomes inv r, the others a - (a_0 inv) r; column 0 (inv, or -a_0 inv) rotates to the end
+        const c64 ip = r[SB];
+        const bool piv = row == p;
+        if (piv) {
+            if (!(q > 0.f)) atomicOr(flag, 1);
+            else if (q < 1e-12f * amax) atomicOr(flag, 2);
+            used = true;
+            D.p[c0 + j] = row;
+            D.k[row] = c0 + j;
+        }
+        const c64 g = piv ? ip : mk<float>(-(a[0].x * ip.x - a[0].y * ip.y), -(a[0].x * ip.y + a[0].y * ip.x));
+        auto step = [&](int i, float x, float y) {
+            c64 t = piv ? mk<float>(0.f, 0.f) : a[i];
+            cmac(t, g, mk<float>(x, y));
+            a[i - 1] = t;
+        };
+        step(1, r[1].x, r[1].y);
+        candidate();   // of the next column, while the others are updated
 #pragma unroll
-                    for (int i = 0; i < SB; ++i) {
-                        a[i] = i == j ? inv : a[i] * inv;
-                        s_row[pb][i] = a[i];
-                    }
-                    used = true;
-                    s_p[c] = tid;
-                    s_k[tid] = c;
-                }
-                tc::named_bar(1, NB);
-                if (tid != p) {
-                    const c64 f = mk<float>(-a[j].x, -a[j].y);
-                    a[j] = mk<float>(0.f, 0.f);
+        for (int i = 1; i < SB / 2; ++i) {
+            const float4 v = reinterpret_cast<const float4*>(r)[i];
+            step(2 * i, v.x, v.y);
+            step(2 * i + 1, v.z, v.w);
+        }
+        a[SB - 1] = g;
+    }
 #pragma unroll
-                    for (int i = 0; i < SB; i += 2) {
-                        const float4 r = *reinterpret_cast<const float4*>(&s_row[pb][i]);
-                        cmac(a[i], f, mk<float>(r.x, r.y));
-                        cmac(a[i + 1], f, mk<float>(r.z, r.w));
-                    }
-                }
+    for (int j = 0; j < SB; j += 2) *reinterpret_cast<float4*>(Wr + j) = make_float4(a[j].x, a[j].y, a[j + 1].x, a[j + 1].y);
+}
+
+// slots I0 .. I1 - 1 of X <- [rows not used here] X + W X[pivot rows]
+template <int I0, int I1>
+__device__ __forceinline__ void diag_step(c64 (&x)[4][8], const c64* W, const c64* Brow, int rg, int cg, uint32_t piv) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = I0; i < I1; ++i)
+            if ((piv >> r) & 1) x[r][i] = mk<float>(0.f, 0.f);
+#pragma unroll(I1 - I0 > 1 ? 1 : 4)
+    for (int c = 0; c < SB; c += 2) {
+        float4 w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) w[r] = *reinterpret_cast<const float4*>(W + (4 * rg + r) * SWP + c);
+#pragma unroll
+        for (int i = I0; i < I1; ++i) {
+            const c64 b0 = Brow[c * NB + i * 16 + cg], b1 = Brow[(c + 1) * NB + i * 16 + cg];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                cmac(x[r][i], mk<float>(w[r].x, w[r].y), b0);
+                cmac(x[r][i], mk<float>(w[r].z, w[r].w), b1);
             }
-#pragma unroll
-            for (int j = 0; j < SB; ++j) X[tid * DP + c0 + j] = a[j];
         }
-        __syncthreads();
-        for (int e = tid; e < SB * NB; e += DIAG_THREADS) Brow[e] = X[s_p[c0 + e / NB] * DP + e % NB];
-        __syncthreads();
-        // thread (row group of 4, column group of 8): rows 4 rg .. 4 rg + 3, columns cg + 16 i
-        const int rg = tid >> 4, cg = tid & 15;
-        c64 acc[4][8];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int k = s_k[4 * rg + r];
-            const bool piv = k >= c0 && k < c0 + SB;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[r][i] = piv ? mk<float>(0.f, 0.f) : X[(4 * rg + r) * DP + cg + 16 * i];
-        }
-#pragma unroll 4
-        for (int c = 0; c < SB; ++c) {
-            c64 w[4], b[8];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) w[r] = X[(4 * rg + r) * DP + c0 + c];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) b[i] = Brow[c * NB + cg + 16 * i];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) cmac(acc[r][i], w[r], b[i]);
-        }
-        // the sub-panel's own columns (i = c0 / 16) are left as they are
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (i != c0 / SB) X[(4 * rg + r) * DP + cg + 16 * i] = acc[r][i];
-        __syncthreads();
     }
 }
 
-// hi and lo parts of the pair (a, b) at an operand position
-__device__ __forceinline__ void split2(float* h, float* l, size_t at, float a, float b) {
-    const float ah = tf32_hi(a), bh = tf32_hi(b);
-    *reinterpret_cast<float2*>(h + at) = make_float2(ah, bh);
-    *reinterpret_cast<float2*>(l + at) = make_float2(a - ah, b - bh);
+// the inverse P of the 128 x 128 block at A (pitch L) into X (pitch DP)
+__device__ __forceinline__ void diag_inverse(const c64* __restrict__ A, int L, c64* X, DiagShared& D, float* s_max, int* flag) {
+    constexpr int RT = DIAG_THREADS - NB;   // threads of the rank steps
+    const int tid = threadIdx.x;
+    c64* const Wb = X;                    // [2][NB][SWP]
+    c64* const Brow = X + 2 * NB * SWP;   // [SB][NB]
+    if (tid >= RT) {
+        const int row = tid - RT;
+        bool used = false;
+        D.k[row] = -1;
+        tc::named_bar(2, DIAG_THREADS);
+        float amax = 0.f;
+        for (int w = 0; w < RT / 32; ++w) amax = fmaxf(amax, s_max[w]);
+        diag_columns(Wb + row * SWP, D, used, row, 0, amax, flag);
+#pragma unroll 1
+        for (int s = 0; s < NB / SB; ++s) {
+            for (int i = 0; i < 3; ++i) tc::named_bar(2, DIAG_THREADS);
+            if (s + 1 < NB / SB) diag_columns(Wb + (((s + 1) & 1) * NB + row) * SWP, D, used, row, (s + 1) * SB, amax, flag);
+        }
+        tc::named_bar(2, DIAG_THREADS);
+        __syncthreads();
+        return;
+    }
+    const int rg = tid >> 4, cg = tid & 15;
+    c64 x[4][8];
+    float amax = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[r][i] = A[(size_t)(4 * rg + r) * L + cg + 16 * i];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) amax = fmaxf(amax, x[r][i].x * x[r][i].x + x[r][i].y * x[r][i].y);
+    amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));   // non-negative: ordered like the bits
+    if ((tid & 31) == 0) s_max[tid >> 5] = amax;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) Wb[(4 * rg + r) * SWP + cg] = x[r][0];
+    tc::named_bar(2, DIAG_THREADS);
+#pragma unroll 1
+    for (int s = 0; s < NB / SB; ++s) {
+        const c64* W = Wb + (s & 1) * NB * SWP;
+        c64* Wn = Wb + ((s + 1) & 1) * NB * SWP;
+        const int c0 = s * SB;
+        tc::named_bar(2, DIAG_THREADS);   // W is complete
+        uint32_t piv = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int k = D.k[4 * rg + r] - c0;
+            if (k >= 0 && k < SB) {
+                piv |= 1u << r;
+#pragma unroll
+                for (int i = 1; i < 8; ++i) Brow[k * NB + i * 16 + cg] = x[r][i];
+            }
+        }
+        __syncwarp();
+        tc::named_bar(2, DIAG_THREADS);   // and the pivot rows
+        diag_step<1, 2>(x, W, Brow, rg, cg, piv);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) Wn[(4 * rg + r) * SWP + cg] = x[r][1];
+        tc::named_bar(2, DIAG_THREADS);   // the next sub-panel's columns
+        diag_step<2, 8>(x, W, Brow, rg, cg, piv);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const c64 own = W[(4 * rg + r) * SWP + cg];
+#pragma unroll
+            for (int i = 0; i < 7; ++i) x[r][i] = x[r][i + 1];
+            x[r][7] = own;
+        }
+    }
+    tc::named_bar(2, DIAG_THREADS);       // X takes the sub-panels' place
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int c = D.k[4 * rg + r];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) X[c * DP + D.p[cg + 16 * i]] = x[r][i];
+    }
+    __syncthreads();
+}
+
+// hi and lo parts of four values at an operand position
+__device__ __forceinline__ void split4(float* h, float* l, size_t at, float a, float b, float c, float d) {
+    const float4 v = make_float4(tf32_hi(a), tf32_hi(b), tf32_hi(c), tf32_hi(d));
+    *reinterpret_cast<float4*>(h + at) = v;
+    *reinterpret_cast<float4*>(l + at) = make_float4(a - v.x, b - v.y, c - v.z, d - v.w);
 }
 
 // The panel's first launch, in which nothing depends on anything else: CTA b < nbox inverts the diagonal block of box b
@@ -254,38 +353,24 @@ __global__ void __launch_bounds__(DIAG_THREADS) tgj_panel(const BoxInfo* __restr
                                                           float* __restrict__ Bh, float* __restrict__ Bl,
                                                           int* __restrict__ flag, int j0, int k) {
     extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ int s_p[NB], s_k[NB];
-    __shared__ float s_wmax[DIAG_THREADS / 32];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    c64* X = reinterpret_cast<c64*>(dsm);   // [NB][DP], then the pivot rows of a sub-panel [SB][NB]
+    __shared__ __align__(16) DiagShared s_d;
+    __shared__ float s_max[DIAG_THREADS / 32];
+    const int tid = threadIdx.x;
+    c64* X = reinterpret_cast<c64*>(dsm);   // [NB][DP]
     if ((int)blockIdx.x < nbox) {
         const int box = blockIdx.x;
         const int m = boxes[box].m;
         if (k >= boxes[box].dims[2] || j0 >= m) return;
-        const c64* A = S + (size_t)box * L * L;
-        float amax = 0.f;
-        for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
-            const c64 v = A[(size_t)(j0 + e / NB) * L + j0 + e % NB];
-            X[(e / NB) * DP + e % NB] = v;
-            amax = fmaxf(amax, v.x * v.x + v.y * v.y);
-        }
-        if (tid < NB) s_k[tid] = -1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        if (lane == 0) s_wmax[wid] = amax;
-        __syncthreads();
-        amax = 0.f;
-        for (int w = 0; w < DIAG_THREADS / 32; ++w) amax = fmaxf(amax, s_wmax[w]);
-        diag_inverse(X, X + NB * DP, s_p, s_k, amax, flag);
+        diag_inverse(S + (size_t)box * L * L + (size_t)j0 * L + j0, L, X, s_d, s_max, flag);
         float *wh = Wh + ((size_t)box * L + j0) * K2, *wl = Wl + ((size_t)box * L + j0) * K2;
         float *ph = Ph + (size_t)box * K2 * K2, *pl = Pl + (size_t)box * K2 * K2;
-        for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
-            const int c = e / NB, q = e % NB;
-            const c64 v = X[s_p[c] * DP + s_k[q]];
-            split2(wh, wl, (size_t)c * K2 + 2 * q, -v.x, -v.y);
-            const c64 u = X[s_p[q] * DP + s_k[c]];   // P[q][c]: rows 2c, 2c + 1 of the right operand, K index q
-            split2(ph, pl, (size_t)(2 * c) * K2 + 2 * q, u.x, -u.y);
-            split2(ph, pl, (size_t)(2 * c + 1) * K2 + 2 * q, u.y, u.x);
+        for (int e = tid; e < NB * NB / 2; e += DIAG_THREADS) {
+            const int c = e / (NB / 2), q = 2 * (e % (NB / 2));
+            const c64 v0 = X[c * DP + q], v1 = X[c * DP + q + 1];
+            split4(wh, wl, (size_t)c * K2 + 2 * q, -v0.x, -v0.y, -v1.x, -v1.y);
+            const c64 u0 = X[q * DP + c], u1 = X[(q + 1) * DP + c];   // P[q][c]: rows 2c, 2c + 1 of the right operand, K index q
+            split4(ph, pl, (size_t)(2 * c) * K2 + 2 * q, u0.x, -u0.y, u1.x, -u1.y);
+            split4(ph, pl, (size_t)(2 * c + 1) * K2 + 2 * q, u0.y, u0.x, u1.y, u1.x);
         }
         return;
     }
@@ -299,26 +384,33 @@ __global__ void __launch_bounds__(DIAG_THREADS) tgj_panel(const BoxInfo* __restr
             const int I0 = part * 32;
             if (I0 >= j0 && I0 < j0 + NB) continue;   // rows J: -P, from the block's CTA
             float *wh = Wh + ((size_t)box * L + I0) * K2, *wl = Wl + ((size_t)box * L + I0) * K2;
-            for (int e = tid; e < 32 * NB; e += DIAG_THREADS) {
-                const int I = e / NB, c = e % NB;
-                const c64 v = I0 + I < m ? A[(size_t)(I0 + I) * L + j0 + c] : mk<float>(0.f, 0.f);
-                split2(wh, wl, (size_t)I * K2 + 2 * c, v.x, v.y);
+#pragma unroll 4
+            for (int e = tid; e < 32 * NB / 2; e += DIAG_THREADS) {
+                const int I = e / (NB / 2), c = 2 * (e % (NB / 2));
+                const float4 v = I0 + I < m ? *reinterpret_cast<const float4*>(&A[(size_t)(I0 + I) * L + j0 + c])
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                split4(wh, wl, (size_t)I * K2 + 2 * c, v.x, v.y, v.z, v.w);
             }
         } else {
             const int jc = (part - t32) * 32;
             __syncthreads();
-            for (int e = tid; e < NB * 32; e += DIAG_THREADS) {
-                const int c = e / 32, jj = e % 32, j = jc + jj;
-                X[c * 33 + jj] = j >= j0 && j < j0 + NB ? mk<float>(c == j - j0 ? 1.f : 0.f, 0.f)
-                                                        : A[(size_t)(j0 + c) * L + j];
+#pragma unroll 4
+            for (int e = tid; e < NB * 16; e += DIAG_THREADS) {
+                const int c = e / 16, jj = 2 * (e % 16), j = jc + jj;
+                float4 v;
+                if (j >= j0 && j < j0 + NB) v = make_float4(c == j - j0 ? 1.f : 0.f, 0.f, c == j + 1 - j0 ? 1.f : 0.f, 0.f);
+                else v = *reinterpret_cast<const float4*>(&A[(size_t)(j0 + c) * L + j]);
+                X[c * 33 + jj] = mk<float>(v.x, v.y);
+                X[c * 33 + jj + 1] = mk<float>(v.z, v.w);
             }
             __syncthreads();
             float *bh = Bh + ((size_t)box * 2 * L + 2 * jc) * K2, *bl = Bl + ((size_t)box * 2 * L + 2 * jc) * K2;
-            for (int e = tid; e < 32 * NB; e += DIAG_THREADS) {
-                const int jj = e / NB, c = e % NB;
-                const c64 v = X[c * 33 + jj];
-                split2(bh, bl, (size_t)(2 * jj) * K2 + 2 * c, v.x, -v.y);
-                split2(bh, bl, (size_t)(2 * jj + 1) * K2 + 2 * c, v.y, v.x);
+#pragma unroll 2
+            for (int e = tid; e < 32 * NB / 2; e += DIAG_THREADS) {
+                const int jj = e / (NB / 2), c = 2 * (e % (NB / 2));
+                const c64 v = X[c * 33 + jj], w = X[(c + 1) * 33 + jj];
+                split4(bh, bl, (size_t)(2 * jj) * K2 + 2 * c, v.x, -v.y, w.x, -w.y);
+                split4(bh, bl, (size_t)(2 * jj + 1) * K2 + 2 * c, v.y, v.x, w.y, w.x);
             }
         }
     }
