@@ -20,7 +20,9 @@
 // more) the box takes a third step; |R0| > 1e-3, |R1| > 1e-4 or a third residual above 1e-9 sets the flag too.
 //
 // A product costs 30 (8 x 5 digits, 8 orders), 14, 8 or 6 BF16 MMAs; the matrices of a plane are read and written a few
-// times.  Bound: the tensor pipe for the 30- and 14-product steps, launches for small planes.
+// times.  Bound: the operands' loads (0.43 of the tensor pipe at 8 boxes of 676 unknowns: 30 products 814 us, 14 464 us, 8
+// 243 us; with 64-column tiles, half the instruction's rate, and four epilogue warps 1046, 593, 264 us), launches for
+// small planes.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>

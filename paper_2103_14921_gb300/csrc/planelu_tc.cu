@@ -150,7 +150,9 @@ __global__ void tgj_pad_diag(const BoxInfo* __restrict__ boxes, c64* __restrict_
 // column.  The transform W
 // then reaches the other columns in a rank-SB step of the other 16 warps, X <- [rows not used here] X + W X[pivot rows]: the
 // next sub-panel's columns first, so that the four warps eliminate it during the rest of the step.
-// Bound: the serial column chain, and the rank-SB steps (128^3 complex multiply-adds on one SM's FP32 lanes, 32 us).
+// Bound: the serial column chain (670 clocks a column by itself, 1,080 beside the rank steps: 17,300 of a sub-panel's
+// 22,000), and the rank-SB steps (128^3 complex multiply-adds on one SM's FP32 lanes, 32 us).  27 boxes: 103 us a panel
+// (chain and rank steps one after the other, X in shared memory: 123).
 constexpr int SB = 16;
 constexpr int SWP = SB + 2;           // row pitch of a sub-panel in shared memory
 constexpr int DIAG_SMEM = NB * DP * (int)sizeof(c64);

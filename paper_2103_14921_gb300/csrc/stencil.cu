@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(128) stencil_kernel(const cplx<T>* __restrict_
 // not per plane.  Ghost nodes are zero-filled by the copy.
 //
 // complex128 is bound by the FP64 pipe (two lanes per SM and clock): the form with the fewest FP64 operations is
-// taken wherever it holds, and plain axes are tested at run time in the product form too.  112^3 x 16: 2.9 ms
+// taken wherever it holds, and plain axes are tested at run time in the product form too.  112^3 x 16: 2.84 ms
 // (per-node kernel 5.1 ms), 87 % of the pipe while a block runs; 101 x 93 x 77 x 10: 1.30 (2.54) ms; 48^3 x 1: 0.11
 // (0.18) ms.  complex64 is bound by instruction latency at 12 warps per SM (issue 36 % active, DRAM a third of its
-// rate): 112^3 x 16 170 us (per-node 361), 160 x 160 x 80 x 128 with complex k^2 1.39 (5.07) ms, 101 x 93 x 77 x 10
-// 80 (169) us.  MN = 2 (more warps) measured 247, MN = 8 171 us at 112^3 x 16, so 4.
+// rate): 112^3 x 16 163 us (per-node 361), 160 x 160 x 80 x 128 with complex k^2 1.39 (5.07) ms, 101 x 93 x 77 x 10
+// 86 (168) us.  MN = 2 (more warps) measured 247, MN = 8 171 us at 112^3 x 16, so 4.
 struct PlainRange {
     int lo[3], hi[3];   // per axis: indices whose stretched coefficients are exactly (1, -2, 1)
 };
@@ -778,7 +778,7 @@ helm_status launch_any(helm_grid g, int prec, const void* u, const void* b, void
     bool done = false;
     // complex64 calls of fewer than 2^20 values run the per-node kernel: a walk's planes are a serial chain, and too
     // few blocks hide its latency (48^3 x 1: 27 us per call against 38; 64^3 x 4, 2^20 values: 44 against 40;
-    // 112^3 x 1: 76 against 69).  complex128 is FP64-bound at any size and always walks.
+    // 112^3 x 1: 77 against 74).  complex128 is FP64-bound at any size and always walks.
     const bool walk = g->ctx->stencil_march == 2 || g->ctx->stencil_planes || prec == HELM_PREC_FP64 ||
                       g->n * nrhs >= (1 << 20);
     if (g->ctx->stencil_march && !g->wtab && walk) {
