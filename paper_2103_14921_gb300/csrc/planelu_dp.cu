@@ -500,6 +500,8 @@ void launch_gemm_n(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const C
 template <int SA, int SB, int O, bool ADD>
 void launch_gemm(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const int* ea, const BoxInfo* dbox, int nbox, int m_max,
                  c128* out, float limit, int k, int* flag, int* stat = nullptr, const int* gate = nullptr) {
+    // 128-column tiles once every SM has one: 8 boxes of 676 unknowns (528 tiles) 814 us with 30 products against 1046;
+    // small coarse boxes (fewer tiles than SMs) 37 us, with 64 columns, twice the CTAs and all orders in one pass, 27
     const long long tiles = (long long)((2 * m_max + 127) / 128) * ((m_max + GM - 1) / GM) * nbox;
     if (tiles > ctx->sm_count)
         launch_gemm_n<SA, SB, O, ADD, 128>(ctx, D, mA, D.mB128, ea, dbox, nbox, m_max, out, limit, k, flag, stat, gate);
