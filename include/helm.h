@@ -125,8 +125,8 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * bit-identical results.  HELM_TUNE_STENCIL_MARCH: 1 (default) applies stencils with constant weights by
  * walking z-planes (the in-plane terms of a plane are formed once and reused by the three output planes it
  * touches; warps wholly inside the interior take class-sum forms, the others the product form), except
- * complex64 calls of fewer than 2^20 values; 2 the same at every size; 0 uses the per-node kernel.  All agree to
- * FP32 rounding.  Returns HELM_EINVAL for an unknown key or value out of range. */
+ * complex64 calls of fewer than 2^20 values and complex128 calls of fewer than 40,000 nodes and 90,000 values; 2 the
+ * same at every size; 0 uses the per-node kernel.  All agree to FP32 rounding.  Returns HELM_EINVAL for an unknown key or value out of range. */
 #define HELM_TUNE_TC_STAGES 1
 #define HELM_TUNE_COARSE_COOP 2
 #define HELM_TUNE_GRAPHS 3

@@ -778,9 +778,11 @@ helm_status launch_any(helm_grid g, int prec, const void* u, const void* b, void
     bool done = false;
     // complex64 calls of fewer than 2^20 values run the per-node kernel: a walk's planes are a serial chain, and too
     // few blocks hide its latency (48^3 x 1: 27 us per call against 38; 64^3 x 4, 2^20 values: 44 against 40;
-    // 112^3 x 1: 77 against 74).  complex128 is FP64-bound at any size and always walks.
-    const bool walk = g->ctx->stencil_march == 2 || g->ctx->stencil_planes || prec == HELM_PREC_FP64 ||
-                      g->n * nrhs >= (1 << 20);
+    // 112^3 x 1: 77 against 74).  complex128 is FP64-bound sooner, and the per-node kernel
+    // forms its coefficients per node: below 40,000 nodes and 90,000 values (per-node against walk, us: 30 x 33 x 29 x 1 66,
+    // 106; 33 x 40 x 25 x 2 96, 106; 36^3 x 1 118, 107; 40^3 x 1 136, 106; 32^3 x 3 123, 103).
+    const bool walk = g->ctx->stencil_march == 2 || g->ctx->stencil_planes ||
+                      (prec == HELM_PREC_FP64 ? g->n >= 40000 || g->n * nrhs >= 90000 : g->n * nrhs >= (1 << 20));
     if (g->ctx->stencil_march && !g->wtab && walk) {
         if (prec == HELM_PREC_FP64) done = (al & 15) == 0 && launch_march<double2, SUB>(g, u, b, y, nrhs, s);
         else if (nrhs % 2 == 0 && (al & 15) == 0) done = launch_march<float4, SUB>(g, u, b, y, nrhs / 2, s);
