@@ -314,6 +314,13 @@ struct TcCfg {
     static constexpr int THREADS = NPAD >= 256 ? 512 : 256;
     static constexpr uint32_t TCOLS = NPAD <= 32 ? 32 : (NPAD <= 64 ? 64 : (NPAD <= 128 ? 128 : 256));
     static constexpr int SMEM = STAGES * STAGE + (2 * STAGES + 1) * 8 + 16 + 1024;
+    // Bytes the stages hold when a tile's output passes through them, and what np column pairs of it take (128 rows, the
+    // pairs rounded up to the swizzle's 8).
+    static constexpr int RING = STAGES * STAGE;
+    __host__ __device__ static constexpr int out_bytes(int np) { return TC_BM * ((np + 7) / 8 * 8) * 16; }
+    // Every column count of the width fits, but for two stages of N = 256 (96 KB against 128 KB at 98 and more columns): there
+    // the rows go straight from TMEM to memory.
+    static_assert(out_bytes(NPAD / 4) <= RING || (NPAD == 256 && NST == 2), "a tile's output against the stages");
 };
 
 // Position of a CTA in its operand ring: chunks issued so far (stage = g mod NST, phase = g / NST)
@@ -449,12 +456,13 @@ __device__ __forceinline__ void gemm_core(const CUtensorMap* mapA, const CUtenso
             const uint32_t gi = R.g + kc;
             tc::mbar_drain(&full[gi % NST], (gi / NST) & 1);
         }
-    if ((nrhs & 1) == 0) {
+    if ((nrhs & 1) == 0 && Cfg::out_bytes(nrhs >> 1) <= Cfg::RING) {
         // The tile's output is one contiguous block of loc (rows row0.., all columns).  The accumulator passes through the
         // stages' shared memory (every load of this tile has been consumed) as column pairs, the pair index XORed with
         // the row so that the 8 rows of a store phase fall in different banks; the block is then read and written in
         // 16-byte vectors along memory, four in flight per thread.  (Rows straight from TMEM took an 8-byte access per
-        // column and 32 lines per warp access: at 128 columns more than half of a tile's time.)
+        // column and 32 lines per warp access: at 128 columns more than half of a tile's time.  Odd column counts, and blocks
+        // that do not fit in the stages, take them so.)
         const int npair = nrhs >> 1, np8 = (npair + 7) & ~7;
         float4* ep = reinterpret_cast<float4*>(base);
         if (ok) {
