@@ -372,6 +372,9 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
 // (16 or more) basis loads in flight per thread, and the template widths follow ni in steps of four vectors.  112^3 x
 // 16: 5.1 - 5.8 TB/s, where the wide kernel (one block per SM, widths 16 and 32) ran at 3.2 - 4.7 (17 vectors: 1084 -> 671
 // us, 24: 1167 -> 809); at 5 to 8 vectors the wide kernel is the faster one (8: 348 us against 407).
+// Shared memory: 16 KB for the reductions and the ni nrhs coefficients, together at most the 48 KB of a launch without opt-in.
+constexpr int UDS_SLOTS = RED_THREADS / 2, UDS_QG = 4;
+constexpr size_t UDS_STATIC = (size_t)UDS_QG * 2 * UDS_SLOTS * sizeof(c128);
 template <typename T, int IMH, int EPT>
 __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T>* __restrict__ V, long long vstride,
                                                                    cplx<T>* __restrict__ w, long long n_el, int nrhs, int ni,
@@ -380,9 +383,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
                                                                    double* __restrict__ npart) {
     extern __shared__ __align__(16) unsigned char uds_smem[];
     cplx<T>* hs = reinterpret_cast<cplx<T>*>(uds_smem);   // [ni][nrhs]
-    constexpr int SLOTS = RED_THREADS / 2, QG = 4;
+    constexpr int SLOTS = UDS_SLOTS, QG = UDS_QG;
+    static_assert(UDS_STATIC + 2 * IMH * SLOTS * sizeof(cplx<T>) <= 48 * 1024, "2 IMH vectors of SLOTS columns");
     __shared__ c128 s[QG][2][SLOTS];
-    __shared__ double sn[SLOTS];
     const int lane = threadIdx.x & 31, z = lane >> 4, slot = (threadIdx.x >> 5) * 16 + (lane & 15);
     const long long t = (long long)blockIdx.x * SLOTS + slot, stride = (long long)gridDim.x * SLOTS;
     const int r = (int)(t % nrhs);
@@ -427,7 +430,6 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
             }
         }
     }
-    if (z == 0) sn[slot] = nrm.value();
     const int nr = min(nrhs, SLOTS);
 #pragma unroll
     for (int i0 = 0; i0 < IMH; i0 += QG) {
@@ -446,6 +448,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
             partial[((long long)blockIdx.x * ldp + 2 * i0 + q) * nrhs + rr] = sum;
         }
     }
+    __syncthreads();
+    double* sn = reinterpret_cast<double*>(&s[0][0][0]);   // [SLOTS]
+    if (z == 0) sn[slot] = nrm.value();
     __syncthreads();
     if (threadIdx.x < nr) {
         double sum = 0.0;
@@ -838,7 +843,7 @@ struct CgsBuffers {
 };
 
 // Bases the fused CGS2 takes: up to 32 vectors (complex128: 16, the register budget of its kernels), coefficients
-// within 40 KB of shared memory.
+// within 40 KB of shared memory (32 KB in the split form, which takes at most 128 columns).
 template <typename T>
 inline bool cgs2_fits(int ni, int S) {
     return ni <= (sizeof(T) == 4 ? 32 : 16) && (size_t)ni * S * sizeof(cplx<T>) <= 40 * 1024;
