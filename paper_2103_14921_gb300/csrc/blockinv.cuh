@@ -1,18 +1,19 @@
 // In-place inverse of an NB x NB complex block held in shared memory, for the panel step of the block-pivot
-// Gauss-Jordan factorisations (planelu.cu, planelu_tc.cu): Gauss-Jordan with partial pivoting inside the
+// Gauss-Jordan factorisations on the CUDA cores (planelu.cu): Gauss-Jordan with partial pivoting inside the
 // block, in sub-panels of SB columns.  Within a sub-panel each column is eliminated on the sub-panel's
 // columns only (whole rows are swapped at once); the accumulated transform W of the sub-panel then reaches
 // the other columns B in one rank-SB step, B <- [rows outside the sub-panel] B + W[:, sub] B[sub rows, :]
 // (the rows of B it reads are copied out first), so the per-column work is NB x SB instead of NB x NB.
 // On return X holds the inverse of the row-permuted block; the caller undoes the permutation (s_perm: the
 // pivot row chosen at each column).  flag bit 0: a zero pivot (replaced by 1 to stay finite); bit 1: a pivot
-// below 1e-6 of the block's largest entry (amax is the largest |x|^2 of the block).
+// below 1e-6 of the block's largest entry (amax is the largest |x|^2 of its first nr rows and columns; the rest is an
+// identity that pads a partial panel, whose pivots are not tested).
 #pragma once
 #include "internal.h"
 
 template <typename T, int NB, int DP, int SB, int NT>
 __device__ __forceinline__ void block_inverse(cplx<T>* X, cplx<T>* Brow, int* s_perm, cplx<T>* s_row, cplx<T>* s_col,
-                                              int* s_piv, T amax, int* flag) {
+                                              int* s_piv, T amax, int nr, int* flag) {
     static_assert(NB % SB == 0 && NT % 32 == 0 && NT >= NB, "block_inverse: shape");
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     for (int c0 = 0; c0 < NB; c0 += SB) {
@@ -35,7 +36,7 @@ __device__ __forceinline__ void block_inverse(cplx<T>* X, cplx<T>* Brow, int* s_
                     if (!(best > (T)0) || bi >= NB) {
                         atomicOr(flag, 1);
                         bi = c;
-                    } else if (best < (T)1e-12 * amax) {
+                    } else if (c < nr && best < (T)1e-12 * amax) {
                         atomicOr(flag, 2);
                     }
                     *s_piv = bi;

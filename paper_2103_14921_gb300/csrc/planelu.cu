@@ -752,9 +752,11 @@ __global__ void __launch_bounds__(512) bgj_diag(const BoxInfo* __restrict__ boxe
     for (int e = tid; e < NB * NB; e += 512) {
         const int r = e / NB, c = e % NB;
         cplx<T> v = mk<T>(r == c ? (T)1 : (T)0, (T)0);   // identity beyond a partial panel
-        if (r < nbw && c < nbw) v = A[(size_t)(j0 + r) * m + j0 + c];
+        if (r < nbw && c < nbw) {
+            v = A[(size_t)(j0 + r) * m + j0 + c];
+            amax = max(amax, v.x * v.x + v.y * v.y);
+        }
         X[r * DP + c] = v;
-        amax = max(amax, v.x * v.x + v.y * v.y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, o));
@@ -762,7 +764,7 @@ __global__ void __launch_bounds__(512) bgj_diag(const BoxInfo* __restrict__ boxe
     __syncthreads();
     amax = 0;
     for (int w = 0; w < 16; ++w) amax = max(amax, s_wmax[w]);
-    block_inverse<T, NB, DP, 16, 512>(X, X + NB * DP, s_perm, s_row, s_col, &s_piv, amax, flag);
+    block_inverse<T, NB, DP, 16, 512>(X, X + NB * DP, s_perm, s_row, s_col, &s_piv, amax, nbw, flag);
     if (tid == 0) {
         for (int j = 0; j < NB; ++j) s_pos[j] = j;
         for (int c = NB - 1; c >= 0; --c) {

@@ -12,8 +12,8 @@
 // A[I,J] P (one row of tiles) waits for the block inverse, and it runs on the tensor cores too; R is a copy.
 // Pivoting stays inside each diagonal block: for these Helmholtz Schur complements (condition numbers
 // 1e0-1e2 at the workload sizes) block pivots give the same accuracy as full partial pivoting, and a block
-// pivot below 1e-6 of its block's largest entry is reported so that the caller can fall back to the
-// fully pivoted CUDA-core elimination.
+// pivot below 1e-6 of its block's largest entry (the rows and columns below m, so that the bar has the matrix's own
+// scale) is reported so that the caller can fall back to an elimination on the CUDA cores.
 //
 // The product W R (m x NB times NB x m, complex; W = A[I,J] P is the same with N = 2 NB) is one real GEMM with the 2x2 embedding used by the plane
 // sweeps: A operand = rows of W read as 2 NB reals (K-major), B operand = B^T[2j][2c] = Re R[c][j],
@@ -165,8 +165,9 @@ struct DiagShared {
 };
 
 // One sub-panel, columns c0 .. c0 + SB - 1 of the block, by 128 threads: Wr is the row'th row.  The columns rotate through
-// the registers, so that the loop stays rolled: sixteen copies of its body ran at the speed of instruction fetch.
-__device__ __forceinline__ void diag_columns(c64* Wr, DiagShared& D, bool& used, int row, int c0, float amax, int* flag) {
+// the registers, so that the loop stays rolled: sixteen copies of its body ran at the speed of instruction fetch.  bar: the
+// least |pivot|^2 of the row that is not weak.
+__device__ __forceinline__ void diag_columns(c64* Wr, DiagShared& D, bool& used, int row, int c0, float bar, int* flag) {
     const int lane = row & 31, wid = row >> 5;
     c64 a[SB];
 #pragma unroll
@@ -208,7 +209,7 @@ __device__ __forceinline__ void diag_columns(c64* Wr, DiagShared& D, bool& used,
         const bool piv = row == p;
         if (piv) {
             if (!(q > 0.f)) atomicOr(flag, 1);
-            else if (q < 1e-12f * amax) atomicOr(flag, 2);
+            else if (q < bar) atomicOr(flag, 2);
             used = true;
             D.p[c0 + j] = row;
             D.k[row] = c0 + j;
@@ -258,8 +259,9 @@ __device__ __forceinline__ void diag_step(c64 (&x)[4][8], const c64* W, const c6
     }
 }
 
-// the inverse P of the 128 x 128 block at A (pitch L) into X (pitch DP)
-__device__ __forceinline__ void diag_inverse(const c64* __restrict__ A, int L, c64* X, DiagShared& D, float* s_max, int* flag) {
+// the inverse P of the 128 x 128 block at A (pitch L) into X (pitch DP); rows and columns from nr on are padding
+__device__ __forceinline__ void diag_inverse(const c64* __restrict__ A, int L, int nr, c64* X, DiagShared& D, float* s_max,
+                                             int* flag) {
     constexpr int RT = DIAG_THREADS - NB;   // threads of the rank steps
     const int tid = threadIdx.x;
     c64* const Wb = X;                    // [2][NB][SWP]
@@ -271,11 +273,13 @@ __device__ __forceinline__ void diag_inverse(const c64* __restrict__ A, int L, c
         tc::named_bar(2, DIAG_THREADS);
         float amax = 0.f;
         for (int w = 0; w < RT / 32; ++w) amax = fmaxf(amax, s_max[w]);
-        diag_columns(Wb + row * SWP, D, used, row, 0, amax, flag);
+        // a row of the padding (pivot 1) is never weak; a |pivot|^2 below the normal range has no reciprocal
+        const float bar = row < nr ? fmaxf(1e-12f * amax, 1.1754944e-38f) : 0.f;
+        diag_columns(Wb + row * SWP, D, used, row, 0, bar, flag);
 #pragma unroll 1
         for (int s = 0; s < NB / SB; ++s) {
             for (int i = 0; i < 3; ++i) tc::named_bar(2, DIAG_THREADS);
-            if (s + 1 < NB / SB) diag_columns(Wb + (((s + 1) & 1) * NB + row) * SWP, D, used, row, (s + 1) * SB, amax, flag);
+            if (s + 1 < NB / SB) diag_columns(Wb + (((s + 1) & 1) * NB + row) * SWP, D, used, row, (s + 1) * SB, bar, flag);
         }
         tc::named_bar(2, DIAG_THREADS);
         __syncthreads();
@@ -291,7 +295,8 @@ __device__ __forceinline__ void diag_inverse(const c64* __restrict__ A, int L, c
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) amax = fmaxf(amax, x[r][i].x * x[r][i].x + x[r][i].y * x[r][i].y);
+        for (int i = 0; i < 8; ++i)
+            if (4 * rg + r < nr) amax = fmaxf(amax, x[r][i].x * x[r][i].x + x[r][i].y * x[r][i].y);
     amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));   // non-negative: ordered like the bits
     if ((tid & 31) == 0) s_max[tid >> 5] = amax;
 #pragma unroll
@@ -363,7 +368,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) tgj_panel(const BoxInfo* __restr
         const int box = blockIdx.x;
         const int m = boxes[box].m;
         if (k >= boxes[box].dims[2] || j0 >= m) return;
-        diag_inverse(S + (size_t)box * L * L + (size_t)j0 * L + j0, L, X, s_d, s_max, flag);
+        diag_inverse(S + (size_t)box * L * L + (size_t)j0 * L + j0, L, min(NB, m - j0), X, s_d, s_max, flag);
         float *wh = Wh + ((size_t)box * L + j0) * K2, *wl = Wl + ((size_t)box * L + j0) * K2;
         float *ph = Ph + (size_t)box * K2 * K2, *pl = Pl + (size_t)box * K2 * K2;
         for (int e = tid; e < NB * NB / 2; e += DIAG_THREADS) {
