@@ -425,9 +425,13 @@ __global__ void __launch_bounds__(320, 1) dp_gemm(const __grid_constant__ CUtens
             dp_consume<PL, TWO ? 4 : 0, O, GN>(p, tmem, nK);
             if (TWO) {
                 if (p.ok) p.ok = tc::mbar_wait(p.drained, 0, p.err, 36);
+                if (!p.ok) tc::mbar_drain(p.done, 0);   // the first pass's products, before the barrier's next phase
                 tc::fence_after_sync();
                 dp_consume<PH, 0, 4, GN>(p, tmem, nK);
             }
+            // every product issued has completed before this warp meets the CTA's barrier and frees TMEM: an epilogue warp
+            // that gave up on the first pass does not wait for the second
+            tc::mbar_drain(p.done, TWO ? 1 : 0);
         }
     } else {
         const int q = warp & 3, I = row0 + q * 32 + lane, cb = (warp - 2) / 4 * (GN / 2);
