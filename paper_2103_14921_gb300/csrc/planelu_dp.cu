@@ -25,7 +25,6 @@
 // small planes.
 #include <cuda.h>
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
 
 #include <atomic>
 
@@ -470,14 +469,7 @@ __global__ void __launch_bounds__(320, 1) dp_gemm(const __grid_constant__ CUtens
 
 // bf16 [z][rows][cols] with row pitch Kp, boxes of 64 x box_rows, 128-byte swizzle
 bool encode_slices(CUtensorMap* map, void* base, uint64_t cols, uint64_t rows, uint64_t z, uint64_t Kp, uint32_t box_rows) {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
+    const PFN_cuTensorMapEncodeTiled_v12000 fn = tc::tensor_map_encoder();
     if (!fn) return false;
     cuuint64_t dims[3] = {cols, rows, z};
     cuuint64_t strides[2] = {Kp * 2, Kp * 2 * rows};

@@ -26,7 +26,6 @@
 // columns beyond the box's m, written once and never touched again, so the block inverse of a partial last
 // panel is that of block-diag(S_JJ, I) and the padding contributes nothing to rows and columns below m.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <atomic>
 
@@ -653,22 +652,9 @@ __global__ void tgj_store(const BoxInfo* __restrict__ boxes, const c64* __restri
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn_f() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
 // the work matrices S as fp32 [nb][L][2L], boxes of 32 floats x 128 rows, 128-byte swizzle (epilogue stores)
 bool encode_matrix(CUtensorMap* map, void* base, uint64_t L, uint64_t nb) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn_f();
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tc::tensor_map_encoder();
     if (!enc) return false;
     cuuint64_t dims[3] = {2 * L, L, nb};
     cuuint64_t strides[2] = {2 * L * 4, 2 * L * 4 * L};
@@ -681,7 +667,7 @@ bool encode_matrix(CUtensorMap* map, void* base, uint64_t L, uint64_t nb) {
 
 // fp32 [nb][rows][K2] operand, boxes of 32 x box_rows, 128-byte swizzle
 bool encode_operand(CUtensorMap* map, void* base, uint64_t rows, uint64_t nb, uint32_t box_rows) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn_f();
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tc::tensor_map_encoder();
     if (!enc) return false;
     cuuint64_t dims[3] = {(cuuint64_t)K2, rows, nb};
     cuuint64_t strides[2] = {(cuuint64_t)K2 * 4, (cuuint64_t)K2 * 4 * rows};

@@ -23,7 +23,6 @@
 // TMEM (thread t <-> row t) and write y_k (FWD) or x_k = y_k - D (BWD).
 #include <cuda.h>
 #include <cuda_bf16.h>
-#include <cudaTypedefs.h>
 
 #include <atomic>
 #include <vector>
@@ -712,24 +711,9 @@ __global__ void __launch_bounds__(TcCfg<E, NPAD, NST>::THREADS, TcCfg<E, NPAD, N
     gemm_teardown<E, NPAD, NST>(tmem);
 }
 
-// cuTensorMapEncodeTiled from the driver, looked up through the runtime so that the
-// library itself does not link against libcuda (it still loads on machines without a driver).
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
 bool encode_3d(CUtensorMap* map, void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1, uint64_t s2,
                uint32_t b0, uint32_t b1, bool bf16) {
-    PFN_cuTensorMapEncodeTiled_v12000 cuTensorMapEncodeTiled = encode_fn();
+    PFN_cuTensorMapEncodeTiled_v12000 cuTensorMapEncodeTiled = tc::tensor_map_encoder();
     if (!cuTensorMapEncodeTiled) return false;
     cuuint64_t dims[3] = {d0, d1, d2};
     cuuint64_t strides[2] = {s1, s2};   // bytes

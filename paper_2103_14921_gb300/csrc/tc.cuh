@@ -4,9 +4,30 @@
 // and reports failure to the caller, which then skips its remaining work.
 #pragma once
 #include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace tc {
+
+// cuTensorMapEncodeTiled from the driver, looked up through the runtime so that the library itself does not link against
+// libcuda (it still loads on machines without a driver); null where there is none.  Called by several host threads.
+inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};
+    PFN_cuTensorMapEncodeTiled_v12000 f = fn.load(std::memory_order_acquire);
+    if (!f) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess) {
+            f = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+            fn.store(f, std::memory_order_release);
+        }
+    }
+    return f;
+}
 
 // ~2^24 polls with back-off (about a second on a GB300) before a wait gives up.
 constexpr uint32_t WAIT_LIMIT = 1u << 24;
