@@ -154,6 +154,14 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * SM), falling back to full partial pivoting after a tiny block pivot.  0: always the fully pivoted elimination.  Read by
  * oras_factor. */
 #define HELM_TUNE_BLOCK_GJ 8
+/* How often oras_factor (of this context, its frequency sweeps and its serving loop) factored a plane set again by another
+ * method: counts[HELM_FALLBACK_PIVOT] after a zero or tiny block pivot, [HELM_FALLBACK_ACCURACY] because an FP64 inverse did not
+ * come out to FP64 by Newton steps, [HELM_FALLBACK_ROOM] because their workspace did not fit (the set was then factored by
+ * HELM_TUNE_BLOCK_GJ 1 at once). */
+#define HELM_FALLBACK_PIVOT 0
+#define HELM_FALLBACK_ACCURACY 1
+#define HELM_FALLBACK_ROOM 2
+helm_status helm_factor_fallbacks(helm_ctx ctx, uint64_t counts[3]);
 /* HELM_TUNE_STENCIL_PLANES: output planes per block of the z-marching stencil (HELM_TUNE_STENCIL_MARCH), at
  * any size of the call; 0 (default) picks the block shape and the planes per grid from an estimate of the
  * blocks' time; else 4..128.  The split decides which warps lie wholly inside the interior (and take the

@@ -94,6 +94,12 @@ extern "C" const char* helm_last_error(helm_ctx ctx) {
 
 extern "C" size_t helm_bytes_in_use(helm_ctx ctx) { return ctx ? ctx->in_use : 0; }
 
+extern "C" helm_status helm_factor_fallbacks(helm_ctx ctx, uint64_t counts[3]) {
+    if (!ctx || !counts) return HELM_EINVAL;
+    for (int i = 0; i < 3; ++i) counts[i] = ctx->fallbacks[i].load();
+    return HELM_OK;
+}
+
 extern "C" helm_status helm_set_tuning(helm_ctx ctx, int key, int value) {
     if (!ctx) return HELM_EINVAL;
     if (key == HELM_TUNE_TC_STAGES) {

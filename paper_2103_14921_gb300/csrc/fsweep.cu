@@ -92,6 +92,7 @@ extern "C" helm_status helm_frequency_sweep(helm_ctx ctx, const helm_sweep_desc*
             cudaStreamDestroy(st2);
             return set_error(ctx, rc, "helm_frequency_sweep: second context: %s", helm_last_error(nullptr));
         }
+        ctx2->count_in = ctx;
         ctx2->tc_stages = ctx->tc_stages;
         ctx2->coarse_coop = ctx->coarse_coop;
         ctx2->use_graphs = ctx->use_graphs;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <algorithm>
+#include <atomic>
 #include <memory>
 #include <string>
 #include <vector>
@@ -80,7 +81,9 @@ struct helm_ctx_s {
     int tc_factor = 1;         // tuning: tensor-core blocked Gauss-Jordan for complex64 tensor-core factor sets
     int block_gj = 2;          // tuning: the other factor sets: 1 block-pivot Gauss-Jordan on the CUDA cores, 2 the same
                                // for complex64, tensor-core inverses with Newton steps for complex128
-    uint64_t factor_fallbacks = 0;   // sets refactored with full pivoting after a tiny block pivot
+    std::atomic<uint64_t> fallbacks[3] = {};   // plane sets factored again by another method (HELM_FALLBACK_*)
+    helm_ctx_s* count_in = nullptr;            // the context that counts them instead (a builder's: its caller's)
+    void count_fallback(int why) { (count_in ? count_in : this)->fallbacks[why]++; }
     uint64_t graph_gen = 1;    // bumped when a setting that captured graphs depend on changes
     cudaStream_t cap_stream = nullptr;   // private stream graphs are captured on (the context's may be
                                          // the legacy default stream, which cannot be captured)

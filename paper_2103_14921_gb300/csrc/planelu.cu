@@ -1007,7 +1007,7 @@ helm_status factor_block_t(helm_ctx ctx, PlaneSet& P, int* singular, int* weak) 
 
 // complex128 set from complex64 inverses and Newton steps on the tensor cores (planelu_dp.cu), a batch of boxes at a
 // time so that the workspace stays within 4 GB.  *ok = false: no room, a tiny pivot or a plane that did not come out to
-// FP64 (the caller then eliminates in FP64).
+// FP64 (counted; the caller then eliminates in FP64) or planes too large.  Other failures are the call's.
 helm_status factor_newton(helm_ctx ctx, PlaneSet& P, bool* ok) {
     *ok = false;
     cudaStream_t st = ctx->stream;
@@ -1026,17 +1026,20 @@ helm_status factor_newton(helm_ctx ctx, PlaneSet& P, bool* ok) {
         dp_free(ctx, D);
         tgj_free(ctx, T);
     };
-    if (tgj_alloc(ctx, batch, m, T) || dp_alloc(ctx, batch, m, D) ||
-        dev_alloc(ctx, (void**)&S, (size_t)batch * mm * sizeof(c128), "factor work S") ||
-        dev_alloc(ctx, (void**)&Tm, (size_t)batch * mm * sizeof(c128), "factor work T")) {
+    const std::string before = ctx->last_error;
+    helm_status rc;
+    if ((rc = tgj_alloc(ctx, batch, m, T)) || (rc = dp_alloc(ctx, batch, m, D)) ||
+        (rc = dev_alloc(ctx, (void**)&S, (size_t)batch * mm * sizeof(c128), "factor work S")) ||
+        (rc = dev_alloc(ctx, (void**)&Tm, (size_t)batch * mm * sizeof(c128), "factor work T"))) {
         cleanup();
-        ctx->last_error.clear();   // not an error of the caller's: the general elimination needs less room
+        if (rc != HELM_ENOMEM) return rc;
+        ctx->last_error = before;   // not an error of the caller's: the general elimination needs less room
+        ctx->count_fallback(HELM_FALLBACK_ROOM);
         return HELM_OK;
     }
     const c128* coef = (const c128*)P.coef;
     c128* G = (c128*)P.G;
     int hflag[2] = {0, 0};
-    helm_status rc = HELM_OK;
     for (int b0 = 0; b0 < P.nbox && rc == HELM_OK && !hflag[0] && !hflag[1]; b0 += batch) {
         const int nb = std::min(batch, P.nbox - b0);
         const BoxInfo* dbox = P.dbox + b0;
@@ -1074,6 +1077,7 @@ helm_status factor_newton(helm_ctx ctx, PlaneSet& P, bool* ok) {
     if (rc) return rc;
     if (hflag[1]) return set_error(ctx, HELM_ETIMEOUT, "plane factorisation: a bounded wait gave up");
     *ok = hflag[0] == 0;
+    if (!*ok) ctx->count_fallback(hflag[0] & 3 ? HELM_FALLBACK_PIVOT : HELM_FALLBACK_ACCURACY);
     return HELM_OK;
 }
 
@@ -1235,7 +1239,7 @@ helm_status planeset_factor(helm_ctx ctx, PlaneSet& P, int* singular) {
     if (P.prec == HELM_PREC_FP32 && P.padded && ctx->tc_factor) {
         HELM_TRY(planeset_factor_tc(ctx, P, singular, &weak));
         if (!weak && !*singular) return HELM_OK;
-        ctx->factor_fallbacks++;   // a tiny (or zero) block pivot: factor the set again with full partial pivoting
+        ctx->count_fallback(HELM_FALLBACK_PIVOT);   // a tiny (or zero) block pivot: again, with full partial pivoting
     } else if (!P.padded && ctx->block_gj) {
         if (P.prec == HELM_PREC_FP64 && ctx->block_gj == 2) {
             bool ok = false;
@@ -1248,7 +1252,7 @@ helm_status planeset_factor(helm_ctx ctx, PlaneSet& P, int* singular) {
         if (P.prec == HELM_PREC_FP64) HELM_TRY(factor_block_t<double>(ctx, P, singular, &weak));
         else HELM_TRY(factor_block_t<float>(ctx, P, singular, &weak));
         if (!weak && !*singular) return HELM_OK;
-        ctx->factor_fallbacks++;
+        ctx->count_fallback(HELM_FALLBACK_PIVOT);
     }
     if (P.prec == HELM_PREC_FP64) return factor_t<double>(ctx, P, singular);
     return factor_t<float>(ctx, P, singular);

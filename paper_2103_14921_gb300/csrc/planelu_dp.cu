@@ -50,7 +50,7 @@ __device__ __forceinline__ double pow2(int e) {
 __device__ __forceinline__ int exponent_of(uint32_t hi, int* flag) {
     const int E = (int)(hi >> 20);
     if (E == 0) return 0;
-    if (E >= 1923 || E <= 123) atomicOr(flag, 2);
+    if (E >= 1923 || E <= 123) atomicOr(flag, 4);
     return E - 1022;
 }
 __device__ __forceinline__ uint32_t high_word(double x) { return (uint32_t)(__double_as_longlong(x) >> 32) & 0x7FFFFFFFu; }
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(320, 1) dp_gemm(const __grid_constant__ CUtens
             if (ok) dp_epilogue<0, 4, GN, ADD, true, false>(tm, cb, n0, I, m, er, ebb, row, bad, big);
         }
         const float f = (float)__hiloint2double((int)big, 0);
-        if (ok && (bad || (!ADD && !(f <= limit)))) atomicOr(flag, 2);
+        if (ok && (bad || (!ADD && !(f <= limit)))) atomicOr(flag, 4);
         if (ok && !ADD && stat) {   // the largest entry (non-negative floats compare like their bits)
             const int b = __reduce_max_sync(0xffffffffu, __float_as_int(f));
             if (lane == 0) atomicMax(stat + box, b);

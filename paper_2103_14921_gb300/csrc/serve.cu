@@ -645,6 +645,7 @@ extern "C" helm_status helm_serve_start(helm_ctx ctx, int slots) {
         return set_error(ctx, rc, "helm_serve_start: builder context");
     }
     for (helm_ctx b : sv->bctxs) {
+        b->count_in = ctx;
         b->tc_stages = ctx->tc_stages;
         b->coarse_coop = ctx->coarse_coop;
         b->use_graphs = ctx->use_graphs;

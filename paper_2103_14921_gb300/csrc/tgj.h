@@ -9,7 +9,7 @@ struct TgjWork {
     int nb = 0, L = 0;                       // boxes; pitch of the work matrices (m_max rounded up to 128)
     size_t s_bytes = 0, w_bytes = 0, b_bytes = 0, p_bytes = 0;
     void *S = nullptr, *Wh = nullptr, *Wl = nullptr, *Bh = nullptr, *Bl = nullptr, *Ph = nullptr, *Pl = nullptr;
-    int* flag = nullptr;                     // [0] pivots (bit 0 zero, bit 1 tiny), [1] bounded waits
+    int* flag = nullptr;                     // [0] pivots (bit 0 zero, bit 1 tiny) and bit 2 of dp_invert, [1] bounded waits
     CUtensorMap mWh, mWl, mBh, mBl, mPh, mPl, mS;
 };
 
@@ -33,6 +33,6 @@ size_t dp_bytes(int nb, int m_max);
 helm_status dp_alloc(helm_ctx ctx, int nb, int m_max, DpWork& W);
 void dp_free(helm_ctx ctx, DpWork& W);
 // G_k <- S^{-1} (FP64) of plane k of the boxes: S is [nbox][m_max^2] with pitch m, R a scratch of the same size, G the
-// factor storage.  flag bit 1 is set when the result is not good to FP64 (the caller then eliminates in FP64).
+// factor storage.  flag bit 2 is set when the result is not good to FP64 (the caller then eliminates in FP64).
 void dp_invert(helm_ctx ctx, const TgjWork& T, const DpWork& D, const BoxInfo* dbox, const BoxInfo* hbox, int nbox, int m_max,
                int k, const c128* S, c128* R, c128* G);

@@ -98,6 +98,7 @@ def lib():
         "helm_last_error": (C.c_char_p, [vp]),
         "helm_bytes_in_use": (C.c_size_t, [vp]),
         "helm_launch_count": (C.c_uint64, [vp]),
+        "helm_factor_fallbacks": (st, [vp, C.POINTER(C.c_uint64)]),
         "helm_profile_enable": (st, [vp, i32]),
         "helm_set_tuning": (st, [vp, i32, i32]),
         "helm_profile_select": (st, [vp, C.c_char_p]),
@@ -177,6 +178,13 @@ class Context:
     @property
     def launches(self):
         return lib().helm_launch_count(self._h)
+
+    @property
+    def factor_fallbacks(self):
+        """Plane sets factored again by another method: ``{"pivot", "accuracy", "room"}`` counts."""
+        n = (C.c_uint64 * 3)()
+        self.check(lib().helm_factor_fallbacks(self._h, n), "helm_factor_fallbacks")
+        return dict(zip(("pivot", "accuracy", "room"), n))
 
     def set_tuning(self, key, value):
         """``helm_set_tuning`` (e.g. ``TUNE_TC_STAGES``)."""
