@@ -16,10 +16,12 @@
 // digits of S (2^-40), X1 = X0 + X0 R0 cut to 5 digits, R1 = I - S X1 with all 8 digits of S (64 bits below its row's largest
 // entry) and the orders 0..7, X = X1 + X1 R1.  The error left is |R1|^2 and R1's own, of which the orders left out are the
 // larger part: sums of about 2^19 at 2^-64 of the scale 2^14, 2^-59 of |S| |X| (with 7 digits and orders: 2^-51, and
-// residuals 20 times an FP64 elimination's).  Where an entry of R1 exceeds 3e-10 (condition numbers of about 1e3 and
-// more) the box takes a third step; |R0| > 1e-3, |R1| > 1e-4 or a third residual above 1e-9 sets the flag too.
+// residuals 20 times an FP64 elimination's).  Where an entry of R1 exceeds 3e-10 (condition numbers of about 3e2 and
+// more) the box takes a third step, with all 8 digits of X1: at 5 digits the cut alone leaves a residual of 2^-40 of |S| |X|,
+// again above 3e-10, and an inverse up to four times as far off as an FP64 elimination's.  |R0| > 1e-3, |R1| > 1e-4 or a
+// third residual above 1e-9 (condition numbers of about 1e5) sets the flag too.
 //
-// A product costs 30 (8 x 5 digits, 8 orders), 14, 8 or 6 BF16 MMAs; the matrices of a plane are read and written a few
+// A product costs 36 (8 x 8 digits, 8 orders; third step), 30 (8 x 5 digits), 14, 8 or 6 BF16 MMAs; the matrices of a plane are read and written a few
 // times.  Bound: the operands' loads (0.43 of the tensor pipe at 8 boxes of 676 unknowns: 30 products 814 us, 14 464 us, 8
 // 243 us; with 64-column tiles, half the instruction's rate, and four epilogue warps 1046, 593, 264 us), launches for
 // small planes.
@@ -36,7 +38,7 @@ namespace {
 
 constexpr int SAS = 8;    // digits of S
 constexpr int SAX = 3;    // digits of X as a left operand
-constexpr int SBM = 5;    // digits of a right operand at most
+constexpr int SBM = 8;    // digits of a right operand at most
 constexpr int GM = 128, GK = 64;
 constexpr int A_SLOT = GM * 128;
 
@@ -597,9 +599,13 @@ void dp_invert(helm_ctx ctx, const TgjWork& T, const DpWork& D, const BoxInfo* d
     for (int step = 0; step < 2; ++step) {   // the second time for the boxes that need it
         const int* gate = step ? stat : nullptr;
         // R1 = I - S X1 (X1 cut to its digits), X = X1 + X1 R1
-        slice_cols<SBM>(ctx, D, T, dbox, nbox, m_max, g, G, k, gate);
-        launch_gemm<SAS, SBM, 8, false>(ctx, D, D.mAS, D.eS, dbox, nbox, m_max, R, step ? 1e-9f : 1e-4f, k, T.flag,
-                                        step ? nullptr : stat, gate);
+        if (step == 0) {
+            slice_cols<5>(ctx, D, T, dbox, nbox, m_max, g, G, k);
+            launch_gemm<SAS, 5, 8, false>(ctx, D, D.mAS, D.eS, dbox, nbox, m_max, R, 1e-4f, k, T.flag, stat);
+        } else {
+            slice_cols<SBM>(ctx, D, T, dbox, nbox, m_max, g, G, k, gate);
+            launch_gemm<SAS, SBM, 8, false>(ctx, D, D.mAS, D.eS, dbox, nbox, m_max, R, 1e-9f, k, T.flag, nullptr, gate);
+        }
         slice_rows<SAX>(ctx, D, T, dbox, nbox, m_max, G, true, D.AX, D.eX, nullptr, k, nullptr, gate);
         slice_cols<3>(ctx, D, T, dbox, nbox, m_max, r, nullptr, k, gate);
         launch_gemm<3, 3, 3, true>(ctx, D, D.mAX, D.eX, dbox, nbox, m_max, G, 0.f, k, T.flag, nullptr, gate);

@@ -1,12 +1,15 @@
-"""The FP64 factorisation where it leaves its usual way: the reasons for which a set goes to the FP64 elimination, and sets that are
-factored in several batches of boxes.
+"""The FP64 factorisation where it leaves its usual way: the third Newton step of ill-conditioned planes, the two reasons for which a
+set goes to the FP64 elimination (and the third, no room), and sets that are factored in several batches of boxes.
 
 Ill-conditioned planes come from a uniform medium without layers or loss, driven next to an eigenfrequency of its first
 plane's operator (f (1 + d): condition number about 1 / d).  The numbers beside the cases are max |I - S X| of a complex64 inverse X0
 and of a Newton step on it, X1, cut to 24 and 40 bits of their columns' largest entries, as numpy gives them; an elimination
-by blocks leaves up to ten times as much.  The set is given up where the first exceeds 1e-3.
+by blocks leaves up to ten times as much.  The third step is taken from 3e-10 of the second on, and the set given up where
+the first exceeds 1e-3.
 
-Bars.  After a fallback the factors are those of the elimination that it names, bit for bit.  Batches: 1e-11 in relative Frobenius norm from the pivoted elimination, as for one batch."""
+Bars.  After a fallback the factors are those of the elimination that it names, bit for bit.  A third Newton step: the residual
+|I - D_0 G_0| of the first plane at most twice the fully pivoted FP64 elimination's (both are bounded by eps times the condition
+number) plus 1e-14 sqrt(m); with the exact coarse solve, applications equal to 1e-9, the bar of FP64 applications.  Batches: 1e-11 in relative Frobenius norm from the pivoted elimination, as for one batch."""
 import numpy as np
 import pytest
 
@@ -67,6 +70,39 @@ def _factor(helm, ctx, dims, f, mode):
     o = helm.Oras(grid, (1, 1, 1), 0, factor_prec=helm.PREC_FP64)
     ctx.set_tuning(helm.TUNE_BLOCK_GJ, 2)
     return [o.plane_inverse(0, k).cpu().numpy() for k in range(nz)]
+
+
+@pytest.mark.parametrize("dims", [(9, 8, 2), (20, 16, 2)])   # 9e-6, 2e-10 and 7e-6, 4e-10
+def test_third_newton_step(helm, dims):
+    nx, ny, _ = dims
+    a, b = _planes(dims, 1e-9)[0], _planes(dims, 5.0)[0]
+    v = np.outer(np.sin(np.pi * np.arange(1, ny + 1) / (ny + 1)), np.sin(np.pi * np.arange(1, nx + 1) / (nx + 1))).ravel()
+    k2 = (v @ a @ v).real / (v @ (a - b) @ v).real * (2 * np.pi * 5.0 / C0) ** 2   # the plane's longest wave
+    f = np.sqrt(k2) * C0 / (2 * np.pi) * (1 + 1e-3)
+    S = _planes(dims, f)
+    res = [_newton_residuals(s) for s in S]
+    assert max(r[0] for r in res) < 5e-5 and max(r[1] for r in res) > 1e-10
+    ctx = helm.Context(0)
+    got = _factor(helm, ctx, dims, f, 2)
+    assert sum(ctx.factor_fallbacks.values()) == 0
+    ref = _factor(helm, ctx, dims, f, 0)
+    off = [np.linalg.norm(np.eye(len(S[0])) - S[0] @ x[0]) for x in (got, ref)]
+    assert off[0] <= 2 * off[1] + 1e-14 * np.sqrt(len(S[0]))
+
+
+def test_third_newton_step_of_a_large_coarse_plane(helm):
+    """An exact coarse problem with planes of 44 x 42 (tiles of 128 columns; 5e-5, 9e-10)."""
+    import torch
+    nx, ny, nz = 86, 82, 6
+    ctx = helm.Context(0)
+    grid = helm.Grid(ctx, nx, ny, nz, H, 4.0, synth.linear_gradient(nx, ny, nz, H, C0, 0.6), npml=2, weights=helm.fit_weights())
+    v = torch.from_numpy(synth.random_complex((nz, ny, nx, 2), 31)).cuda()
+    got = {}
+    for mode in (2, 0):
+        ctx.set_tuning(helm.TUNE_BLOCK_GJ, mode)
+        got[mode] = helm.Oras(grid, (4, 4, 1), 2, coarse_ratio=2, factor_prec=helm.PREC_FP64).apply(v)
+    assert sum(ctx.factor_fallbacks.values()) == 0
+    assert float(torch.linalg.norm(got[2] - got[0])) <= 1e-9 * float(torch.linalg.norm(got[0]))
 
 
 @pytest.mark.parametrize("d,why", [(1e-6, "accuracy"),    # 6e-2; smallest pivot 1e-5 of the block
