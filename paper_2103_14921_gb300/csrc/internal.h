@@ -337,4 +337,5 @@ helm_status coarse_dd_apply(helm_oras o, int wp, const void* v, void* out, int n
 helm_status coarse_E_apply(helm_oras o, int wp, const void* x, void* y, int nrhs);      // y = E x
 helm_status inner_alloc(helm_oras o, int wp, int nrhs);
 void inner_free(helm_oras o);
+int inner_columns(helm_oras o);   // the column count its workspace is laid out for (0: none)
 helm_status inner_solve(helm_oras o, int wp, const void* c, void* y, int nrhs);

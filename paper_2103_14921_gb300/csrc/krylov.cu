@@ -1391,6 +1391,8 @@ helm_status inner_alloc(helm_oras o, int wp, int nrhs) {
     return HELM_OK;
 }
 
+int inner_columns(helm_oras o) { return o->inner ? o->inner->S : 0; }
+
 void inner_free(helm_oras o) {
     if (!o->inner) return;
     helm_ctx ctx = o->g->ctx;

@@ -759,8 +759,16 @@ static void free_scratch(helm_oras o) {
 }
 
 static helm_status ensure_scratch(helm_oras o, int wp, int nrhs) {
-    if (o->cap_nrhs >= nrhs && o->cap_wp == wp) return HELM_OK;
     helm_ctx ctx = o->g->ctx;
+    if (o->cap_nrhs >= nrhs && o->cap_wp == wp) {
+        // the inner coarse solve's vectors are laid out for one column count: another one takes a workspace of its own
+        if (o->d.coarse_iters == 0 || inner_columns(o) == nrhs) return HELM_OK;
+        cudaStreamSynchronize(ctx->stream);
+        o->scratch_gen++;
+        const helm_status rc = inner_alloc(o, wp, nrhs);
+        if (rc) inner_free(o);
+        return rc;
+    }
     cudaStreamSynchronize(ctx->stream);
     free_scratch(o);
     o->scratch_gen++;   // graphs captured over the old buffers are stale
