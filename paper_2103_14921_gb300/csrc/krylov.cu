@@ -372,9 +372,11 @@ __global__ void __launch_bounds__(RED_THREADS, IM <= 4 ? 2 : 1) update_dots_kern
 // (16 or more) basis loads in flight per thread, and the template widths follow ni in steps of four vectors.  112^3 x
 // 16: 5.1 - 5.8 TB/s, where the wide kernel (one block per SM, widths 16 and 32) ran at 3.2 - 4.7 (17 vectors: 1084 -> 671
 // us, 24: 1167 -> 809); at 5 to 8 vectors the wide kernel is the faster one (8: 348 us against 407).
-// Shared memory: 16 KB for the reductions and the ni nrhs coefficients, together at most the 48 KB of a launch without opt-in.
+// Shared memory: 17 KB for the reductions beside up to 32 KB of coefficients (past 48 KB together, at 125 columns and more, the
+// launch asks for it).  With the norm's sums in the reductions' memory it would never be more than 48 KB, but the kernel
+// then ran 5 % slower.
 constexpr int UDS_SLOTS = RED_THREADS / 2, UDS_QG = 4;
-constexpr size_t UDS_STATIC = (size_t)UDS_QG * 2 * UDS_SLOTS * sizeof(c128);
+constexpr size_t UDS_STATIC = UDS_SLOTS * (UDS_QG * 2 * sizeof(c128) + sizeof(double));
 template <typename T, int IMH, int EPT>
 __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T>* __restrict__ V, long long vstride,
                                                                    cplx<T>* __restrict__ w, long long n_el, int nrhs, int ni,
@@ -384,8 +386,9 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
     extern __shared__ __align__(16) unsigned char uds_smem[];
     cplx<T>* hs = reinterpret_cast<cplx<T>*>(uds_smem);   // [ni][nrhs]
     constexpr int SLOTS = UDS_SLOTS, QG = UDS_QG;
-    static_assert(UDS_STATIC + 2 * IMH * SLOTS * sizeof(cplx<T>) <= 48 * 1024, "2 IMH vectors of SLOTS columns");
     __shared__ c128 s[QG][2][SLOTS];
+    __shared__ double sn[SLOTS];
+    static_assert(sizeof(s) + sizeof(sn) == UDS_STATIC, "static shared memory");
     const int lane = threadIdx.x & 31, z = lane >> 4, slot = (threadIdx.x >> 5) * 16 + (lane & 15);
     const long long t = (long long)blockIdx.x * SLOTS + slot, stride = (long long)gridDim.x * SLOTS;
     const int r = (int)(t % nrhs);
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
             }
         }
     }
+    if (z == 0) sn[slot] = nrm.value();
     const int nr = min(nrhs, SLOTS);
 #pragma unroll
     for (int i0 = 0; i0 < IMH; i0 += QG) {
@@ -448,9 +452,6 @@ __global__ void __launch_bounds__(RED_THREADS, 2) update_dots_split(const cplx<T
             partial[((long long)blockIdx.x * ldp + 2 * i0 + q) * nrhs + rr] = sum;
         }
     }
-    __syncthreads();
-    double* sn = reinterpret_cast<double*>(&s[0][0][0]);   // [SLOTS]
-    if (z == 0) sn[slot] = nrm.value();
     __syncthreads();
     if (threadIdx.x < nr) {
         double sum = 0.0;
@@ -855,7 +856,11 @@ template <typename T, typename... Args>
 void launch_update_dots_split(int nblk, size_t hsm, cudaStream_t st, const cplx<T>* V, long long vs, cplx<T>* w, long long n_el,
                               int S, int ni, Args... args) {
     constexpr bool F = sizeof(T) == 4;
-    auto go = [&](auto kern) { kern<<<nblk, RED_THREADS, hsm, st>>>(V, vs, w, n_el, S, ni, args...); };
+    auto go = [&](auto kern) {
+        if (UDS_STATIC + hsm > 48 * 1024)
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * 1024);
+        kern<<<nblk, RED_THREADS, hsm, st>>>(V, vs, w, n_el, S, ni, args...);
+    };
     if (ni <= 12) go(update_dots_split<T, 6, F ? 3 : 1>);
     else if (ni <= 16) go(update_dots_split<T, 8, F ? 2 : 1>);
     else if constexpr (F) {
