@@ -46,7 +46,7 @@ from paper_2103_14921_gb300 import synth  # noqa: E402
 # the headline metric, the same on the library's line and the reference (oracle) line
 METRIC = "RHS solved/s to rel-res 1e-6 (mixed batched vs FP64 plain GPU)"
 # DRAM bytes per launch over algorithmic bytes, per kernel family (ncu, TF32 factors)
-TRAFFIC_RATIO = {"sweep_flow": 0.994, "sweep_gemm_tc": 1.037}
+TRAFFIC_RATIO = {"sweep_flow": 0.992, "sweep_gemm_tc": 1.041}
 # the autotuner's cache of tuned problem classes (decomposition, coarse level, sweep knobs)
 TUNE_CACHE = os.path.join(ROOT, "paper_2103_14921_gb300", "tuned.json")
 
@@ -223,6 +223,8 @@ class RequestMix:
     and released when it is done."""
 
     SIZES = (48, 64, 80, 96, 112, 128, 144, 160)
+    SHORT = ("cubic 48..160, 4 layered models per size, 2-6 Hz, 1-64 RHS, two-level ORAS with ~24-node boxes, coarse problem "
+             "by 10 GMRES iterations, TF32 factors, FGMRES(15) to 1e-6")
 
     def __init__(self, seed, count):
         import numpy as np
@@ -304,7 +306,7 @@ def run_serving(helm, device, stream, weights, args):
     mix = RequestMix(synth.workload_seed(5), args.serve_requests + args.serve_burst + 2 * args.serve_sweep)
     ctx = helm.Context(device, stream=stream.cuda_stream, budget_bytes=150 << 30)
     items = mix.items
-    res = {"mix": RequestMix.__doc__.split("\n\n")[0].replace("\n", " "), "budget_gb": 150, "slots_per_batch": 64}
+    res = {"mix": RequestMix.SHORT, "budget_gb": 150, "slots_per_batch": 64}
 
     def summary(st, wall, rate=None):
         done = [s_ for s_ in st if not s_.get("timed_out")]
@@ -403,6 +405,12 @@ def columns_summary(stats):
             "converged": all(s["converged"] for s in stats)}
 
 
+def tune_trials(tr):
+    """The candidates that the autotuner timed in this run (a choice from the cache has its trials there)."""
+    keep = ("parts", "overlap", "rhs_per_s", "iterations", "setup_s")
+    return [] if tr.get("cached") else [{k: t[k] for k in keep if k in t} for t in tr.get("trials") or []]
+
+
 def short_floats(x):
     """x with every float in it (a detail of the line) at six significant digits."""
     if isinstance(x, dict):
@@ -477,7 +485,7 @@ def run_thrust_fold(helm, ctx, stream, weights, peaks, retune=False):
            "value": b.shape[-1] / (ms / 1e3), "unit": "RHS/s", "solve_s": ms / 1e3, "setup_s": setup_s,
            "tune_s": tune_s, "parts": tr["parts"], "overlap": tr["overlap"], "knobs": tr.get("knobs"),
            "coarse_ratio": tr.get("coarse_ratio"), "coarse_iters": tr.get("coarse_iters"),
-           "tune_cached": tr.get("cached", False), "tune_trials": tr.get("trials"),
+           "tune_cached": tr.get("cached", False), "tune_trials": tune_trials(tr),
            "iterations_max": max(s_["iterations"] for s_ in stats),
            "iterations_mean": float(np.mean([s_["iterations"] for s_ in stats])),
            "max_true_relres": max(s_["true_relres"] for s_ in stats),
@@ -560,7 +568,7 @@ def run_attenuating(helm, ctx, stream, weights, peaks, retune=False):
     return {"workload": "attenuating linear gradient (Q = 100) 160x160x80, 3/4/6 Hz x 128 RHS, two-level ORAS "
                         "autotuned boxes, ov2 r4, TF32 factors, FGMRES(30) tol 1e-6, one batch of 128 per frequency",
             "value": n_all / (tot_ms / 1e3), "unit": "RHS/s", "solve_s": tot_ms / 1e3, "parts": list(parts),
-            "overlap": ov, "tune_s": tune_s, "tune_cached": tr.get("cached", False), "tune_trials": tr.get("trials"),
+            "overlap": ov, "tune_s": tune_s, "tune_cached": tr.get("cached", False), "tune_trials": tune_trials(tr),
             "per_frequency": freqs}
 
 
@@ -868,8 +876,7 @@ def run_gpu(args, W):
         vb, _ = replicas.job_throughput(nrhs * kv, v0.elapsed_time(v1) / 1000.0, dev)
         err = float(torch.linalg.vector_norm(xb - x) / torch.linalg.vector_norm(x))
         variants["bf16_factors"] = {"value": vb, "unit": "RHS/s", "steps": kv,
-                                    "iterations": [s_["iterations"] for s_ in stb],
-                                    "max_true_relres": max(s_["true_relres"] for s_ in stb),
+                                    **columns_summary(stb),
                                     "rel_l2_vs_tf32_solution": err}
         del ob, xb
         if W["coarse"]:
@@ -891,8 +898,7 @@ def run_gpu(args, W):
             vi, _ = replicas.job_throughput(nrhs * kv, v0.elapsed_time(v1) / 1000.0, dev)
             err = float(torch.linalg.vector_norm(xi - x) / torch.linalg.vector_norm(x))
             variants["coarse_gmres10"] = {"value": vi, "unit": "RHS/s", "steps": kv, "setup_s": oi.setup_seconds,
-                                          "iterations": [s_["iterations"] for s_ in sti],
-                                          "max_true_relres": max(s_["true_relres"] for s_ in sti),
+                                          **columns_summary(sti),
                                           "rel_l2_vs_exact_coarse_solution": err}
             del oi, xi
         # a frequency sweep of the same model and sources (three neighbouring frequencies): warm starts from
@@ -1020,7 +1026,7 @@ def run_gpu(args, W):
     }
     # one line of a few kilobytes: readers that keep the end of a program's output only must still get all of it
     line = {k: v if k in ("value", "ms_per_step", "e2e") else short_floats(v) for k, v in line.items()}
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line, separators=(",", ":")), flush=True)
     if ws > 1:
         torch.distributed.destroy_process_group()
 
