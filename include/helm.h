@@ -126,7 +126,8 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * walking z-planes (the in-plane terms of a plane are formed once and reused by the three output planes it
  * touches; warps wholly inside the interior take class-sum forms, the others the product form), except
  * complex64 calls of fewer than 2^20 values and complex128 calls of fewer than 40,000 nodes and 90,000 values; 2 the
- * same at every size; 0 uses the per-node kernel.  All agree to FP32 rounding.  Returns HELM_EINVAL for an unknown key or value out of range. */
+ * same at every size; 0 uses the per-node kernel.  All agree to the rounding of the call's precision.  Returns HELM_EINVAL
+ * for an unknown key or value out of range. */
 #define HELM_TUNE_TC_STAGES 1
 #define HELM_TUNE_COARSE_COOP 2
 #define HELM_TUNE_GRAPHS 3
@@ -146,10 +147,10 @@ helm_status helm_profile_query(helm_ctx ctx, const char* name, uint64_t* launche
  * Gauss-Jordan on the CUDA cores.  Read by oras_factor. */
 #define HELM_TUNE_TC_FACTOR 7
 /* HELM_TUNE_BLOCK_GJ: how the other plane sets (FP64 and FP32 local factors, the FP64 coarse problem) are factored.
- * 2 (default): FP64 planes by the tensor-core elimination in complex64 and two Newton steps whose products are exact
- * sums of integer digits on the tensor cores (inverses good to FP64; planes of up to 2304 unknowns, a workspace of up to
- * 4 GB while factoring); a tiny block pivot, a plane that does not come out to FP64 or a workspace that does not fit the
- * budget goes to 1.  FP32 planes as with 1.  1: the same blocked Gauss-Jordan as the tensor-core elimination with
+ * 2 (default): FP64 planes by the tensor-core elimination in complex64 and two Newton steps whose products are sums
+ * of integer digits on the tensor cores, three steps for ill-conditioned planes (inverses good to FP64; planes of up to
+ * 2304 unknowns, a workspace of up to 4 GB while factoring); a tiny block pivot, a plane that does not come out to FP64 or
+ * a workspace that does not fit the budget goes to 1.  FP32 planes as with 1.  1: the same blocked Gauss-Jordan as the tensor-core elimination with
  * block pivots on the CUDA cores (64-column panels for complex64, 32 for complex128; the rank-NB updates spread over every
  * SM), falling back to full partial pivoting after a tiny block pivot.  0: always the fully pivoted elimination.  Read by
  * oras_factor. */

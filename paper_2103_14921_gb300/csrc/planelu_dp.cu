@@ -1,16 +1,18 @@
 // complex128 plane inverses on the tensor cores: G = S^{-1} in FP64 from the complex64 inverse X0 of the tensor-core
-// elimination (planelu_tc.cu) by two Newton steps X <- X + X (I - S X), whose products are exact sums of small integers.
+// elimination (planelu_tc.cu) by two Newton steps X <- X + X (I - S X), whose products are sums of small integers.
 //
 // Why: the FP64 pipe of this part does two multiply-adds per SM and clock, so the block elimination in FP64 (planelu.cu)
 // runs at 1.0 TFLOP/s at best and inverts one 32 x 32 block at a time beside it.  The products here run as BF16 MMAs.
 //
 // Slices (the Ozaki scheme): a row of the left operand, or a column of the right one, is scaled by a power of two so that
 // its entries lie in (-1, 1) and written as digits d_0, d_1, ... in base 256, |d_i| <= 128, x = 2^(e-7) sum d_i 256^-i.
-// Digits are exact in BF16 and a product of two is an integer of at most 2^14; sums below 2^24 are exact in the FP32
-// accumulators, so the product of slices i and j contributes exactly to order i + j.  Orders are accumulated apart (one
-// TMEM accumulator each), the products of the orders kept (i + j < O) are added as 64-bit integers and converted once.
-// Sums of K <= 4608 products of digits that are as good as random stay near 2^19; an accumulator beyond 2^23 sets
-// the flag that sends the set to the FP64 elimination.
+// Digits are exact in BF16 and a product of two is an integer of at most 2^14.  Orders are accumulated apart (one TMEM
+// accumulator each), the products of the orders kept (i + j < O) are added as 64-bit integers and converted once.
+// An FP32 accumulator is exact while its running sum stays below 2^24.  The digits' range does not ensure that (K <= 4608
+// products of up to eight digit pairs), their distribution does: leading digits follow |S| |X|, whose rows decay from the
+// diagonal (sums below 2^21), the others are as good as random, so that sums have a standard deviation of 2^20 at most
+// (2^20 at 320 unknowns in an emulation), 2^24 being sixteen of them.  An accumulator that ends beyond 2^23 sets the flag
+// that sends the set to the FP64 elimination; one that went beyond 2^24 and came back would be rounded there unseen.
 //
 // Precision.  X0 is cut to 3 digits (24 bits of its column's largest entry) and taken as exact.  R0 = I - S X0 with 5
 // digits of S (2^-40), X1 = X0 + X0 R0 cut to 5 digits, R1 = I - S X1 with all 8 digits of S (64 bits below its row's largest
@@ -21,10 +23,10 @@
 // again above 3e-10, and an inverse up to four times as far off as an FP64 elimination's.  |R0| > 1e-3, |R1| > 1e-4 or a
 // third residual above 1e-9 (condition numbers of about 1e5) sets the flag too.
 //
-// A product costs 36 (8 x 8 digits, 8 orders; third step), 30 (8 x 5 digits), 14, 8 or 6 BF16 MMAs; the matrices of a plane are read and written a few
-// times.  Bound: the operands' loads (0.43 of the tensor pipe at 8 boxes of 676 unknowns: 30 products 814 us, 14 464 us, 8
-// 243 us; with 64-column tiles, half the instruction's rate, and four epilogue warps 1046, 593, 264 us), launches for
-// small planes.
+// A product costs 36 (8 x 8 digits, 8 orders; third step), 30 (8 x 5 digits), 14, 8 or 6 BF16 MMAs; the matrices of a plane
+// are read and written a few times.  Bound: the operands' loads (0.43 of the tensor pipe at 8 boxes of 676 unknowns: 30
+// products 814 us, 14 464 us, 8 243 us; with 64-column tiles, half the instruction's rate, and four epilogue warps 1046,
+// 593, 264 us), launches for small planes.
 #include <cuda.h>
 #include <cuda_bf16.h>
 

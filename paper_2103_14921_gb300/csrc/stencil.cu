@@ -212,9 +212,10 @@ __global__ void __launch_bounds__(128) stencil_kernel(const cplx<T>* __restrict_
 // complex128 is bound by the FP64 pipe (two lanes per SM and clock): the form with the fewest FP64 operations is
 // taken wherever it holds, and plain axes are tested at run time in the product form too.  112^3 x 16: 2.84 ms
 // (per-node kernel 5.1 ms), 87 % of the pipe while a block runs; 101 x 93 x 77 x 10: 1.30 (2.54) ms; 48^3 x 1: 0.11
-// (0.18) ms.  complex64 is bound by instruction latency at 12 warps per SM (issue 36 % active, DRAM a third of its
-// rate): 112^3 x 16 163 us (per-node 361), 160 x 160 x 80 x 128 with complex k^2 1.39 (5.07) ms, 101 x 93 x 77 x 10
-// 86 (168) us.  MN = 2 (more warps) measured 247, MN = 8 171 us at 112^3 x 16, so 4.
+// (0.18) ms.  complex64 is bound by instruction latency at 12 warps per SM (issue 38 to 44 % active on a slab of 24
+// planes, DRAM a third of its rate at 112^3): 112^3 x 16 163 us (per-node 361), 160 x 160 x 80 x 128 with complex k^2 1.40
+// (5.07) ms, 101 x 93 x 77 x 10 85 (168) us; in brackets the per-node kernel throughout.  MN = 2 (more warps) measured 247
+// and MN = 8 171 us at 112^3 x 16 when MN = 4 took 170 (163 since the tile is chosen by total work), so 4.
 struct PlainRange {
     int lo[3], hi[3];   // per axis: indices whose stretched coefficients are exactly (1, -2, 1)
 };
@@ -650,8 +651,9 @@ Interior interior_of(helm_grid g) {
     return in;
 }
 
-// Per axis, the index range whose complex64 stretched coefficients are exactly (1, -2, 1) (the table is
-// contiguous-plain in the middle and stretched in the absorbing layers); empty if not contiguous.
+// Per axis, the index range whose stretched coefficients are exactly (1, -2, 1) (the table is contiguous-plain in the
+// middle and stretched in the absorbing layers); empty if not contiguous.  Tested in complex64 for both types: a stretched
+// coefficient has an imaginary part, which only rounds away below 1e-45, where complex128 results do not see it either.
 PlainRange plain_range(helm_grid g) {
     PlainRange r;
     const int n[3] = {g->d.nx, g->d.ny, g->d.nz};
