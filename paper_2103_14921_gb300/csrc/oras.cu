@@ -758,6 +758,8 @@ static void free_scratch(helm_oras o) {
     o->cap_nrhs = 0;
 }
 
+static helm_status alloc_scratch(helm_oras o, int wp, int R);
+
 static helm_status ensure_scratch(helm_oras o, int wp, int nrhs) {
     helm_ctx ctx = o->g->ctx;
     if (o->cap_nrhs >= nrhs && o->cap_wp == wp) {
@@ -772,11 +774,17 @@ static helm_status ensure_scratch(helm_oras o, int wp, int nrhs) {
     cudaStreamSynchronize(ctx->stream);
     free_scratch(o);
     o->scratch_gen++;   // graphs captured over the old buffers are stale
-    const size_t fe = o->fine.cesize();
-    const size_t we = wp == HELM_PREC_FP64 ? sizeof(c128) : sizeof(c64);
     o->cap_nrhs = nrhs;
     o->cap_wp = wp;
-    const int R = nrhs;
+    const helm_status rc = alloc_scratch(o, wp, nrhs);
+    if (rc) free_scratch(o);   // all or nothing: the next call of this width must not find half of it
+    return rc;
+}
+
+static helm_status alloc_scratch(helm_oras o, int wp, int R) {
+    helm_ctx ctx = o->g->ctx;
+    const size_t fe = o->fine.cesize();
+    const size_t we = wp == HELM_PREC_FP64 ? sizeof(c128) : sizeof(c64);
     HELM_TRY(dev_alloc(ctx, &o->loc, (size_t)o->fine.nloc * R * fe, "local vectors"));
     HELM_TRY(dev_alloc(ctx, &o->rbuf, (size_t)rbuf_planes(o) * o->fine.m_max * R * fe, "sweep buffer"));
     if (o->fine.padded) {
