@@ -214,14 +214,14 @@ BoxPlan box_plan(helm_ctx ctx, const PlaneSet& P, int nrhs) {
 }
 
 template <typename TV, typename TL, int CT>
-cudaError_t launch_ct(const PlaneSet& P, const cplx<TV>* v, cplx<TV>* out, cplx<TL>* loc, int nx, int ny, int nrhs,
+cudaError_t launch_ct(helm_ctx ctx, const PlaneSet& P, const cplx<TV>* v, cplx<TV>* out, cplx<TL>* loc, int nx, int ny, int nrhs,
                       const BoxPlan& p, cudaStream_t st) {
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(ctx->device)) {
         const cudaError_t e = cudaFuncSetAttribute(box_solve<TV, TL, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    200 * 1024);
         if (e != cudaSuccess) return e;
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     box_solve<TV, TL, CT><<<dim3((nrhs + p.cc - 1) / p.cc, P.nbox), BS_THREADS, p.smem, st>>>(
         P.dbox, (const cplx<TL>*)P.coef, (const cplx<TL>*)P.G, v, out, loc, nx, ny, nrhs, P.m_max, p);
@@ -237,9 +237,9 @@ helm_status run(helm_ctx ctx, const PlaneSet& P, const void* v, void* out, void*
     const cplx<TV>* vv = (const cplx<TV>*)v;
     cplx<TV>* oo = (cplx<TV>*)out;
     cplx<TL>* ll = (cplx<TL>*)loc;
-    const cudaError_t e = p.cc >= 4   ? launch_ct<TV, TL, 4>(P, vv, oo, ll, nx, ny, nrhs, p, st)
-                          : p.cc == 2 ? launch_ct<TV, TL, 2>(P, vv, oo, ll, nx, ny, nrhs, p, st)
-                                      : launch_ct<TV, TL, 1>(P, vv, oo, ll, nx, ny, nrhs, p, st);
+    const cudaError_t e = p.cc >= 4   ? launch_ct<TV, TL, 4>(ctx, P, vv, oo, ll, nx, ny, nrhs, p, st)
+                          : p.cc == 2 ? launch_ct<TV, TL, 2>(ctx, P, vv, oo, ll, nx, ny, nrhs, p, st)
+                                      : launch_ct<TV, TL, 1>(ctx, P, vv, oo, ll, nx, ny, nrhs, p, st);
     HELM_CUDA(ctx, e);
     ctx->launches++;
     *done = true;

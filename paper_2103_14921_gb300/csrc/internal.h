@@ -92,6 +92,13 @@ struct helm_ctx_s {
     }
 };
 
+// What is set once per kernel and device (function attributes belong to a device); a bit per device.
+struct PerDevice {
+    std::atomic<uint64_t> mask{0};
+    bool done(int device) const { return (mask.load(std::memory_order_acquire) >> (device & 63)) & 1; }
+    void mark(int device) { mask.fetch_or(1ull << (device & 63), std::memory_order_release); }
+};
+
 // Bracket one launch of an instrumented family with events on the context's stream.
 int prof_begin(helm_ctx ctx, const char* family);   // returns a token (-1 when profiling is off)
 void prof_end(helm_ctx ctx, int token, double bytes);

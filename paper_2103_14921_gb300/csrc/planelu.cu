@@ -660,11 +660,11 @@ helm_status factor_t(helm_ctx ctx, PlaneSet& P, int* singular) {
     // else the global-memory panel of nb columns
     constexpr int NBS = 24;
     const size_t psm = (size_t)m * NBS * sizeof(cplx<T>);
-    static std::atomic<bool> psm_attr{false};
+    static PerDevice psm_attr;
     if constexpr (sizeof(T) == 4) {
-        if (!psm_attr.load(std::memory_order_acquire)) {
+        if (!psm_attr.done(ctx->device)) {
             cudaFuncSetAttribute(gj_panel_smem<T, NBS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-            psm_attr.store(true, std::memory_order_release);
+            psm_attr.mark(ctx->device);
         }
     }
     const bool smem_panel = sizeof(T) == 4 && psm <= 200 * 1024;
@@ -950,11 +950,11 @@ helm_status factor_block_t(helm_ctx ctx, PlaneSet& P, int* singular, int* weak) 
         cleanup();
         return rc;
     }
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(ctx->device)) {
         cudaFuncSetAttribute(bgj_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)((NB * (NB + 1) + 16 * NB) * sizeof(cplx<T>)));
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     cudaMemsetAsync(flag, 0, sizeof(int), st);
     const cplx<T>* coef = (const cplx<T>*)P.coef;
@@ -1097,11 +1097,11 @@ void launch_sweep_rn(const PlaneSet& P, cplx<T>* loc, cplx<T>* rbuf, int nrhs, c
     const dim3 pgrid(pblocks, P.nbox);
     const cplx<T>* coef = (const cplx<T>*)P.coef;
     const cplx<T>* G = (const cplx<T>*)P.G;
-    static std::atomic<bool> attr_set{false};
-    if (!attr_set.load(std::memory_order_acquire)) {
+    static PerDevice attr_set;
+    if (!attr_set.done(ctx->device)) {
         cudaFuncSetAttribute(sweep_gemv<T, RN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(sweep_gemv<T, RN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        attr_set.store(true, std::memory_order_release);
+        attr_set.mark(ctx->device);
     }
     // algorithmic bytes of one step: every active box reads its m x m factor plane once,
     // the prepared plane (m x nrhs) and writes (backward: also reads) its output plane;
@@ -1125,10 +1125,10 @@ void launch_sweep_rn(const PlaneSet& P, cplx<T>* loc, cplx<T>* rbuf, int nrhs, c
         const dim3 sgrid((m + rows - 1) / rows, KSPLIT, (nrhs + RN - 1) / RN);
         const size_t ssm = (size_t)RN * kw * sizeof(cplx<T>);
         cplx<T>* part = rbuf + (size_t)m * nrhs;   // the caller sizes rbuf (1 + KSPLIT) planes deep
-        static std::atomic<bool> sattr{false};
-        if (!sattr.load(std::memory_order_acquire)) {
+        static PerDevice sattr;
+        if (!sattr.done(ctx->device)) {
             cudaFuncSetAttribute(sweep_gemv_splitk<T, RN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-            sattr.store(true, std::memory_order_release);
+            sattr.mark(ctx->device);
         }
         const unsigned rblocks = (unsigned)std::min<long long>(((long long)m * nrhs + 255) / 256, 512);
         for (int pass = 0; pass < 2; ++pass) {

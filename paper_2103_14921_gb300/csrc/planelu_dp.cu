@@ -486,10 +486,10 @@ bool encode_slices(CUtensorMap* map, void* base, uint64_t cols, uint64_t rows, u
 template <int SA, int SB, int O, bool ADD, int GN>
 void launch_gemm_n(helm_ctx ctx, const DpWork& D, const CUtensorMap& mA, const CUtensorMap& mB, const int* ea, const BoxInfo* dbox,
                    int nbox, int m_max, c128* out, float limit, int k, int* flag, int* stat, const int* gate) {
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(ctx->device)) {
         cudaFuncSetAttribute(dp_gemm<SA, SB, O, ADD, GN>, cudaFuncAttributeMaxDynamicSharedMemorySize, dp_smem());
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     const dim3 grid((2 * m_max + GN - 1) / GN, (m_max + GM - 1) / GM, nbox);
     dp_gemm<SA, SB, O, ADD, GN><<<grid, 320, dp_smem(), ctx->stream>>>(mA, mB, dbox, ea, D.eB, D.nb, D.Lr, D.Nr / 2, D.m_max, out,

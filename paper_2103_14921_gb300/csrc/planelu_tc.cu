@@ -725,12 +725,12 @@ helm_status tgj_alloc(helm_ctx ctx, int nbox, int m_max, TgjWork& W) {
         tgj_free(ctx, W);
         return set_error(ctx, HELM_ECUDA, "cuTensorMapEncodeTiled failed for the tensor-core factorisation");
     }
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(ctx->device)) {
         cudaFuncSetAttribute(tgj_update_pers<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
         cudaFuncSetAttribute(tgj_update_pers<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PSMEM);
         cudaFuncSetAttribute(tgj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, DIAG_SMEM);
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     cudaMemsetAsync(W.S, 0, W.s_bytes, ctx->stream);
     cudaMemsetAsync(W.flag, 0, 2 * sizeof(int), ctx->stream);

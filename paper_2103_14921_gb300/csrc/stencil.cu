@@ -752,11 +752,11 @@ bool launch_march(helm_grid g, const void* u, const void* b, void* y, int nrs, c
     w.a3 = (T)g->w.a3;
     w.ih2 = (T)g->w.inv_h2;
     const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(g->ctx->device)) {
         cudaFuncSetAttribute(stencil_march<V, SUB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
         cudaFuncSetAttribute(stencil_march<V, SUB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-        attr.store(true, std::memory_order_release);
+        attr.mark(g->ctx->device);
     }
     if (g->k2_real)
         stencil_march<V, SUB, true><<<grid, t.threads, smem, s>>>((const V*)u, (const V*)b, (V*)y, k2, tab, d.nx, d.ny,

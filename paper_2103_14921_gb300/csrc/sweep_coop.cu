@@ -242,10 +242,10 @@ CoopPlan plan_for(helm_ctx ctx, const PlaneSet& P) {
     c.gp = m | 1;
     c.smem = ((size_t)CO_RN * m + (size_t)c.rpc * c.gp + (size_t)CO_WARPS * CO_ROWS * CO_RN) * sizeof(c64);
     if (c.smem > 200 * 1024) return c;
-    static std::atomic<bool> attr{false};
-    if (!attr.load(std::memory_order_acquire)) {
+    static PerDevice attr;
+    if (!attr.done(ctx->device)) {
         cudaFuncSetAttribute(coarse_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coarse_sweeps, CO_THREADS, c.smem) != cudaSuccess ||

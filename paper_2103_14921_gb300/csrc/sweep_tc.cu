@@ -743,9 +743,9 @@ helm_status run_tc(helm_ctx ctx, const PlaneSet& P, const c64* lb, c64* loc, E* 
         !encode_3d(&mapB, bt, 2ull * ld, (uint64_t)NPAD, (uint64_t)P.nbox, 2ull * ld * eb, 2ull * ld * NPAD * eb,
                    Cfg::BK, NPAD, BF))
         return set_error(ctx, HELM_ECUDA, "cuTensorMapEncodeTiled failed for the tensor-core sweep");
-    static std::atomic<bool> attr{false};
+    static PerDevice attr;
     static std::atomic<int> flow_occ{0};
-    if (!attr.load(std::memory_order_acquire)) {
+    if (!attr.done(ctx->device)) {
         cudaFuncSetAttribute(tc_sweep_gemm<E, NPAD, NST>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
         cudaFuncSetAttribute(tc_sweep_flow<E, NPAD, NST>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
         // all of the unified L1 as shared memory, so that as many persistent CTAs fit per SM as its 228 KB allow
@@ -766,7 +766,7 @@ helm_status run_tc(helm_ctx ctx, const PlaneSet& P, const c64* lb, c64* loc, E* 
         }
         cudaFuncSetAttribute(tc_prep2<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(128 * (PREP2_TP + 1) * sizeof(c64)));
-        attr.store(true, std::memory_order_release);
+        attr.mark(ctx->device);
     }
     const int m = P.m_max;
     const int gtiles = (m + TC_BM - 1) / TC_BM;
